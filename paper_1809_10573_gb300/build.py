@@ -18,7 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(HERE, "lib")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libidbf.so")
-SOURCES = ["plan.cu", "apply.cu", "apply_tc.cu", "batch.cu", "build_gpu.cu"]
+SOURCES = ["plan.cu", "apply.cu", "node.cu", "apply_tc.cu", "batch.cu", "build_gpu.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # host code: no contraction of a * b + c into an FMA, so that host arithmetic (e.g. the dyadic leaf
 # edges) rounds the same on x86-64 and aarch64

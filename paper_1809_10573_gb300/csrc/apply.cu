@@ -17,182 +17,6 @@
 
 namespace idbf {
 
-template <class P, int RB, int RPT = 0>
-__global__ void __launch_bounds__(512) k_level_fwd(DevLevel d, const typename P::mat_t* __restrict__ mat,
-                                                   IO<typename P::vec_t> io, int gcap, int rcap, int max_in) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  fwd_node<P, RB, RPT>(d, mat, io, gcap, rcap, max_in, (int64_t)blockIdx.x, (int)blockIdx.y * RB, smem);
-}
-
-// Several right-hand sides, FP32 / FP64 (fwd_node_tiled): node blockIdx.x, right-hand sides
-// blockIdx.y * RB ...
-template <class P>
-__host__ __device__ constexpr bool tiled_ok() {
-  return std::is_same<typename P::vec_t, typename P::gv_t>::value;
-}
-// The right-hand-side blocks of a node are adjacent CTAs (blockIdx.x = node * nblk + block), so
-// that their reads of the node's factors meet in L2.
-template <class P, int RB, int TC, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_level_fwd_tiled(DevLevel d, const typename P::mat_t* __restrict__ mat,
-                                                         IO<typename P::vec_t> io, int max_rows, int max_in,
-                                                         int max_out, int nblk) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  if constexpr (tiled_ok<P>())
-    fwd_node_tiled<P, RB, TC>(d, mat, io, max_rows, max_in, max_out, (int64_t)(blockIdx.x / nblk),
-                              (int)(blockIdx.x % nblk) * RB, smem);
-}
-
-// Several right-hand sides, FP32 / FP64 adjoint (adj_node_tiled): node blockIdx.x / nblk,
-// right-hand-side block blockIdx.x % nblk.
-template <class P, int RB, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_level_adj_tiled(DevLevel d, const typename P::mat_t* __restrict__ mat,
-                                                               IO<typename P::vec_t> io, int max_in, int max_out,
-                                                               int max_rows, int max_cols, int nblk) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  if constexpr (tiled_ok<P>())
-    adj_node_tiled<P, RB>(d, mat, io, max_in, max_out, max_rows, max_cols, (int64_t)(blockIdx.x / nblk),
-                          (int)(blockIdx.x % nblk) * RB, smem);
-}
-
-// ---------------------------------------------------------------------------------------------
-// adjoint level kernel: reads the forward outputs of node j, writes its forward inputs.
-// Shared memory: v[max_out][RB], g[2][gcap][RB], res[2][rcap][RB], ub[max_in][RB].
-template <class P, int RB>
-__global__ void __launch_bounds__(256) k_level_adj(DevLevel d, const typename P::mat_t* __restrict__ mat,
-                                                   IO<typename P::vec_t> io, int gcap, int rcap, int max_out) {
-  using V = typename P::vec_t;
-  using G = typename P::gv_t;
-  using M = typename P::mat_t;
-  extern __shared__ __align__(16) unsigned char smem[];
-  V* v = (V*)smem;
-  G* g = (G*)(v + (size_t)max_out * RB);
-  V* res = (V*)(g + (size_t)2 * gcap * RB);
-  V* ub = res + (size_t)2 * rcap * RB;
-  const int64_t j = blockIdx.x;
-  const int r0 = blockIdx.y * RB;
-  const int nrb = min(RB, io.R - r0);
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-
-  // phase 1: adjoint inputs (forward outputs) -> v
-  int o0len, o1len;
-  if (d.lev == d.L) {
-    o0len = leaf_len(d, j);
-    o1len = 0;
-    const int64_t x0 = leaf_start(d, j);
-    for (int i = tid; i < o0len * RB; i += nt) {
-      const int e = i / RB, rb = i % RB;
-      v[i] = rb < nrb ? io.x[x0 + e + (int64_t)(r0 + rb) * io.ldx] : P::zero();
-    }
-  } else {
-    const int64_t s0 = out_seg_id(d, j, 0), s1 = out_seg_id(d, j, 1);
-    o0len = d.out_len[s0];
-    o1len = d.out_len[s1];
-    const int64_t b0 = d.out_off[s0], b1 = d.out_off[s1];
-    for (int i = tid; i < (o0len + o1len) * RB; i += nt) {
-      const int e = i / RB, rb = i % RB;
-      const int64_t off = e < o0len ? b0 + e : b1 + (e - o0len);
-      v[i] = rb < nrb ? io.win[off * io.R + r0 + rb] : P::zero();
-    }
-  }
-  const int rows0 = d.rows[2 * j], rows1 = d.rows[2 * j + 1];
-  const int cols0 = d.cols[2 * j], cols1 = d.cols[2 * j + 1];
-  const int64_t mo0 = d.moff[2 * j], mo1 = d.moff[2 * j + 1];
-  const int32_t* ix0 = d.idx + d.ioff[2 * j];
-  const int32_t* ix1 = d.idx + d.ioff[2 * j + 1];
-  __syncthreads();
-
-  // phase 2: operands of the conjugate-transposed products (indexed by block row r)
-  if (d.kind == KIND_U) {  // g_c[r] = v[p_c[r]]
-    for (int i = tid; i < rows0 * RB; i += nt) g[i] = P::cvt(v[ix0[cols0 + i / RB] * RB + i % RB]);
-    for (int i = tid; i < rows1 * RB; i += nt) g[gcap * RB + i] = P::cvt(v[ix1[cols1 + i / RB] * RB + i % RB]);
-  } else {  // g_c = v_c (the c-th forward output)
-    for (int i = tid; i < rows0 * RB; i += nt) g[i] = P::cvt(v[i]);
-    for (int i = tid; i < rows1 * RB; i += nt) g[gcap * RB + i] = P::cvt(v[o0len * RB + i]);
-  }
-  __syncthreads();
-
-  // phase 3: res_c[i] = sum_r conj(M_c(r, i)) g_c[r]; a warp per column i (contiguous in r)
-  const int items = d.kind == KIND_S ? cols0 : cols0 + cols1;
-  for (int it = warp; it < items; it += nw) {
-    typename P::acc_t acc[RB];
-#pragma unroll
-    for (int rb = 0; rb < RB; ++rb) P::init(acc[rb]);
-    const int cfirst = d.kind == KIND_S ? 0 : (it >= cols0);
-    const int clast = d.kind == KIND_S ? 1 : cfirst;
-    const int i = (d.kind != KIND_S && cfirst) ? it - cols0 : it;
-    for (int c = cfirst; c <= clast; ++c) {
-      const int rows = c ? rows1 : rows0;
-      const M* col = mat + (c ? mo1 : mo0) + (int64_t)i * rows;
-      const G* gc = g + c * gcap * RB;
-      int cnt = 0;
-      for (int r = lane; r < rows; r += 32) {
-        const M mv = P::ld(col + r);
-#pragma unroll
-        for (int rb = 0; rb < RB; ++rb) P::macc(acc[rb], mv, gc[r * RB + rb]);
-        if (++cnt == P::CHUNK) {
-#pragma unroll
-          for (int rb = 0; rb < RB; ++rb) P::flush(acc[rb]);
-          cnt = 0;
-        }
-      }
-    }
-#pragma unroll
-    for (int rb = 0; rb < RB; ++rb) {
-      P::warp_sum(acc[rb]);
-      if (lane == 0) res[(cfirst * rcap + i) * RB + rb] = P::fin(acc[rb]);
-    }
-  }
-  __syncthreads();
-
-  // phase 4: combine and write the forward inputs
-  int nin;
-  if (d.kind == KIND_U) {
-    // out_c[i] = v[q_c[i]] + res_c[i]  ->  forward input segment c
-    for (int c = 0; c < 2; ++c) {
-      const int cols = c ? cols1 : cols0;
-      const int32_t* q = c ? ix1 : ix0;
-      const int64_t ob = d.in_off[2 * j + c];
-      for (int k = tid; k < cols * nrb; k += nt) {
-        const int i = k / nrb, rb = k % nrb;
-        io.wout[(ob + i) * io.R + r0 + rb] = P::add(v[q[i] * RB + rb], res[(c * rcap + i) * RB + rb]);
-      }
-    }
-    return;
-  }
-  if (d.kind == KIND_S) {
-    nin = cols0;
-    for (int k = tid; k < nin * RB; k += nt) ub[k] = res[k];
-  } else {
-    nin = rows0 + cols0;
-    for (int k = tid; k < nin * RB; k += nt) ub[k] = P::zero();
-    __syncthreads();
-    for (int k = tid; k < rows0 * RB; k += nt) { V* dst = &ub[ix0[k / RB] * RB + k % RB]; *dst = P::add(*dst, v[k]); }
-    __syncthreads();
-    for (int k = tid; k < rows1 * RB; k += nt) { V* dst = &ub[ix1[k / RB] * RB + k % RB]; *dst = P::add(*dst, v[o0len * RB + k]); }
-    __syncthreads();
-    for (int k = tid; k < cols0 * RB; k += nt) { V* dst = &ub[ix0[rows0 + k / RB] * RB + k % RB]; *dst = P::add(*dst, res[k]); }
-    __syncthreads();
-    for (int k = tid; k < cols1 * RB; k += nt) { V* dst = &ub[ix1[rows1 + k / RB] * RB + k % RB]; *dst = P::add(*dst, res[rcap * RB + k]); }
-  }
-  __syncthreads();
-  if (d.lev == 0) {
-    const int64_t y0 = leaf_start(d, j);
-    for (int k = tid; k < nin * nrb; k += nt) {
-      const int e = k / nrb, rb = k % nrb;
-      io.y[y0 + e + (int64_t)(r0 + rb) * io.ldy] = ub[e * RB + rb];
-    }
-  } else {
-    const int len0 = d.in_len[2 * j];
-    const int64_t b0 = d.in_off[2 * j], b1 = d.in_off[2 * j + 1];
-    for (int k = tid; k < nin * nrb; k += nt) {
-      const int e = k / nrb, rb = k % nrb;
-      const int64_t off = e < len0 ? b0 + e : b1 + (e - len0);
-      io.wout[off * io.R + r0 + rb] = ub[e * RB + rb];
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------------------------
 // Streaming forward level kernel (one right-hand side). Persistent CTAs (one to four per SM,
 // by ring layout), each a producer warp and TEAMS consumer teams of TCW warps. The producer
@@ -781,6 +605,11 @@ constexpr int kFirstPairVariant = 16;
 static_assert(kFirstPairVariant + 4 == kNumFwdVariants, "pair variants close the list");
 static bool is_pair_variant(int v) { return v >= kFirstPairVariant && v < kNumFwdVariants; }
 
+template <class P>
+constexpr Arith arith_of() {
+  return std::is_same<P, FP64P>::value ? ARITH_FP64 : std::is_same<P, DF64P>::value ? ARITH_DF64 : ARITH_FP32;
+}
+
 static int default_variant(int fmt) { return fmt == IDBF_STORE_C128 ? 0 : 1; }
 
 // One level l (pair = false) or the fused pair of levels l, l + 1 (pair = true) with the
@@ -895,19 +724,7 @@ static idbf_status launch_fwd_variant(Plan* p, int l, int v, const void* x, void
     case 6: return launch_stream<P, strm::RingC>(p, l, false, false, split, x, io, st);
     default: break;
   }
-  const LevelInfo& li = p->lv[l];
-  const DevLevel d = p->level(l);
-  const typename P::mat_t* mat = (const typename P::mat_t*)p->lmat[fmt][l];
-  const int gcap = std::max(std::max(li.max_cols, li.max_rows), li.max_in);
-  const int rcap = std::max(li.max_rows, li.max_cols);
-  const size_t sm = li.max_in * sizeof(V) + 2 * gcap * sizeof(typename P::gv_t) + 2 * rcap * sizeof(V) + li.max_out * sizeof(V);
-  if (sm > 200 * 1024) return IDBF_EUNSUPPORTED;
-  if (sm > 48 * 1024) IDBF_CUDA_TRY(cudaFuncSetAttribute(k_level_fwd<P, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  int threads = ((li.max_rows_pair + 31) / 32) * 32;
-  threads = std::max(64, std::min(512, threads));
-  k_level_fwd<P, 1><<<dim3((unsigned)p->m, 1), threads, sm, st>>>(d, mat, io, gcap, rcap, li.max_in);
-  IDBF_CUDA_TRY(cudaGetLastError());
-  return IDBF_OK;
+  return node_fwd(p, arith_of<P>(), l, LevelIO{x, p->N, y, p->N, win, wout, 1}, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -960,99 +777,21 @@ static idbf_status run_fwd1(Plan* p, const void* x, void* y, int64_t ld, cudaStr
   return IDBF_OK;
 }
 
-template <class P, int RB>
+// Levels one by one: the forward apply of one right-hand side through the per-level variants, every
+// other apply through the node kernels. Boundary b lives in buffer b % 2: forward level l reads
+// b = l-1 and writes b = l, adjoint level l reads b = l and writes b = l-1.
+template <class P>
 static idbf_status run_levels(Plan* p, const void* x, void* y, int64_t R, int64_t ld, bool adjoint, cudaStream_t st,
                               int fmt) {
-  using V = typename P::vec_t;
-  if constexpr (RB == 1) {
-    if (!adjoint && R == 1) return run_fwd1<P>(p, x, y, ld, st, fmt);
-  }
-  V* ws0 = (V*)p->d_ws;
-  V* ws1 = (V*)((char*)p->d_ws + (size_t)p->max_seg_total * R * 16);
-  const int nlev = p->L + 1;
-  for (int step = 0; step < nlev; ++step) {
+  if (!adjoint && R == 1) return run_fwd1<P>(p, x, y, ld, st, fmt);
+  void* wb[2] = {p->d_ws, (char*)p->d_ws + (size_t)p->max_seg_total * R * 16};
+  for (int step = 0; step <= p->L; ++step) {
     const int l = adjoint ? p->L - step : step;
-    const LevelInfo& li = p->lv[l];
-    const DevLevel d = p->level(l);
-    const typename P::mat_t* mat = (const typename P::mat_t*)p->lmat[fmt][l];
-    IO<V> io;
-    io.x = (const V*)x; io.ldx = ld; io.y = (V*)y; io.ldy = ld; io.R = (int)R;
-    // boundary b lives in buffer b % 2; forward level l reads b = l-1 and writes b = l,
-    // adjoint level l reads b = l and writes b = l-1.
-    V* wb[2] = {ws0, ws1};
-    if (!adjoint) {
-      io.win = l > 0 ? wb[(l - 1) & 1] : nullptr;
-      io.wout = l < p->L ? wb[l & 1] : nullptr;
-    } else {
-      io.win = l < p->L ? wb[l & 1] : nullptr;
-      io.wout = l > 0 ? wb[(l - 1) & 1] : nullptr;
-    }
-    const int gcap = std::max(std::max(li.max_cols, li.max_rows), li.max_in);
-    const int rcap = std::max(li.max_rows, li.max_cols);
-    dim3 grid((unsigned)p->m, (unsigned)((R + RB - 1) / RB));
-    if (!adjoint && RB == 1) {
-      // one right-hand side, forward: the per-level variant (autotuned, else the default)
-      const int v = p->uneven ? 0
-                    : p->tuned[fmt].size() > (size_t)l && p->tuned[fmt][l] >= 0 ? p->tuned[fmt][l] : default_variant(fmt);
-      idbf_status s = launch_fwd_variant<P>(p, l, v, x, y, io.win, io.wout, st, fmt);
-      if (s == IDBF_EUNSUPPORTED && v != 0) s = launch_fwd_variant<P>(p, l, 0, x, y, io.win, io.wout, st, fmt);
-      if (s != IDBF_OK) return s;
-      continue;
-    }
-    if constexpr (RB >= 8 && tiled_ok<P>()) {
-      if (!adjoint && !p->uneven) {
-      // several right-hand sides, FP32 / FP64: register tiles over streamed factor columns
-      // short blocks: 128 threads per CTA, so that more nodes (each a chain of dependent memory
-      // accesses) are in flight per SM
-      // (FP32: up to 85 registers per thread there), else 256 threads (FP32: up to 128 registers;
-      // FP64: unbounded, its tiles need more)
-      constexpr bool f32 = sizeof(V) == 8;
-      const bool small = f32 && li.max_rows <= 64;
-      const int nt = small ? 128 : 256;
-      const size_t sm = tiled::smem_bytes<P, RB, 4>(li.max_in, li.max_out, li.max_rows, nt);
-      if (sm <= 200 * 1024) {
-        auto kern = !f32 ? k_level_fwd_tiled<P, RB, 4, 1> : small ? k_level_fwd_tiled<P, RB, 4, f32 ? 3 : 1>
-                                                                  : k_level_fwd_tiled<P, RB, 4, f32 ? 2 : 1>;
-        if (sm > 48 * 1024)
-          IDBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        const int nblk = (int)((R + RB - 1) / RB);
-        kern<<<(unsigned)(p->m * nblk), nt, sm, st>>>(d, mat, io, li.max_rows, li.max_in, li.max_out, nblk);
-        IDBF_CUDA_TRY(cudaGetLastError());
-        continue;
-      }
-      }
-    }
-    if (!adjoint) {
-      // several right-hand sides: (row, pair of right-hand sides, column slice) per thread
-      constexpr int RPT = RB >= 2 ? 2 : 1;
-      constexpr int NT = 256;
-      const size_t sm = fwd_node_smem<P, RB, RPT>(li.max_in, gcap, rcap, NT);
-      if (sm > 200 * 1024) return IDBF_EUNSUPPORTED;
-      if (sm > 48 * 1024)
-        IDBF_CUDA_TRY(cudaFuncSetAttribute(k_level_fwd<P, RB, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-      k_level_fwd<P, RB, RPT><<<grid, NT, sm, st>>>(d, mat, io, gcap, rcap, li.max_in);
-    } else {
-      if constexpr (RB >= 8 && tiled_ok<P>()) {
-        // several right-hand sides, FP32 / FP64: register tiles over streamed row chunks
-        const size_t sm = tadj::smem_bytes<P, RB>(li.max_in, li.max_out, li.max_rows, li.max_cols);
-        if (sm <= 200 * 1024 && !p->uneven) {
-          constexpr bool f32 = sizeof(V) == 8;
-          auto kern = k_level_adj_tiled<P, RB, f32 ? 2 : 1>;
-          if (sm > 48 * 1024) IDBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-          const int nblk = (int)((R + RB - 1) / RB);
-          kern<<<(unsigned)(p->m * nblk), 256, sm, st>>>(d, mat, io, li.max_in, li.max_out, li.max_rows, li.max_cols,
-                                                          nblk);
-          IDBF_CUDA_TRY(cudaGetLastError());
-          continue;
-        }
-      }
-      const size_t sm = (size_t)RB * (li.max_out * sizeof(V) + 2 * gcap * sizeof(typename P::gv_t) +
-                                      2 * rcap * sizeof(V) + li.max_in * sizeof(V));
-      if (sm > 200 * 1024) return IDBF_EUNSUPPORTED;
-      if (sm > 48 * 1024) IDBF_CUDA_TRY(cudaFuncSetAttribute(k_level_adj<P, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-      k_level_adj<P, RB><<<grid, 256, sm, st>>>(d, mat, io, gcap, rcap, li.max_out);
-    }
-    IDBF_CUDA_TRY(cudaGetLastError());
+    void* lo = l > 0 ? wb[(l - 1) & 1] : nullptr;
+    void* hi = l < p->L ? wb[l & 1] : nullptr;
+    const LevelIO io{x, ld, y, ld, adjoint ? hi : lo, adjoint ? lo : hi, (int)R};
+    const idbf_status s = adjoint ? node_adj(p, arith_of<P>(), l, io, st) : node_fwd(p, arith_of<P>(), l, io, st);
+    if (s != IDBF_OK) return s;
   }
   return IDBF_OK;
 }
@@ -1089,62 +828,22 @@ static idbf_status apply_common(idbf_plan h, const void* x, void* y, int64_t nrh
   if (s != IDBF_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
   if (tensor) return apply_tf32x3(p, x, y, nrhs, ld, st, mode == IDBF_MODE_TF32X3_S64);
-  const bool one = nrhs == 1;
-  // several right-hand sides in FP32 / FP64 (forward and adjoint): 16 per tile from 16 on, else 8
-  const bool wide = nrhs >= 16, mid = nrhs > 1;
-  idbf_status s2 = IDBF_EUNSUPPORTED;
   switch (mode) {
-    case IDBF_MODE_FP64:
-      if (one) return run_levels<FP64P, 1>(p, x, y, nrhs, ld, adjoint, st, fmt);
-      if (wide) s2 = run_levels<FP64P, 16>(p, x, y, nrhs, ld, adjoint, st, fmt);
-      else if (mid) s2 = run_levels<FP64P, 8>(p, x, y, nrhs, ld, adjoint, st, fmt);
-      // a level too large for the wide tiles' shared memory: all levels again with 4 per tile
-      return s2 != IDBF_EUNSUPPORTED ? s2 : run_levels<FP64P, 4>(p, x, y, nrhs, ld, adjoint, st, fmt);
-    case IDBF_MODE_DF64: return one ? run_levels<DF64P, 1>(p, x, y, nrhs, ld, adjoint, st, fmt)
-                                    : run_levels<DF64P, 4>(p, x, y, nrhs, ld, adjoint, st, fmt);
-    default:
-      if (one) return run_levels<FP32P, 1>(p, x, y, nrhs, ld, adjoint, st, fmt);
-      if (wide) s2 = run_levels<FP32P, 16>(p, x, y, nrhs, ld, adjoint, st, fmt);
-      else if (mid) s2 = run_levels<FP32P, 8>(p, x, y, nrhs, ld, adjoint, st, fmt);
-      return s2 != IDBF_EUNSUPPORTED ? s2 : run_levels<FP32P, 4>(p, x, y, nrhs, ld, adjoint, st, fmt);
+    case IDBF_MODE_FP64: return run_levels<FP64P>(p, x, y, nrhs, ld, adjoint, st, fmt);
+    case IDBF_MODE_DF64: return run_levels<DF64P>(p, x, y, nrhs, ld, adjoint, st, fmt);
+    default: return run_levels<FP32P>(p, x, y, nrhs, ld, adjoint, st, fmt);
   }
 }
 
 // ---------------------------------------------------------------------------------------------
 // The middle factor S^h of IDBF_MODE_TF32X3_S64 (the other levels run on the tensor cores): the
 // complex64 boundaries h_V - 1 and h_V of the workspace, the products and sums in double-float
-// (DF64 storage of the level, preferred: FP32 issue) or FP64 (C128 storage: the FP64 pipes), four
-// right-hand sides per CTA, two per thread.
+// (DF64 storage of the level, preferred: FP32 issue) or FP64 (C128 storage: the FP64 pipes).
 idbf_status apply_middle_wide(Plan* p, const void* win, void* wout, int64_t R, cudaStream_t st) {
   const int l = p->hV;
-  const LevelInfo& li = p->lv[l];
   const bool df = p->lmat[IDBF_STORE_DF64][l] != nullptr;
   if (!df && !p->lmat[IDBF_STORE_C128][l]) return IDBF_EUNSUPPORTED;
-  constexpr int RPT = 2, NT = 256;
-  const int gcap = std::max(std::max(li.max_cols, li.max_rows), li.max_in);
-  const int rcap = std::max(li.max_rows, li.max_cols);
-  const DevLevel d = p->level(l);
-  IO<float2> io;
-  io.x = nullptr; io.ldx = p->N; io.y = nullptr; io.ldy = p->N; io.R = (int)R;
-  io.win = (const float2*)win; io.wout = (float2*)wout;
-  // four right-hand sides per CTA: two CTAs per SM (eight per CTA halve the re-reads of the
-  // node's blocks but leave one CTA per SM: 348 ms against 200 ms for this level at N = 2^18 with
-  // 256 right-hand sides)
-  auto go = [&](auto pol, auto rbc, const void* mat) -> idbf_status {
-    using Pol = decltype(pol);
-    constexpr int RB = decltype(rbc)::value;
-    const size_t sm = fwd_node_smem<Pol, RB, RPT>(li.max_in, gcap, rcap, NT);
-    if (sm > 200 * 1024) return IDBF_EUNSUPPORTED;
-    if (sm > 48 * 1024)
-      IDBF_CUDA_TRY(cudaFuncSetAttribute(k_level_fwd<Pol, RB, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    const dim3 grid((unsigned)p->m, (unsigned)((R + RB - 1) / RB));
-    k_level_fwd<Pol, RB, RPT><<<grid, NT, sm, st>>>(d, (const typename Pol::mat_t*)mat, io, gcap, rcap, li.max_in);
-    IDBF_CUDA_TRY(cudaGetLastError());
-    return IDBF_OK;
-  };
-  using RB4 = std::integral_constant<int, 4>;
-  if (df) return go(DF64S32P(), RB4(), p->lmat[IDBF_STORE_DF64][l]);
-  return go(FP64S32P(), RB4(), p->lmat[IDBF_STORE_C128][l]);
+  return node_fwd(p, df ? ARITH_DF64_C64 : ARITH_FP64_C64, l, LevelIO{nullptr, p->N, nullptr, p->N, win, wout, (int)R}, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1175,7 +874,8 @@ static idbf_status noalloc_scratch(int dev, void** out) {
   return IDBF_OK;
 }
 
-// Shared memory of the per-node forward kernel k_level_fwd<P, RB> on level l.
+// The size limit of the allocation-free apply on level l: 200 KB for the inputs, operands, products
+// and outputs of a node, RB right-hand sides at a time (the node kernels themselves need less).
 template <class P, int RB>
 static size_t scratch_level_smem(const Plan* p, int l) {
   using V = typename P::vec_t;
@@ -1187,32 +887,16 @@ static size_t scratch_level_smem(const Plan* p, int l) {
 }
 
 // The forward level loop of run_levels with the two ping-pong buffers placed in `ws`. Every
-// level's shared memory is checked before the first launch, so that a refused request leaves
-// y untouched.
+// level's size is checked before the first launch, so that a refused request leaves y untouched.
 template <class P, int RB>
-static idbf_status run_levels_scratch(Plan* p, const void* x, void* y, int64_t R, int64_t ld, cudaStream_t st,
-                                      int fmt, void* ws) {
-  using V = typename P::vec_t;
+static idbf_status run_levels_scratch(Plan* p, const void* x, void* y, int64_t R, int64_t ld, cudaStream_t st, void* ws) {
   for (int l = 0; l <= p->L; ++l)
     if (scratch_level_smem<P, RB>(p, l) > 200 * 1024) return IDBF_EUNSUPPORTED;
-  V* wb[2] = {(V*)ws, (V*)((char*)ws + (size_t)p->max_seg_total * R * 16)};
+  void* wb[2] = {ws, (char*)ws + (size_t)p->max_seg_total * R * 16};
   for (int l = 0; l <= p->L; ++l) {
-    const LevelInfo& li = p->lv[l];
-    const DevLevel d = p->level(l);
-    const typename P::mat_t* mat = (const typename P::mat_t*)p->lmat[fmt][l];
-    IO<V> io;
-    io.x = (const V*)x; io.ldx = ld; io.y = (V*)y; io.ldy = ld; io.R = (int)R;
-    io.win = l > 0 ? wb[(l - 1) & 1] : nullptr;
-    io.wout = l < p->L ? wb[l & 1] : nullptr;
-    const int gcap = std::max(std::max(li.max_cols, li.max_rows), li.max_in);
-    const int rcap = std::max(li.max_rows, li.max_cols);
-    dim3 grid((unsigned)p->m, (unsigned)((R + RB - 1) / RB));
-    const size_t sm = scratch_level_smem<P, RB>(p, l);
-    if (sm > 48 * 1024) IDBF_CUDA_TRY(cudaFuncSetAttribute(k_level_fwd<P, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    int threads = ((li.max_rows_pair + 31) / 32) * 32;
-    threads = std::max(64, std::min(512, threads));
-    k_level_fwd<P, RB><<<grid, threads, sm, st>>>(d, mat, io, gcap, rcap, li.max_in);
-    IDBF_CUDA_TRY(cudaGetLastError());
+    const LevelIO io{x, ld, y, ld, l > 0 ? wb[(l - 1) & 1] : nullptr, l < p->L ? wb[l & 1] : nullptr, (int)R};
+    const idbf_status s = node_fwd(p, arith_of<P>(), l, io, st);
+    if (s != IDBF_OK) return s;
   }
   return IDBF_OK;
 }
@@ -1234,7 +918,7 @@ static idbf_status autotune_fmt(Plan* p, int fmt, cudaStream_t st, int reps, flo
   cudaEventCreate(&e1);
   // workspace filled with real values: every level once, boundary b left in buffer b % 2
   p->tuned[fmt].assign(p->L + 1, -1);
-  s = run_levels<P, 1>(p, x, y, 1, p->N, false, st, fmt);
+  s = run_levels<P>(p, x, y, 1, p->N, false, st, fmt);
   // best time of one variant (single level: v < kFirstPairVariant; else the pair l, l + 1)
   auto time_variant = [&](int l, int v, float* ms_out) -> idbf_status {
     const V* win = l > 0 ? wb[(l - 1) & 1] : nullptr;
@@ -1363,12 +1047,12 @@ idbf_status idbf_apply_noalloc(idbf_plan h, const void* x, void* y, int64_t nrhs
   cudaStream_t st = (cudaStream_t)stream;
   const bool one = nrhs == 1;
   switch (mode) {
-    case IDBF_MODE_FP64: return one ? run_levels_scratch<FP64P, 1>(p, x, y, nrhs, ld, st, fmt, ws)
-                                    : run_levels_scratch<FP64P, 4>(p, x, y, nrhs, ld, st, fmt, ws);
-    case IDBF_MODE_DF64: return one ? run_levels_scratch<DF64P, 1>(p, x, y, nrhs, ld, st, fmt, ws)
-                                    : run_levels_scratch<DF64P, 4>(p, x, y, nrhs, ld, st, fmt, ws);
-    default: return one ? run_levels_scratch<FP32P, 1>(p, x, y, nrhs, ld, st, fmt, ws)
-                        : run_levels_scratch<FP32P, 4>(p, x, y, nrhs, ld, st, fmt, ws);
+    case IDBF_MODE_FP64: return one ? run_levels_scratch<FP64P, 1>(p, x, y, nrhs, ld, st, ws)
+                                    : run_levels_scratch<FP64P, 4>(p, x, y, nrhs, ld, st, ws);
+    case IDBF_MODE_DF64: return one ? run_levels_scratch<DF64P, 1>(p, x, y, nrhs, ld, st, ws)
+                                    : run_levels_scratch<DF64P, 4>(p, x, y, nrhs, ld, st, ws);
+    default: return one ? run_levels_scratch<FP32P, 1>(p, x, y, nrhs, ld, st, ws)
+                        : run_levels_scratch<FP32P, 4>(p, x, y, nrhs, ld, st, ws);
   }
 }
 

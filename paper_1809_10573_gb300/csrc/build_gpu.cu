@@ -671,37 +671,34 @@ template <bool DF>
 __global__ void k_emit(const IDDesc* __restrict__ D, const EmitDesc* __restrict__ E, const double2* __restrict__ Aall,
                        const int32_t* __restrict__ pscr, const int32_t* __restrict__ bl, const int32_t* __restrict__ kin,
                        double2* __restrict__ Tout, int32_t* __restrict__ Iout, int32_t* __restrict__ Sout, int side) {
-  extern __shared__ int32_t sq[];  // q[k], order[k]
+  extern __shared__ int32_t sq[];  // perm[b], order[b]: sorted position -> pivot position, skeletons then the rest
   const IDDesc d = D[blockIdx.x];
   const EmitDesc e = E[blockIdx.x];
   const int k = kin[blockIdx.x], b = d.b, np = b - k, ns = d.ns;
   const int32_t* perm = pscr + d.bl_off;
-  int32_t* order = sq + k;
-  for (int i = threadIdx.x; i < k; i += blockDim.x) sq[i] = perm[i];
+  int32_t* order = sq + b;
+  for (int i = threadIdx.x; i < b; i += blockDim.x) sq[i] = perm[i];
   __syncthreads();
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+  // skeletons and redundant columns, each in ascending order (the apply cuts nodes into slices of
+  // consecutive positions, whose rows or columns of a block are consecutive only in this order)
+  for (int i = threadIdx.x; i < b; i += blockDim.x) {
     const int32_t v = sq[i];
-    int rank = 0;
-    for (int l = 0; l < k; ++l) rank += sq[l] < v;
-    order[rank] = i;  // sorted position rank holds original skeleton i
+    const int lo = i < k ? 0 : k, hi = i < k ? k : b;
+    int rank = lo;
+    for (int l = lo; l < hi; ++l) rank += sq[l] < v;
+    order[rank] = i;
   }
   __syncthreads();
-  for (int r = threadIdx.x; r < k; r += blockDim.x) {
+  for (int r = threadIdx.x; r < b; r += blockDim.x) {
     const int32_t q = sq[order[r]];
     Iout[e.i_off + r] = q;
-    Sout[e.s_off + r] = bl[d.bl_off + q];
+    if (r < k) Sout[e.s_off + r] = bl[d.bl_off + q];
   }
-  for (int c = threadIdx.x; c < np; c += blockDim.x) Iout[e.i_off + k + c] = perm[k + c];
   const double2* A = Aall + d.a_off;
   auto at = [&](int64_t i) -> double2 { return DF ? df_join(((const float4*)A)[i]) : A[i]; };
   for (int64_t t = threadIdx.x; t < (int64_t)k * np; t += blockDim.x) {
-    if (side == 0) {
-      const int r = (int)(t / np), c = (int)(t % np);
-      Tout[e.t_off + t] = at((int64_t)(k + c) * ns + order[r]);
-    } else {
-      const int c = (int)(t / k), r = (int)(t % k);
-      Tout[e.t_off + t] = at((int64_t)(k + c) * ns + order[r]);
-    }
+    const int r = side == 0 ? (int)(t / np) : (int)(t % k), c = side == 0 ? (int)(t % np) : (int)(t / k);
+    Tout[e.t_off + t] = at((int64_t)order[k + c] * ns + order[r]);
   }
 }
 
@@ -990,7 +987,6 @@ idbf_status Builder::run_step(int side, int s) {
     r.lo = bt.lo; r.hi = bt.hi; r.T = nullptr; r.I = nullptr; r.S = nullptr;
     std::vector<EmitDesc> E(nb);
     int64_t to = 0, io = 0, sk = 0;
-    int maxk = 1;
     for (int64_t i = 0; i < nb; ++i) {
       const int k = kb[i], b = Db[i].b;
       out.k[bt.lo + i] = k;
@@ -998,7 +994,6 @@ idbf_status Builder::run_step(int side, int s) {
       E[i].t_off = to; to += (int64_t)k * (b - k);
       E[i].i_off = io; io += b;
       E[i].s_off = sk; sk += k;
-      maxk = std::max(maxk, k);
       r.toff.push_back(E[i].t_off); r.ioff.push_back(E[i].i_off); r.soff.push_back(E[i].s_off);
     }
     r.toff.push_back(to); r.ioff.push_back(io); r.soff.push_back(sk);
@@ -1010,7 +1005,10 @@ idbf_status Builder::run_step(int side, int s) {
     if ((e = emits.ensure(nb * sizeof(EmitDesc))) != cudaSuccess) { free_res(); return IDBF_ENOMEM; }
     TRY_CUDA(cudaMemcpyAsync(emits.p, E.data(), nb * sizeof(EmitDesc), cudaMemcpyHostToDevice, st));
     auto emit = df ? k_emit<true> : k_emit<false>;
-    emit<<<(unsigned)nb, 256, (size_t)maxk * 8, st>>>(dD, (EmitDesc*)emits.p, (double2*)A.p, (int32_t*)pscr.p,
+    const size_t smE = (size_t)maxb * 8;
+    if (smE > 200 * 1024) { free_res(); return IDBF_EUNSUPPORTED; }  // never above the QR's own need
+    if (smE > 48 * 1024) TRY_CUDA(cudaFuncSetAttribute(emit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smE));
+    emit<<<(unsigned)nb, 256, smE, st>>>(dD, (EmitDesc*)emits.p, (double2*)A.p, (int32_t*)pscr.p,
                                                     (int32_t*)blist.p, (int32_t*)kbuf.p, (double2*)res.back().T,
                                                     res.back().I, res.back().S, side);
     TRY_CUDA(cudaGetLastError());

@@ -127,6 +127,23 @@ idbf_status convert_storage(Plan* p, uint32_t mask, cudaStream_t st);
 // workspace (apply.cu)
 idbf_status ensure_workspace(Plan* p, int64_t nrhs);
 
+// arithmetic of a level on the CUDA cores; the last two take complex64 vectors (the middle factor
+// of IDBF_MODE_TF32X3_S64)
+enum Arith { ARITH_FP64, ARITH_DF64, ARITH_FP32, ARITH_FP64_C64, ARITH_DF64_C64 };
+// vectors of one level: the user blocks (leading dimensions ldx, ldy) and the workspace boundaries
+struct LevelIO {
+  const void* x;
+  int64_t ldx;
+  void* y;
+  int64_t ldy;
+  const void* win;
+  void* wout;
+  int R;
+};
+// level l with the node kernels (node.cu), R right-hand sides
+idbf_status node_fwd(Plan* p, Arith a, int l, const LevelIO& io, cudaStream_t st);
+idbf_status node_adj(Plan* p, Arith a, int l, const LevelIO& io, cudaStream_t st);
+
 // 3xTF32 tensor-core forward apply of all levels (apply_tc.cu); workspace must be reserved.
 // wide_middle: the middle factor in FP64 / double-float on the CUDA cores (apply_middle_wide).
 idbf_status apply_tf32x3(Plan* p, const void* x, void* y, int64_t R, int64_t ld, cudaStream_t st, bool wide_middle);

@@ -1,0 +1,545 @@
+// Per-node bodies of the level kernels, forward and adjoint, for any number of right-hand sides.
+//
+// A CTA computes one slice of one node for a block of RB right-hand sides. The node's input
+// vectors are staged once in shared memory as operands; the factor blocks are read straight from
+// global memory into registers (a warp reads consecutive rows of a column), several columns ahead,
+// with no barrier between a node's first and last column, so that the loads of all resident CTAs
+// overlap freely and the memory system, or the FMA pipes, set the time. Every thread keeps a
+// small tile of the result in registers (rows or columns x right-hand sides).
+//
+// What bounds it: with one right-hand side the factor bytes (HBM) or the FP64 pipe; with many,
+// the FMA pipes.
+#pragma once
+
+#include "level_kernels.cuh"
+
+namespace idbf {
+namespace node {
+
+// double-float vectors between levels stay in the double-float format for any number of
+// right-hand sides
+template <class P>
+using BndOf = Bnd<P, std::is_same<P, DF64P>::value>;
+
+// operands of one element (RB right-hand sides) are padded by 16 bytes when a row of them is a
+// multiple of 64 bytes, so that lanes reading neighbouring elements hit different banks
+template <class P, int RB>
+__host__ __device__ constexpr int op_pitch() {
+  using G = typename P::gv_t;
+  return (RB * sizeof(G)) % 64 == 0 && RB > 1 ? RB + (int)(16 / sizeof(G)) : RB;
+}
+
+// RB operands of one element
+template <class P, int RB>
+__device__ __forceinline__ void load_ops(const typename P::gv_t* p, typename P::gv_t (&g)[RB]) {
+  if constexpr (sizeof(typename P::gv_t) == 8 && RB % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < RB; i += 2) {
+      const float4 v = *reinterpret_cast<const float4*>(p + i);
+      g[i] = make_float2(v.x, v.y);
+      g[i + 1] = make_float2(v.z, v.w);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < RB; ++i) g[i] = p[i];
+  }
+}
+
+// sum of the accumulators of lanes that differ in the lane bits below `n` (a power of two); every
+// one of those lanes gets the sum
+template <class P>
+__device__ __forceinline__ void lane_sum(typename P::acc_t& a, int n) {
+  P::flush(a);
+  for (int o = 1; o < n; o <<= 1) P::shfl_add(a, o);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Forward. Work of slice sl of nsl of node j:
+//   V and S levels: the rows [T sl / nsl, T (sl+1) / nsl) of the T = rows_0 + rows_1 output rows;
+//   U levels: the output positions [t sl / nsl, t (sl+1) / nsl) of t = concat(out_0, out_1); the
+//     rows of block c that land there are consecutive, because the lists p_c ascend.
+// A thread takes TR rows (ntile apart, so that a warp reads consecutive rows) and all RB
+// right-hand sides; when the slice has fewer row tiles than half the CTA, the columns are dealt to
+// S = 2, 4 or 8 neighbouring lanes, which add their sums by shuffles. U levels collect the
+// products in shared memory (res) and add the two terms of every position at the end.
+template <class P, int RB>
+__host__ __device__ constexpr size_t fwd_smem(int max_in, int max_out, int max_rows, int max_cols, int max_rows_pair,
+                                              bool u_level) {
+  using B = typename BndOf<P>::b_t;
+  size_t n = ((size_t)max_in * op_pitch<P, RB>() * sizeof(typename P::gv_t) + 15) & ~(size_t)15;
+  if (u_level) n += (size_t)max_rows_pair * RB * sizeof(B);
+  n += 2 * (size_t)max_cols * sizeof(int32_t);                              // operand of every column
+  n += 2 * (size_t)(u_level ? max_out : max_rows) * sizeof(int32_t);       // V: q lists; U: term of every position
+  return (n + 15) & ~(size_t)15;
+}
+
+template <class P, int RB, int TR, int U, bool STREAM>
+__device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::mat_t* __restrict__ mat,
+                                         const IO<typename P::vec_t>& io, int max_in, int max_out, int max_rows,
+                                         int max_cols, int max_rows_pair, int64_t j, int sl, int nsl, int r0,
+                                         unsigned char* smem) {
+  using G = typename P::gv_t;
+  using M = typename P::mat_t;
+  using BP = BndOf<P>;
+  using B = typename BP::b_t;
+  constexpr int PITCH = op_pitch<P, RB>();
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int nrb = min(RB, io.R - r0);
+  const bool ulev = d.kind == KIND_U;
+  G* opd = (G*)smem;
+  B* res = (B*)(smem + (((size_t)max_in * PITCH * sizeof(G) + 15) & ~(size_t)15));
+  int32_t* kix = (int32_t*)(res + (ulev ? (size_t)max_rows_pair * RB : 0));  // [2][max_cols]
+  int32_t* aux = kix + 2 * max_cols;  // V: q lists [2][max_rows]; U: terms [2][max_out]
+  __shared__ int s_ra[2], s_rb[2];    // U: rows of each block in this slice
+
+  // ---- the node: everything here is independent of the input vectors
+  const int rowsv[2] = {d.rows[2 * j], d.rows[2 * j + 1]};
+  const int colsv[2] = {d.cols[2 * j], d.cols[2 * j + 1]};
+  const int64_t mov[2] = {d.moff[2 * j], d.moff[2 * j + 1]};
+  int l0, l1;
+  int64_t i0 = 0, i1 = 0;
+  if (d.lev == 0) {
+    l0 = leaf_len(d, j);
+    l1 = 0;
+    i0 = leaf_start(d, j);
+  } else {
+    l0 = d.in_len[2 * j];
+    l1 = d.in_len[2 * j + 1];
+    i0 = d.in_off[2 * j];
+    i1 = d.in_off[2 * j + 1];
+  }
+  int ra[2], rn[2];      // first row and number of rows of each block in this slice
+  int e0 = 0, e1 = 0;    // U: output positions of this slice
+  if (!ulev) {
+    const int tot = rowsv[0] + rowsv[1];
+    const int g0 = (int)((int64_t)tot * sl / nsl), g1 = (int)((int64_t)tot * (sl + 1) / nsl);
+    ra[0] = min(g0, rowsv[0]);
+    rn[0] = min(g1, rowsv[0]) - ra[0];
+    ra[1] = max(g0 - rowsv[0], 0);
+    rn[1] = max(g1 - rowsv[0], 0) - ra[1];
+    if (d.kind == KIND_V) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int32_t* ix = d.idx + d.ioff[2 * j + c];
+        for (int i = tid; i < rn[c]; i += nt) aux[c * max_rows + ra[c] + i] = ix[ra[c] + i];
+        for (int k = tid; k < colsv[c]; k += nt) kix[c * max_cols + k] = ix[rowsv[c] + k] * PITCH;
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        for (int k = tid; k < colsv[c]; k += nt) kix[c * max_cols + k] = k * PITCH;
+    }
+  } else {
+    const int tl = l0 + rowsv[0];  // |t| = |q_0| + |p_0|
+    e0 = (int)((int64_t)tl * sl / nsl);
+    e1 = (int)((int64_t)tl * (sl + 1) / nsl);
+    if (tid < 2) {
+      s_ra[tid] = rowsv[tid];
+      s_rb[tid] = rowsv[tid];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int lc = c ? l1 : l0;
+      const int32_t* ix = d.idx + d.ioff[2 * j + c];
+      for (int i = tid; i < lc; i += nt) {
+        const int e = ix[i];
+        if (e >= e0 && e < e1) aux[c * max_out + e - e0] = i;
+      }
+      for (int r = tid; r < rowsv[c]; r += nt) {
+        const int e = ix[lc + r];
+        if (e >= e0 && e < e1) aux[c * max_out + e - e0] = ~r;
+        if (nsl > 1) {
+          const int ep = r > 0 ? ix[lc + r - 1] : -1;
+          if (e >= e0 && ep < e0) s_ra[c] = r;
+          if (e >= e1 && ep < e1) s_rb[c] = r;
+        }
+      }
+      for (int k = tid; k < colsv[c]; k += nt) kix[c * max_cols + k] = ((c ? l0 : 0) + k) * PITCH;
+    }
+  }
+  // ---- inputs -> operands
+  if (d.lev == 0) {
+    for (int i = tid; i < l0 * RB; i += nt) {
+      const int rb = i / l0, e = i - rb * l0;
+      opd[e * PITCH + rb] = P::cvt(rb < nrb ? io.x[i0 + e + (int64_t)(r0 + rb) * io.ldx] : P::zero());
+    }
+  } else {
+    const B* winb = (const B*)io.win;
+    for (int i = tid; i < (l0 + l1) * RB; i += nt) {
+      const int e = i / RB, rb = i - e * RB;
+      const int64_t off = e < l0 ? i0 + e : i1 + (e - l0);
+      opd[e * PITCH + rb] = BP::g_of(rb < nrb ? winb[off * io.R + r0 + rb] : BP::zero());
+    }
+  }
+  __syncthreads();
+  if (ulev) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      ra[c] = nsl > 1 ? s_ra[c] : 0;
+      rn[c] = (nsl > 1 ? s_rb[c] : rowsv[c]) - ra[c];
+    }
+  }
+
+  // ---- block products
+  const int nt0 = (rn[0] + TR - 1) / TR, T = nt0 + (rn[1] + TR - 1) / TR;
+  const int maxc = max(colsv[0], colsv[1]);
+  int S = 1;
+  while (S < 8 && 2 * S * T <= nt && maxc >= 16 * S) S *= 2;
+  int64_t obv[2] = {0, 0};
+  if (!ulev) {
+    obv[0] = d.out_off[out_seg_id(d, j, 0)];
+    obv[1] = d.out_off[out_seg_id(d, j, 1)];
+  }
+  B* woutb = (B*)io.wout;
+  for (int w = tid; w - lane < T * S; w += nt) {
+    const bool active = w < T * S;
+    const int tile = active ? w / S : 0, s = w & (S - 1);
+    const int c = tile >= nt0;
+    const int rt = tile - (c ? nt0 : 0);
+    const int ntc = c ? T - nt0 : nt0;
+    const int rows = c ? rowsv[1] : rowsv[0];
+    const int cols = active ? (c ? colsv[1] : colsv[0]) : 0;
+    const int rbeg = c ? ra[1] : ra[0], rcnt = c ? rn[1] : rn[0];
+    const M* Mc = mat + (c ? mov[1] : mov[0]) + rbeg;
+    const int32_t* kc = kix + c * max_cols;
+    int roff[TR];
+#pragma unroll
+    for (int i = 0; i < TR; ++i) roff[i] = min(rt + i * ntc, max(rcnt - 1, 0));
+    typename P::acc_t acc[TR][RB];
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+      for (int rb = 0; rb < RB; ++rb) P::init(acc[i][rb]);
+    // U columns per step: all their entries are loaded before the first is used
+    const int step = S * rows;
+    int k = s, off = s * rows, since = 0;
+    auto load = [&](int u, M (&mv)[TR]) {
+#pragma unroll
+      for (int i = 0; i < TR; ++i) {
+        const M* q = Mc + (off + u * step + roff[i]);
+        mv[i] = STREAM ? __ldcs(q) : __ldg(q);
+      }
+    };
+    auto mac = [&](int u, const M (&mv)[TR]) {
+      G g[RB];
+      load_ops<P, RB>(opd + kc[k + u * S], g);
+#pragma unroll
+      for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int rb = 0; rb < RB; ++rb) P::mac(acc[i][rb], mv[i], g[rb]);
+    };
+    for (; k + (U - 1) * S < cols; k += U * S, off += U * step) {
+      M mv[U][TR];
+#pragma unroll
+      for (int u = 0; u < U; ++u) load(u, mv[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) mac(u, mv[u]);
+      since += U;
+      if (since >= P::CHUNK) {
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+          for (int rb = 0; rb < RB; ++rb) P::flush(acc[i][rb]);
+        since = 0;
+      }
+    }
+    {
+      M mv[U - 1][TR];
+#pragma unroll
+      for (int u = 0; u < U - 1; ++u)
+        if (k + u * S < cols) load(u, mv[u]);
+#pragma unroll
+      for (int u = 0; u < U - 1; ++u)
+        if (k + u * S < cols) mac(u, mv[u]);
+    }
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+      for (int rb = 0; rb < RB; ++rb) lane_sum<P>(acc[i][rb], S);
+    if (!active) continue;
+    // every lane of the S has the sums: lane s writes the right-hand sides rb = s mod S
+#pragma unroll
+    for (int i = 0; i < TR; ++i) {
+      const int rr = rt + i * ntc;
+      if (rr >= rcnt) continue;
+#pragma unroll
+      for (int rb = 0; rb < RB; ++rb) {
+        if ((rb & (S - 1)) != s) continue;
+        B v = BP::of_acc(acc[i][rb]);
+        if (ulev) {
+          res[((size_t)(c ? rn[0] : 0) + rr) * RB + rb] = v;
+        } else if (rb < nrb) {
+          if (d.kind == KIND_V) v = BP::add(v, BP::b_of_g(opd[aux[c * max_rows + rbeg + rr] * PITCH + rb]));
+          woutb[((c ? obv[1] : obv[0]) + rbeg + rr) * io.R + r0 + rb] = v;
+        }
+      }
+    }
+  }
+  if (!ulev) return;
+
+  // ---- U levels: the two terms of every output position
+  __syncthreads();
+  const int ne = e1 - e0;
+  auto term = [&](int c, int e, int rb) -> B {
+    const int t = aux[c * max_out + e];
+    return t >= 0 ? BP::b_of_g(opd[((c ? l0 : 0) + t) * PITCH + rb]) : res[((c ? rn[0] : 0) + ~t - ra[c]) * RB + rb];
+  };
+  if (d.lev == d.L) {
+    const int64_t y0 = leaf_start(d, j) + e0;
+    for (int i = tid; i < ne * nrb; i += nt) {
+      const int rb = i / ne, e = i - rb * ne;
+      io.y[y0 + e + (int64_t)(r0 + rb) * io.ldy] = BP::v_of(BP::add(term(0, e, rb), term(1, e, rb)));
+    }
+  } else {
+    const int64_t s0 = out_seg_id(d, j, 0), s1 = out_seg_id(d, j, 1);
+    const int len0 = d.out_len[s0];
+    const int64_t b0 = d.out_off[s0], b1 = d.out_off[s1];
+    for (int i = tid; i < ne * RB; i += nt) {
+      const int e = i / RB, rb = i - e * RB;
+      if (rb >= nrb) continue;
+      const int64_t off = e0 + e < len0 ? b0 + e0 + e : b1 + (e0 + e - len0);
+      woutb[off * io.R + r0 + rb] = BP::add(term(0, e, rb), term(1, e, rb));
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Adjoint: reads the forward outputs v of node j and writes its forward inputs. An output is a
+// column of a block: sum_r conj(M_c(r, i)) g_c[r]. LR neighbouring lanes take the rows of a column
+// r = lane, lane + LR, ... (consecutive entries), the 32 / LR lane groups of a warp different
+// columns, TC columns per lane; the LR partial sums meet by shuffles.
+// Slices: U and S levels a range of columns; V levels a range of input positions [e0, e1) (the
+// columns of block c that land there are consecutive, because the lists p_c ascend).
+template <class P, int RB>
+__host__ __device__ constexpr size_t adj_smem(int max_in, int max_out, int max_rows, int max_cols_pair, bool v_level) {
+  using B = typename BndOf<P>::b_t;
+  size_t n = ((size_t)max_out * op_pitch<P, RB>() * sizeof(typename P::gv_t) + 15) & ~(size_t)15;
+  if (v_level) n += (size_t)max_cols_pair * RB * sizeof(B) + 2 * (size_t)max_in * sizeof(int32_t);
+  n += 2 * (size_t)max_rows * sizeof(int32_t);  // operand of every row
+  return (n + 15) & ~(size_t)15;
+}
+
+template <class P, int RB, int TC, int LR, int U, bool STREAM>
+__device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::mat_t* __restrict__ mat,
+                                         const IO<typename P::vec_t>& io, int max_in, int max_out, int max_rows,
+                                         int max_cols_pair, int64_t j, int sl, int nsl, int r0, unsigned char* smem) {
+  using G = typename P::gv_t;
+  using M = typename P::mat_t;
+  using BP = BndOf<P>;
+  using B = typename BP::b_t;
+  constexpr int PITCH = op_pitch<P, RB>();
+  constexpr int CG = 32 / LR, CT = CG * TC;  // lane groups of a warp, columns of a warp's tile
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  const int lr = lane & (LR - 1), cg = lane / LR;
+  const int nrb = min(RB, io.R - r0);
+  const bool vlev = d.kind == KIND_V;
+  G* opd = (G*)smem;
+  B* res = (B*)(smem + (((size_t)max_out * PITCH * sizeof(G) + 15) & ~(size_t)15));
+  int32_t* gix = (int32_t*)(res + (vlev ? (size_t)max_cols_pair * RB : 0));  // [2][max_rows]
+  int32_t* aux = gix + 2 * max_rows;                                          // V: terms [2][max_in]
+  __shared__ int s_ia[2], s_ib[2];  // V: columns of each block in this slice
+
+  const int rowsv[2] = {d.rows[2 * j], d.rows[2 * j + 1]};
+  const int colsv[2] = {d.cols[2 * j], d.cols[2 * j + 1]};
+  const int64_t mov[2] = {d.moff[2 * j], d.moff[2 * j + 1]};
+  int o0len, o1len = 0;
+  int64_t b0, b1 = 0;
+  if (d.lev == d.L) {
+    o0len = leaf_len(d, j);
+    b0 = leaf_start(d, j);
+  } else {
+    const int64_t s0 = out_seg_id(d, j, 0), s1 = out_seg_id(d, j, 1);
+    o0len = d.out_len[s0];
+    o1len = d.out_len[s1];
+    b0 = d.out_off[s0];
+    b1 = d.out_off[s1];
+  }
+  int ia[2] = {0, 0}, in[2] = {colsv[0], colsv[1]};  // first column and number of columns of each block
+  int e0 = 0, e1 = 0;
+  if (vlev) {
+    const int nin = rowsv[0] + colsv[0];
+    e0 = (int)((int64_t)nin * sl / nsl);
+    e1 = (int)((int64_t)nin * (sl + 1) / nsl);
+    if (tid < 2) {
+      s_ia[tid] = colsv[tid];
+      s_ib[tid] = colsv[tid];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int32_t* ix = d.idx + d.ioff[2 * j + c];
+      for (int r = tid; r < rowsv[c]; r += nt) {
+        const int e = ix[r];
+        if (e >= e0 && e < e1) aux[c * max_in + e - e0] = r;
+        gix[c * max_rows + r] = ((c ? o0len : 0) + r) * PITCH;
+      }
+      for (int i = tid; i < colsv[c]; i += nt) {
+        const int e = ix[rowsv[c] + i];
+        if (e >= e0 && e < e1) aux[c * max_in + e - e0] = ~i;
+        if (nsl > 1) {
+          const int ep = i > 0 ? ix[rowsv[c] + i - 1] : -1;
+          if (e >= e0 && ep < e0) s_ia[c] = i;
+          if (e >= e1 && ep < e1) s_ib[c] = i;
+        }
+      }
+    }
+  } else {
+    const int tot = d.kind == KIND_S ? colsv[0] : colsv[0] + colsv[1];
+    const int g0 = (int)((int64_t)tot * sl / nsl), g1 = (int)((int64_t)tot * (sl + 1) / nsl);
+    ia[0] = min(g0, colsv[0]);
+    in[0] = min(g1, colsv[0]) - ia[0];
+    ia[1] = max(g0 - colsv[0], 0);
+    in[1] = max(g1 - colsv[0], 0) - ia[1];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int32_t* ix = d.kind == KIND_U ? d.idx + d.ioff[2 * j + c] + colsv[c] : nullptr;
+      for (int r = tid; r < rowsv[c]; r += nt) gix[c * max_rows + r] = (ix ? ix[r] : (c ? o0len : 0) + r) * PITCH;
+    }
+  }
+  // ---- inputs -> operands
+  if (d.lev == d.L) {
+    for (int i = tid; i < o0len * RB; i += nt) {
+      const int rb = i / o0len, e = i - rb * o0len;
+      opd[e * PITCH + rb] = P::cvt(rb < nrb ? io.x[b0 + e + (int64_t)(r0 + rb) * io.ldx] : P::zero());
+    }
+  } else {
+    const B* winb = (const B*)io.win;
+    for (int i = tid; i < (o0len + o1len) * RB; i += nt) {
+      const int e = i / RB, rb = i - e * RB;
+      const int64_t off = e < o0len ? b0 + e : b1 + (e - o0len);
+      opd[e * PITCH + rb] = BP::g_of(rb < nrb ? winb[off * io.R + r0 + rb] : BP::zero());
+    }
+  }
+  __syncthreads();
+  if (vlev) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      ia[c] = nsl > 1 ? s_ia[c] : 0;
+      in[c] = (nsl > 1 ? s_ib[c] : colsv[c]) - ia[c];
+    }
+  }
+  const bool slev = d.kind == KIND_S;
+  const int nt0 = (in[0] + CT - 1) / CT, T = nt0 + (slev ? 0 : (in[1] + CT - 1) / CT);
+  int64_t ib0 = 0, ib1 = 0;
+  int len0 = 0;
+  if (d.lev > 0) {
+    len0 = d.in_len[2 * j];
+    ib0 = d.in_off[2 * j];
+    ib1 = d.in_off[2 * j + 1];
+  }
+  B* woutb = (B*)io.wout;
+  for (int w = warp; w < T; w += nw) {
+    const int c = w >= nt0;
+    const int i_first = (w - (c ? nt0 : 0)) * CT + cg;  // this lane's first column within the slice
+    const int icnt = c ? in[1] : in[0], ibeg = c ? ia[1] : ia[0];
+    typename P::acc_t acc[TC][RB];
+#pragma unroll
+    for (int t = 0; t < TC; ++t)
+#pragma unroll
+      for (int rb = 0; rb < RB; ++rb) P::init(acc[t][rb]);
+    int coff[TC];
+#pragma unroll
+    for (int t = 0; t < TC; ++t) coff[t] = ibeg + min(i_first + t * CG, icnt - 1);
+    for (int bc = c; bc <= (slev ? 1 : c); ++bc) {  // S levels: both blocks have the same columns
+      const int rows = bc ? rowsv[1] : rowsv[0];
+      const M* Mc = mat + (bc ? mov[1] : mov[0]);
+      const int32_t* gc = gix + bc * max_rows;
+      int base[TC];
+#pragma unroll
+      for (int t = 0; t < TC; ++t) base[t] = coff[t] * rows;
+      int r = lr, since = 0;
+      auto load = [&](int u, M (&mv)[TC]) {
+#pragma unroll
+        for (int t = 0; t < TC; ++t) {
+          const M* q = Mc + (base[t] + r + u * LR);
+          mv[t] = STREAM ? __ldcs(q) : __ldg(q);
+        }
+      };
+      auto mac = [&](int u, const M (&mv)[TC]) {
+        G g[RB];
+        load_ops<P, RB>(opd + gc[r + u * LR], g);
+#pragma unroll
+        for (int t = 0; t < TC; ++t)
+#pragma unroll
+          for (int rb = 0; rb < RB; ++rb) P::macc(acc[t][rb], mv[t], g[rb]);
+      };
+      for (; r + (U - 1) * LR < rows; r += U * LR) {
+        M mv[U][TC];
+#pragma unroll
+        for (int u = 0; u < U; ++u) load(u, mv[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) mac(u, mv[u]);
+        since += U;
+        if (since >= P::CHUNK) {
+#pragma unroll
+          for (int t = 0; t < TC; ++t)
+#pragma unroll
+            for (int rb = 0; rb < RB; ++rb) P::flush(acc[t][rb]);
+          since = 0;
+        }
+      }
+      if constexpr (U > 1) {
+        M mv[U - 1][TC];
+#pragma unroll
+        for (int u = 0; u < U - 1; ++u)
+          if (r + u * LR < rows) load(u, mv[u]);
+#pragma unroll
+        for (int u = 0; u < U - 1; ++u)
+          if (r + u * LR < rows) mac(u, mv[u]);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < TC; ++t)
+#pragma unroll
+      for (int rb = 0; rb < RB; ++rb) lane_sum<P>(acc[t][rb], LR);
+#pragma unroll
+    for (int t = 0; t < TC; ++t) {
+      const int ii = i_first + t * CG;
+      if (ii >= icnt) continue;
+      const int i = ibeg + ii;
+#pragma unroll
+      for (int rb = 0; rb < RB; ++rb) {
+        if ((rb & (LR - 1)) != lr) continue;
+        B v = BP::of_acc(acc[t][rb]);
+        if (vlev) {
+          res[((c ? in[0] : 0) + ii) * RB + rb] = v;
+        } else if (rb < nrb) {
+          if (slev) {
+            woutb[(i < len0 ? ib0 + i : ib1 + (i - len0)) * io.R + r0 + rb] = v;
+          } else {  // U: forward input segment c gets v[q_c] + res_c
+            const int q = d.idx[d.ioff[2 * j + c] + i];
+            woutb[((c ? ib1 : ib0) + i) * io.R + r0 + rb] = BP::add(BP::b_of_g(opd[q * PITCH + rb]), v);
+          }
+        }
+      }
+    }
+  }
+  if (!vlev) return;
+
+  // ---- V levels: the two terms of every input position
+  __syncthreads();
+  const int ne = e1 - e0;
+  auto term = [&](int c, int e, int rb) -> B {
+    const int t = aux[c * max_in + e];
+    return t >= 0 ? BP::b_of_g(opd[((c ? o0len : 0) + t) * PITCH + rb]) : res[((c ? in[0] : 0) + ~t - ia[c]) * RB + rb];
+  };
+  if (d.lev == 0) {
+    const int64_t y0 = leaf_start(d, j) + e0;
+    for (int i = tid; i < ne * nrb; i += nt) {
+      const int rb = i / ne, e = i - rb * ne;
+      io.y[y0 + e + (int64_t)(r0 + rb) * io.ldy] = BP::v_of(BP::add(term(0, e, rb), term(1, e, rb)));
+    }
+  } else {
+    for (int i = tid; i < ne * RB; i += nt) {
+      const int e = i / RB, rb = i - e * RB;
+      if (rb >= nrb) continue;
+      const int f = e0 + e;
+      woutb[(f < len0 ? ib0 + f : ib1 + (f - len0)) * io.R + r0 + rb] = BP::add(term(0, e, rb), term(1, e, rb));
+    }
+  }
+}
+
+}  // namespace node
+}  // namespace idbf

@@ -423,19 +423,30 @@ idbf_status idbf_import_factors(const idbf_host_factors* f, int32_t storage, voi
     p.mat_len += tot;
     p.idx_len += itot;
     std::vector<double> colmajor;
-    std::vector<int32_t> idx;
+    std::vector<int32_t> idx, ord;
     try { colmajor.resize(2 * (size_t)tot); idx.resize(itot); } catch (...) { s = IDBF_ENOMEM; break; }
     for (int64_t o = l * nbl; o < (l + 1) * nbl; ++o) {
       const int64_t r = p.h_rows[o], c = p.h_cols[o];
       const double* src = f->mat + 2 * f->blk_moff[o];
       double* dst = colmajor.data() + 2 * p.h_moff[o];
+      // the list p_c is kept ascending (see k_emit in build_gpu.cu), with the columns (V) or rows (U)
+      // of the block in its order; q_c, the order of the segment entries, stays as given
+      const int kind = p.lv[l].kind;
+      ord.resize(kind == KIND_V ? c : kind == KIND_U ? r : 0);
+      if (kind != KIND_S) {
+        const int64_t nq = kind == KIND_V ? r : c;
+        const int32_t* pl = f->idx + f->blk_ioff[o] + nq;
+        for (size_t i = 0; i < ord.size(); ++i) ord[i] = (int32_t)i;
+        std::sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return pl[a] < pl[b]; });
+        if (nq > 0) memcpy(idx.data() + p.h_ioff[o], f->idx + f->blk_ioff[o], nq * sizeof(int32_t));
+        for (size_t i = 0; i < ord.size(); ++i) idx[p.h_ioff[o] + nq + i] = pl[ord[i]];
+      }
       for (int64_t i = 0; i < r; ++i)
         for (int64_t j = 0; j < c; ++j) {
-          dst[2 * (j * r + i)] = src[2 * (i * c + j)];
-          dst[2 * (j * r + i) + 1] = src[2 * (i * c + j) + 1];
+          const int64_t si = kind == KIND_U ? ord[i] : i, sj = kind == KIND_V ? ord[j] : j;
+          dst[2 * (j * r + i)] = src[2 * (si * c + sj)];
+          dst[2 * (j * r + i) + 1] = src[2 * (si * c + sj) + 1];
         }
-      if (p.lv[l].kind != KIND_S)
-        memcpy(idx.data() + p.h_ioff[o], f->idx + f->blk_ioff[o], (r + c) * sizeof(int32_t));
     }
     cudaError_t e = cudaSuccess;
     if (tot > 0) {
