@@ -305,18 +305,19 @@ idbf_status idbf_sync_status(idbf_plan plan, void* stream);
  * copies so that every consumer wait runs out. Not for production use. */
 idbf_status idbf_debug_set_wait(idbf_plan plan, uint64_t limit_ns, int32_t producer_enabled);
 
-/* ---- uneven batches: many operators in one persistent launch ---------------------------- */
+/* ---- uneven batches: many operators in one graph ----------------------------------------- */
 typedef struct idbf_batch_s* idbf_batch;
 
 /* idbf_batch_create - prepare the forward apply of nops plans (any N each), plan o with nrhs[o]
- * right-hand sides, in `mode` (FP64, DF64 or FP32), as ONE persistent kernel launch captured in a
- * CUDA graph (plans with leaves of n0 points; uneven leaves: EUNSUPPORTED). Work items
- * (operator, level, run of nodes, block of right-hand sides) are queued in
- * level order and taken by persistent CTAs; an item waits (bounded) until the previous level of
- * its operator is complete. Operators from a size up can be left out of the launch and applied
- * on their own (idbf_batch_set_split, chosen by idbf_batch_autotune). Allocates each operator's
- * level workspace; the plans must outlive the batch and must not be changed (storage) while it
- * exists. Synchronous. */
+ * right-hand sides, in `mode` (FP64, DF64 or FP32), as one CUDA graph (plans with leaves of n0
+ * points; uneven leaves: EUNSUPPORTED). Depending on the tiling (idbf_batch_set_tiling) the graph
+ * holds ONE persistent kernel launch, whose work items (operator, level, run of nodes, block of
+ * right-hand sides) are queued in level order and taken by persistent CTAs, an item waiting
+ * (bounded) until the previous level of its operator is complete; or one launch per level, a chain
+ * of them for every width of the operators' right-hand-side blocks. Operators from a size up can be
+ * left out of the graph and applied on their own (idbf_batch_set_split, chosen by
+ * idbf_batch_autotune). Allocates each operator's level workspace; the plans must outlive the batch
+ * and must not be changed (storage) while it exists. Synchronous. */
 idbf_status idbf_batch_create(const idbf_plan* plans, int32_t nops, const int64_t* nrhs, int32_t mode,
                               idbf_batch* out);
 
@@ -327,23 +328,21 @@ idbf_status idbf_batch_create(const idbf_plan* plans, int32_t nops, const int64_
 idbf_status idbf_batch_apply(idbf_batch b, const void* const* x, void* const* y, const int64_t* ld,
                              void* stream);
 
-/* idbf_batch_autotune - time the batch for every tiling of idbf_batch_set_tiling below (for the
- * mixed tiling 7 also its row threshold in {32, 64, 96, 128, 192}) and nodes per item in
- * {1, 2, 4}, then, unless a split was set with idbf_batch_set_split, every split with the best
+/* idbf_batch_autotune - time the batch for every tiling of idbf_batch_set_tiling below and nodes per
+ * item in {1, 2, 4}, then, unless a split was set with idbf_batch_set_split, every split with the best
  * tiling (and the tilings again if the split changed); reps launches each, on the given buffers;
  * tilings whose shared memory exceeds 200 KB are skipped. Keeps the fastest; *best_ms receives
  * its time per idbf_batch_apply. Synchronous. */
 idbf_status idbf_batch_autotune(idbf_batch b, const void* const* x, void* const* y, const int64_t* ld,
                                 int32_t reps, void* stream, float* best_ms);
 
-/* idbf_batch_set_tiling - choose the tiling by hand: `tile` indexes the autotuner's list above
- * (0: (1,1), 1: (4,2), 2: (8,2), 3: (8,4) per-thread right-hand sides; 4: 8 and 5: 16 right-hand
- * sides per item in 4 x 4 register tiles over streamed factor columns, 6: 32 in 4 x 8 tiles;
- * 7: mixed per level, 16 per item in register tiles where a level's blocks have more than a row
- * threshold (64 unless the autotuner chose another), else 8 per item, 4 per thread; 4-7 in FP32
- * and FP64 only, 6 in FP32 only), nodes_per_item in {1, 2, 4}. IDBF_EUNSUPPORTED if the
- * tile does not exist for the batch's precision or its shared memory exceeds 200 KB (the
- * previous tiling is then kept), IDBF_EINVAL for other values. Synchronous. */
+/* idbf_batch_set_tiling - choose the tiling by hand: `tile` indexes the autotuner's list above.
+ * 0, 1, 2, 4, 6, 7: the persistent launch with 1, 4, 8, 8, 32 and 16 right-hand sides per item (128
+ * threads per CTA for 2 and 7, else 256); 3, 5: level launches, most CTAs resident (3, reported as 8
+ * right-hand sides per item) or most threads and registers per CTA (5, reported as 16). 4-7 in FP32
+ * and FP64 only, 6 in FP32 only. nodes_per_item in {1, 2, 4}. IDBF_EUNSUPPORTED if the tile does not
+ * exist for the batch's precision or its shared memory exceeds 200 KB (the previous tiling is then
+ * kept), IDBF_EINVAL for other values. Synchronous. */
 idbf_status idbf_batch_set_tiling(idbf_batch b, int32_t tile, int32_t nodes_per_item);
 
 /* idbf_batch_set_split - operators with N >= min_separate_n leave the persistent launch: each
@@ -361,7 +360,7 @@ idbf_status idbf_batch_set_split(idbf_batch b, int64_t min_separate_n);
 idbf_status idbf_batch_split(idbf_batch b, int64_t* min_separate_n, int32_t* separate_ops);
 
 /* idbf_batch_info - the current tiling: right-hand sides and nodes per work item, number of
- * items, persistent CTAs (0 and 0 when every operator runs through idbf_apply). */
+ * items, persistent CTAs (level launches: the items, one CTA each; 0 and 0 when every operator runs through idbf_apply). */
 idbf_status idbf_batch_info(idbf_batch b, int32_t* rhs_per_item, int32_t* nodes_per_item, int32_t* items,
                             int32_t* ctas);
 

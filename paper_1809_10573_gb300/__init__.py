@@ -238,8 +238,8 @@ class Plan:
 
 
 class Batch:
-    """Forward applies of several plans (uneven N, their own numbers of right-hand sides) in one
-    persistent kernel launch captured in a CUDA graph (idbf_batch_* in include/idbf.h)."""
+    """Forward applies of several plans (uneven N, their own numbers of right-hand sides) as one
+    CUDA graph: a persistent launch or one launch per level (idbf_batch_* in include/idbf.h)."""
 
     def __init__(self, plans, nrhs, mode=MODE_DF64):
         self.plans = list(plans)           # keep the plans alive as long as the batch
@@ -284,8 +284,9 @@ class Batch:
                    "idbf_batch_autotune")
         return ms.value
 
-    # tile indices of idbf_batch_set_tiling: (right-hand sides per item, per thread, register-tile width)
-    TILES = ((1, 1, 0), (4, 2, 0), (8, 2, 0), (8, 4, 0), (8, 0, 4), (16, 0, 4), (32, 0, 8), (16, 4, -1))
+    # tile indices of idbf_batch_set_tiling: (right-hand sides per item, threads per CTA of the
+    # persistent launch or 0 for level launches, 1 if in FP32 and FP64 only)
+    TILES = ((1, 256, 0), (4, 256, 0), (8, 128, 0), (8, 0, 0), (8, 256, 1), (16, 0, 1), (32, 256, 1), (16, 128, 1))
 
     def set_tiling(self, tile: int, nodes_per_item: int = 1):
         _lib.check(_lib.lib().idbf_batch_set_tiling(self._h, int(tile), int(nodes_per_item)), "idbf_batch_set_tiling")

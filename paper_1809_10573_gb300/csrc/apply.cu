@@ -697,7 +697,7 @@ static idbf_status launch_warp_node(Plan* p, int l, IO<typename P::vec_t> io, cu
 
 template <class P>
 static idbf_status launch_fwd_variant(Plan* p, int l, int v, const void* x, void* y, const typename P::vec_t* win,
-                                      typename P::vec_t* wout, cudaStream_t st, int fmt) {
+                                      typename P::vec_t* wout, cudaStream_t st, int fmt, bool after) {
   using V = typename P::vec_t;
   IO<V> io;
   io.x = (const V*)x; io.ldx = p->N; io.y = (V*)y; io.ldy = p->N; io.R = 1;
@@ -724,7 +724,7 @@ static idbf_status launch_fwd_variant(Plan* p, int l, int v, const void* x, void
     case 6: return launch_stream<P, strm::RingC>(p, l, false, false, split, x, io, st);
     default: break;
   }
-  return node_fwd(p, arith_of<P>(), l, LevelIO{x, p->N, y, p->N, win, wout, 1}, st);
+  return node_fwd(p, arith_of<P>(), l, LevelIO{x, p->N, y, p->N, win, wout, 1, after}, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -759,17 +759,17 @@ static idbf_status run_fwd1(Plan* p, const void* x, void* y, int64_t ld, cudaStr
     (void)ld;
     idbf_status s = IDBF_EUNSUPPORTED;
     if (is_pair_variant(v) && !pair) v = default_variant(fmt);  // a pair variant on level L: one level
-    s = launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt);
+    s = launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt, l > 0);
     if (s == IDBF_EUNSUPPORTED && pair) {  // the pair does not fit: level l alone, into the next buffer
       V* wout1 = wb[cur ^ 1];               // l < L here, so level l writes a workspace boundary
-      s = launch_fwd_variant<P>(p, l, default_variant(fmt), x, y, win, wout1, st, fmt);
-      if (s == IDBF_EUNSUPPORTED) s = launch_fwd_variant<P>(p, l, 0, x, y, win, wout1, st, fmt);
+      s = launch_fwd_variant<P>(p, l, default_variant(fmt), x, y, win, wout1, st, fmt, l > 0);
+      if (s == IDBF_EUNSUPPORTED) s = launch_fwd_variant<P>(p, l, 0, x, y, win, wout1, st, fmt, l > 0);
       if (s != IDBF_OK) return s;
       if (l < p->L) cur ^= 1;
       ++l;
       continue;
     }
-    if (s == IDBF_EUNSUPPORTED && v != 0) s = launch_fwd_variant<P>(p, l, 0, x, y, win, wout, st, fmt);
+    if (s == IDBF_EUNSUPPORTED && v != 0) s = launch_fwd_variant<P>(p, l, 0, x, y, win, wout, st, fmt, l > 0);
     if (s != IDBF_OK) return s;
     if (last < p->L) cur ^= 1;
     l = last + 1;
@@ -789,7 +789,7 @@ static idbf_status run_levels(Plan* p, const void* x, void* y, int64_t R, int64_
     const int l = adjoint ? p->L - step : step;
     void* lo = l > 0 ? wb[(l - 1) & 1] : nullptr;
     void* hi = l < p->L ? wb[l & 1] : nullptr;
-    const LevelIO io{x, ld, y, ld, adjoint ? hi : lo, adjoint ? lo : hi, (int)R};
+    const LevelIO io{x, ld, y, ld, adjoint ? hi : lo, adjoint ? lo : hi, (int)R, step > 0};
     const idbf_status s = adjoint ? node_adj(p, arith_of<P>(), l, io, st) : node_fwd(p, arith_of<P>(), l, io, st);
     if (s != IDBF_OK) return s;
   }
@@ -843,7 +843,7 @@ idbf_status apply_middle_wide(Plan* p, const void* win, void* wout, int64_t R, c
   const int l = p->hV;
   const bool df = p->lmat[IDBF_STORE_DF64][l] != nullptr;
   if (!df && !p->lmat[IDBF_STORE_C128][l]) return IDBF_EUNSUPPORTED;
-  return node_fwd(p, df ? ARITH_DF64_C64 : ARITH_FP64_C64, l, LevelIO{nullptr, p->N, nullptr, p->N, win, wout, (int)R}, st);
+  return node_fwd(p, df ? ARITH_DF64_C64 : ARITH_FP64_C64, l, LevelIO{nullptr, p->N, nullptr, p->N, win, wout, (int)R, false}, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -894,7 +894,7 @@ static idbf_status run_levels_scratch(Plan* p, const void* x, void* y, int64_t R
     if (scratch_level_smem<P, RB>(p, l) > 200 * 1024) return IDBF_EUNSUPPORTED;
   void* wb[2] = {ws, (char*)ws + (size_t)p->max_seg_total * R * 16};
   for (int l = 0; l <= p->L; ++l) {
-    const LevelIO io{x, ld, y, ld, l > 0 ? wb[(l - 1) & 1] : nullptr, l < p->L ? wb[l & 1] : nullptr, (int)R};
+    const LevelIO io{x, ld, y, ld, l > 0 ? wb[(l - 1) & 1] : nullptr, l < p->L ? wb[l & 1] : nullptr, (int)R, l > 0};
     const idbf_status s = node_fwd(p, arith_of<P>(), l, io, st);
     if (s != IDBF_OK) return s;
   }
@@ -924,10 +924,10 @@ static idbf_status autotune_fmt(Plan* p, int fmt, cudaStream_t st, int reps, flo
     const V* win = l > 0 ? wb[(l - 1) & 1] : nullptr;
     const int last = is_pair_variant(v) ? l + 1 : l;
     V* wout = last < p->L ? wb[l & 1] : nullptr;  // a pair's output goes to the other buffer too
-    idbf_status r = launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt);
+    idbf_status r = launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt, false);
     if (r != IDBF_OK) return r;
     cudaEventRecord(e0, st);
-    for (int k = 0; k < reps; ++k) launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt);
+    for (int k = 0; k < reps; ++k) launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt, false);
     cudaEventRecord(e1, st);
     if (cudaEventSynchronize(e1) != cudaSuccess) return IDBF_ECUDA;
     cudaEventElapsedTime(ms_out, e0, e1);

@@ -1,19 +1,25 @@
 // An uneven batch of IDBF applies (operators of different N, each with its own number of
-// right-hand sides) in ONE persistent kernel launch, captured in a CUDA graph.
+// right-hand sides) as one CUDA graph, in one of two forms (a tile, autotuned).
 //
-// Work items are (operator, level, run of nodes, block of right-hand sides). They are queued in
-// the order of the levels (all level-0 items of every operator, then all level-1 items, ...),
-// and persistent CTAs take them from the queue with an atomic counter. Before starting an item
-// of level l, a CTA waits until every item of level l-1 of the same operator has finished (a
+// Level launches: every width of right-hand-side block in the batch is a chain of launches, one per
+// level, each over all operators of that width; the chains run side by side, and a launch begins
+// (index lists, factor reads) while its predecessor drains. Each launch has the shared memory, the
+// threads and the registers of its own level and width.
+//
+// Persistent launch: work items (operator, level, run of nodes, block of right-hand sides) are
+// queued in the order of the levels (all level-0 items of every operator, then all level-1 items,
+// ...), and persistent CTAs take them from the queue with an atomic counter. Before starting an
+// item of level l, a CTA waits until every item of level l-1 of the same operator has finished (a
 // per-(operator, level) completion counter). Those items are earlier in the queue, so they have
 // already been taken by CTAs that are running, and the wait ends: there is no cycle, whatever the
-// number of resident CTAs. Every wait is bounded in time; on a timeout the item is counted as done
-// (its results are invalid), bit 0 of the status word is set, and idbf_batch_sync_status reports
-// IDBF_ETIMEOUT.
+// number of resident CTAs. (A CTA holds one item ahead of the one it computes; of all unfinished items
+// the earliest in the queue is always one being computed.) Every wait is bounded in time; on a
+// timeout the item is counted as done (its results are invalid), bit 0 of the status word is set,
+// and idbf_batch_sync_status reports IDBF_ETIMEOUT.
 //
-// Each node is computed by fwd_node (right-hand sides per thread) or fwd_node_tiled (register
-// tiles), the bodies of the per-level kernels (level_kernels.cuh); the tile, or a per-level mix
-// of the two by block height, is autotuned.
+// Each node is computed by node::fwd_body, the body of the per-level kernels (node_kernels.cuh).
+// 24 operators of N = 2^10 .. 2^14, 1-32 right-hand sides, FP32: level launches 2.60 ms, persistent
+// launch 3.31 ms, one apply after the other 4.08 ms.
 #include <cuda_runtime.h>
 #include <string.h>
 
@@ -23,7 +29,8 @@
 #include <vector>
 
 #include "idbf_internal.h"
-#include "level_kernels.cuh"
+#include "node_kernels.cuh"
+#include "node_launch.h"
 
 namespace idbf {
 namespace bat {
@@ -31,16 +38,19 @@ namespace bat {
 struct OpLevel {
   DevLevel d;
   const void* mat;
-  int gcap, rcap, max_in, max_out, max_rows;
-  int body;  // mixed tiling: 1 = tiled body (16 right-hand sides per item), 0 = per-thread body (8)
+  int max_in, max_out, max_rows, max_cols, max_rows_pair, pad;
 };
 struct OpDesc {
-  int L, R, level_base, pad;
+  int L, R, level_base;
+  int width;  // right-hand sides per item
   void* ws0;
   void* ws1;
 };
 struct Item {
   int op, level, node0, nodes, r0, pad;
+};
+struct LevelItem {  // a CTA of a level launch: slice sl of nsl of each of `nodes` nodes
+  int op, node0, nodes, r0, sl, nsl;
 };
 
 __device__ __forceinline__ uint64_t gtimer() {
@@ -49,50 +59,96 @@ __device__ __forceinline__ uint64_t gtimer() {
   return t;
 }
 
-constexpr int NT = 256;
+constexpr int NTMAX = 256;
 
-// Tiles: right-hand sides per work item (RB); then either right-hand sides per thread (RPT, the
-// per-node body fwd_node, all precisions) or TC > 0: the tiled body fwd_node_tiled with TR x TC
-// register tiles and streamed factor columns (FP32 and FP64), or TC < 0: mixed, per level: the
-// tiled body with 16 right-hand sides per item where the level's blocks have more than a
-// threshold of rows, else the per-thread body with 8 per item, 4 per thread (FP32 and FP64).
+// Tiles: right-hand sides per work item (rb; above the body's width in several passes), threads per
+// CTA of the persistent launch, or 0 for level launches, one chain of launches per width of the
+// batch's operators: with rb = 8 in the instances of the per-level kernels (most CTAs resident),
+// with rb = 16 in instances of more threads and registers per CTA, whose tall nodes finish
+// sooner (batches of few nodes: 16 operators of N = 2^9 .. 2^12 in FP32 342 against 427 us).
 struct Tile {
-  int rb, rpt, tc;
+  int rb, nt;
+  bool wide;  // FP32 and FP64 only
 };
-constexpr Tile kTiles[] = {{1, 1, 0}, {4, 2, 0}, {8, 2, 0}, {8, 4, 0}, {8, 0, 4}, {16, 0, 4}, {32, 0, 8}, {16, 4, -1}};
+constexpr Tile kTiles[] = {{1, 256, false}, {4, 256, false}, {8, 128, false}, {8, 0, false},
+                           {8, 256, true},  {16, 0, true},   {32, 256, true}, {16, 128, true}};
 constexpr int kNumTiles = 8;
-constexpr int kMixedSmallRB = 8;
 template <class P>
 __host__ __device__ constexpr int max_rb() {
   return std::is_same<P, FP32P>::value ? 32 : std::is_same<P, FP64P>::value ? 16 : 8;
 }
+// right-hand sides that one pass of the body holds in registers
 template <class P>
-__host__ __device__ constexpr bool tiled_ok() {
-  return std::is_same<typename P::vec_t, typename P::gv_t>::value;
-}
-template <class P, int T>
-constexpr bool instantiated() {
-  return kTiles[T].rb <= max_rb<P>() && (kTiles[T].tc == 0 || tiled_ok<P>());
+__host__ __device__ constexpr int pass_rb() {
+  return std::is_same<P, DF64P>::value ? 4 : 8;
 }
 
-template <class P, int RB, int RPT, int TC>
-__global__ void __launch_bounds__(NT, TC == 8 ? 1 : 2) k_batch(const OpDesc* __restrict__ ops, const OpLevel* __restrict__ lv,
-                                              const Item* __restrict__ items, int nitems, const void* const* xs,
-                                              void* const* ys, const int64_t* lds, int* head, int* done,
-                                              const int* __restrict__ target, int* status, uint64_t limit_ns) {
+// The body's width for an item of at most w right-hand sides in one pass: calls f with it.
+template <class P, class F>
+__host__ __device__ __forceinline__ void at_width(int w, F f) {
+  using std::integral_constant;
+  if constexpr (std::is_same<P, FP32P>::value) {
+    if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 2>(), integral_constant<int, 2>());
+  } else if constexpr (std::is_same<P, FP64P>::value) {
+    if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 1>(), integral_constant<int, 2>());
+  } else {
+    if (w == 3) return f(integral_constant<int, 3>(), integral_constant<int, 1>(), integral_constant<int, 2>());
+  }
+  if (w > 2) return f(integral_constant<int, 4>(), integral_constant<int, 1>(), integral_constant<int, 2>());
+  if (w > 1) return f(integral_constant<int, 2>(), integral_constant<int, 1>(), integral_constant<int, 4>());
+  return f(integral_constant<int, 1>(), integral_constant<int, 1>(), integral_constant<int, 4>());
+}
+
+// One node at one width. Not inlined: the widths of a precision share the kernel's registers.
+template <class P, int RB, int TR, int U>
+__device__ __noinline__ void batch_node(const OpLevel& ol, const IO<typename P::vec_t>& io, int64_t j, int r, int r1,
+                                        unsigned char* smem) {
+  node::fwd_body<P, RB, TR, U, false>(ol.d, (const typename P::mat_t*)ol.mat, io, ol.max_in, ol.max_out, ol.max_rows,
+                                      ol.max_cols, ol.max_rows_pair, j, 0, 1, r, r1, smem);
+}
+
+template <class P>
+__global__ void __launch_bounds__(NTMAX, 2) k_batch(const OpDesc* __restrict__ ops, const OpLevel* __restrict__ lv,
+                                                    const Item* __restrict__ items, int nitems, const void* const* xs,
+                                                    void* const* ys, const int64_t* lds, int* head, int* done,
+                                                    const int* __restrict__ target, int* status, uint64_t limit_ns) {
   using V = typename P::vec_t;
+  using M = typename P::mat_t;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int sidx, sfail;
+  __shared__ OpLevel ol;  // the item's level and vectors
+  __shared__ IO<V> io;
+  if (threadIdx.x == 0) sidx = atomicAdd(head, 1);
   for (;;) {
-    __syncthreads();  // the previous item's shared memory and sidx are no longer in use
-    if (threadIdx.x == 0) sidx = atomicAdd(head, 1);
     __syncthreads();
     const int i = sidx;
     if (i >= nitems) break;
     const Item w = items[i];
     const OpDesc od = ops[w.op];
     const int li = od.level_base + w.level;
+    __syncthreads();  // every thread has read sidx and is past the previous item's shared memory
+    static_assert(sizeof(OpLevel) % 4 == 0, "copied in words");
+    if (threadIdx.x >= 32 && threadIdx.x < 64)
+      for (int q = threadIdx.x - 32; q < (int)(sizeof(OpLevel) / 4); q += 32) ((uint32_t*)&ol)[q] = ((const uint32_t*)(lv + li))[q];
+    if (threadIdx.x == 64) {
+      io.x = (const V*)xs[w.op];
+      io.ldx = lds[w.op];
+      io.y = (V*)ys[w.op];
+      io.ldy = lds[w.op];
+      io.R = od.R;
+      io.win = w.level > 0 ? (const V*)(w.level & 1 ? od.ws0 : od.ws1) : nullptr;
+      io.wout = w.level < od.L ? (V*)(w.level & 1 ? od.ws1 : od.ws0) : nullptr;
+    }
     if (threadIdx.x == 0) {
+      const int nxt = atomicAdd(head, 1);
+      sidx = nxt;
+      if (nxt < nitems) {  // the next item's blocks (contiguous over a run of nodes) into L2
+        const Item nw = items[nxt];
+        const OpLevel& nl = lv[ops[nw.op].level_base + nw.level];
+        const int64_t a = nl.d.moff[2 * nw.node0], e = 2 * (int64_t)(nw.node0 + nw.nodes) - 1;
+        const int64_t n = nl.d.moff[e] + (int64_t)nl.d.rows[e] * nl.d.cols[e] - a;
+        if (nw.r0 == 0 && n * (int64_t)sizeof(M) < (1 << 22)) node::prefetch_l2((const M*)nl.mat + a, n * (int64_t)sizeof(M));
+      }
       sfail = 0;
       if (w.level > 0) {
         volatile int* dp = done + (li - 1);
@@ -112,33 +168,16 @@ __global__ void __launch_bounds__(NT, TC == 8 ? 1 : 2) k_batch(const OpDesc* __r
     }
     __syncthreads();
     if (!sfail) {
-      const OpLevel ol = lv[li];
-      IO<V> io;
-      io.x = (const V*)xs[w.op];
-      io.ldx = lds[w.op];
-      io.y = (V*)ys[w.op];
-      io.ldy = lds[w.op];
-      io.R = od.R;
-      V* wb[2] = {(V*)od.ws0, (V*)od.ws1};
-      io.win = w.level > 0 ? wb[(w.level - 1) & 1] : nullptr;
-      io.wout = w.level < od.L ? wb[w.level & 1] : nullptr;
-      for (int n = 0; n < w.nodes; ++n) {
-        if (n) __syncthreads();
-        if constexpr (TC > 0) {
-          fwd_node_tiled<P, RB, TC>(ol.d, (const typename P::mat_t*)ol.mat, io, ol.max_rows, ol.max_in, ol.max_out,
-                                    (int64_t)(w.node0 + n), w.r0, smem);
-        } else if constexpr (TC < 0) {
-          if (ol.body)
-            fwd_node_tiled<P, RB, 4>(ol.d, (const typename P::mat_t*)ol.mat, io, ol.max_rows, ol.max_in, ol.max_out,
-                                     (int64_t)(w.node0 + n), w.r0, smem);
-          else
-            fwd_node<P, kMixedSmallRB, RPT>(ol.d, (const typename P::mat_t*)ol.mat, io, ol.gcap, ol.rcap, ol.max_in,
-                                            (int64_t)(w.node0 + n), w.r0, smem);
-        } else {
-          fwd_node<P, RB, RPT>(ol.d, (const typename P::mat_t*)ol.mat, io, ol.gcap, ol.rcap, ol.max_in,
-                               (int64_t)(w.node0 + n), w.r0, smem);
+      const int r1 = min(od.R, w.r0 + od.width);
+      const int passes = (r1 - w.r0 + pass_rb<P>() - 1) / pass_rb<P>(), pw = (r1 - w.r0 + passes - 1) / passes;
+      for (int n = 0; n < w.nodes; ++n)
+        for (int r = w.r0; r < r1; r += pw) {
+          if (n || r != w.r0) __syncthreads();
+          at_width<P>(pw, [&](auto rb, auto tr, auto u) {
+            batch_node<P, decltype(rb)::value, decltype(tr)::value, decltype(u)::value>(
+                ol, io, (int64_t)(w.node0 + n), r, min(r + pw, r1), smem);
+          });
         }
-      }
     }
     __threadfence();  // release: this item's outputs before its completion count
     __syncthreads();
@@ -146,17 +185,81 @@ __global__ void __launch_bounds__(NT, TC == 8 ? 1 : 2) k_batch(const OpDesc* __r
   }
 }
 
-template <class P, int RB, int RPT, int TC>
-size_t node_smem(const LevelInfo& li, bool tiled_body) {
-  const int gcap = std::max(std::max(li.max_cols, li.max_rows), li.max_in);
-  const int rcap = std::max(li.max_rows, li.max_cols);
-  if constexpr (TC > 0)
-    return tiled::smem_bytes<P, RB, TC>(li.max_in, li.max_out, li.max_rows, NT);
-  else if constexpr (TC < 0)
-    return tiled_body ? tiled::smem_bytes<P, RB, 4>(li.max_in, li.max_out, li.max_rows, NT)
-                      : fwd_node_smem<P, kMixedSmallRB, RPT>(li.max_in, gcap, rcap, NT);
-  else
-    return fwd_node_smem<P, RB, RPT>(li.max_in, gcap, rcap, NT);
+// One level of the operators of one width: a CTA per item. Everything before the body's
+// wait_for_inputs (the item, its level's description, the factors) is independent of the previous
+// level's launch.
+template <class P, int RB, int TR, int U, int NTL, int MINB>
+__global__ void __launch_bounds__(NTL, MINB)
+    k_batch_level(const LevelItem* __restrict__ items, const OpDesc* __restrict__ ops, const OpLevel* __restrict__ lv,
+                  int level, const void* const* xs, void* const* ys, const int64_t* lds) {
+  using V = typename P::vec_t;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ OpLevel ol;
+  __shared__ IO<V> io;
+  __shared__ LevelItem it;
+  node::next_may_begin();
+  if (threadIdx.x < 32) {
+    const LevelItem q = items[blockIdx.x];
+    const OpDesc od = ops[q.op];
+    const uint32_t* src = (const uint32_t*)(lv + od.level_base + level);
+    for (int w = threadIdx.x; w < (int)(sizeof(OpLevel) / 4); w += 32) ((uint32_t*)&ol)[w] = src[w];
+    if (threadIdx.x == 0) {
+      it = q;
+      io.x = (const V*)xs[q.op];
+      io.ldx = lds[q.op];
+      io.y = (V*)ys[q.op];
+      io.ldy = lds[q.op];
+      io.R = od.R;
+      io.win = level > 0 ? (const V*)(level & 1 ? od.ws0 : od.ws1) : nullptr;
+      io.wout = level < od.L ? (V*)(level & 1 ? od.ws1 : od.ws0) : nullptr;
+    }
+  }
+  __syncthreads();
+  for (int n = 0; n < it.nodes; ++n) {
+    if (n) __syncthreads();
+    node::fwd_body<P, RB, TR, U, false>(ol.d, (const typename P::mat_t*)ol.mat, io, ol.max_in, ol.max_out, ol.max_rows,
+                                        ol.max_cols, ol.max_rows_pair, (int64_t)(it.node0 + n), it.sl, it.nsl, it.r0,
+                                        min(it.r0 + RB, io.R), smem);
+  }
+}
+
+// The instances of the level launches, as the per-level kernels of node.cu: calls f with
+// (right-hand sides, rows per thread, columns in flight, threads, CTAs per SM) for items of w
+// right-hand sides.
+template <class P, class F>
+void at_level_width(int w, bool few, F f) {
+#define IDBF_W(RB, TR, U, NT, MB)                                                                              \
+  return f(std::integral_constant<int, RB>(), std::integral_constant<int, TR>(), std::integral_constant<int, U>(), \
+           std::integral_constant<int, NT>(), std::integral_constant<int, MB>())
+  if constexpr (std::is_same<P, FP32P>::value) {
+    if (w > 6 && few) IDBF_W(8, 2, 2, 256, 2);
+    if (w > 6) IDBF_W(8, 2, 4, 192, 4);
+    if (w > 4) IDBF_W(6, 1, 4, 256, 3);
+    if (w > 2) IDBF_W(4, 1, 4, 256, 3);
+    if (w > 1) IDBF_W(2, 1, 8, 256, 3);
+    IDBF_W(1, 1, 6, 256, 4);
+  } else if constexpr (std::is_same<P, FP64P>::value) {
+    if (w > 4) IDBF_W(8, 1, 2, 256, 2);
+    if (w > 2) IDBF_W(4, 1, 4, 256, 2);
+    if (w > 1) IDBF_W(2, 1, 4, 256, 2);
+    IDBF_W(1, 1, 4, 256, 3);
+  } else {
+    if (w > 3) IDBF_W(4, 1, 2, 256, 2);
+    if (w > 2) IDBF_W(3, 1, 2, 256, 2);
+    if (w > 1) IDBF_W(2, 1, 4, 256, 2);
+    IDBF_W(1, 1, 4, 256, 3);
+  }
+#undef IDBF_W
+}
+
+template <class P>
+size_t node_smem(const LevelInfo& li, int pw) {
+  size_t n = 0;
+  at_width<P>(pw, [&](auto rb, auto, auto) {
+    n = node::fwd_smem<P, decltype(rb)::value>(li.max_in, li.max_out, li.max_rows, li.max_cols, li.max_rows_pair,
+                                               li.kind == KIND_U);
+  });
+  return n;
 }
 
 }  // namespace bat
@@ -179,8 +282,7 @@ struct idbf_batch_s {
   int* d_status = nullptr;
   void** d_ptrs = nullptr;    // xs[nops], ys[nops], then lds[nops] (int64)
   int tile = 1, rb = 4, npi = 1;  // tile: index into bat::kTiles
-  int mix_rows = 64;              // mixed tiling: levels with at most this many rows per block use the per-thread body
-  std::vector<bat::OpLevel> h_lv; // host copy of the level table (the body flags change with mix_rows)
+  std::vector<bat::OpDesc> h_ops; // host copy of the operator table (the item widths change with the tile)
   size_t smem = 0;
   int ctas = 0;
   uint64_t limit_ns = 2000000000ull;
@@ -191,6 +293,17 @@ struct idbf_batch_s {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaStream_t cap = nullptr;
+  // level launches (tiles with nt = 0): every width of the batch is a chain of launches, one per
+  // level, of its own stream during the capture
+  struct LevelLaunch {
+    int width, level, first, count, nt;
+    size_t smem;
+  };
+  std::vector<LevelLaunch> level_launches;  // by width, then level
+  bat::LevelItem* d_litems = nullptr;
+  std::vector<cudaStream_t> side;           // capture streams of the second and later widths
+  cudaEvent_t ev_fork = nullptr;
+  std::vector<cudaEvent_t> ev_join;
 };
 
 namespace {
@@ -201,6 +314,9 @@ void free_layout(idbf_batch_s* b) {
   b->exec = nullptr;
   b->graph = nullptr;
   if (b->d_items) cudaFree(b->d_items);
+  if (b->d_litems) cudaFree(b->d_litems);
+  b->d_litems = nullptr;
+  b->level_launches.clear();
   if (b->d_target) cudaFree(b->d_target);
   if (b->d_counters) cudaFree(b->d_counters);
   b->d_items = nullptr;
@@ -208,86 +324,150 @@ void free_layout(idbf_batch_s* b) {
   b->d_counters = nullptr;
 }
 
-template <class P, int T>
-idbf_status launch_batch(idbf_batch_s* b, cudaStream_t st) {
-  constexpr int RB = bat::kTiles[T].rb, RPT = bat::kTiles[T].rpt, TC = bat::kTiles[T].tc;
-  if constexpr (!bat::instantiated<P, T>()) {
-    return IDBF_EUNSUPPORTED;
-  } else {
-    if (b->smem > 48 * 1024)
-      IDBF_CUDA_TRY(cudaFuncSetAttribute(bat::k_batch<P, RB, RPT, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)b->smem));
-    const void* const* xs = (const void* const*)b->d_ptrs;
-    void* const* ys = (void* const*)(b->d_ptrs + b->nops);
-    const int64_t* lds = (const int64_t*)(b->d_ptrs + 2 * b->nops);
-    IDBF_CUDA_TRY(cudaMemsetAsync(b->d_counters, 0, sizeof(int) * (1 + b->nlevels_total), st));
-    bat::k_batch<P, RB, RPT, TC><<<b->ctas, bat::NT, b->smem, st>>>(b->d_ops, b->d_lv, b->d_items, b->nitems, xs, ys, lds,
-                                                                 b->d_counters, b->d_counters + 1, b->d_target,
-                                                                 b->d_status, b->limit_ns);
-    IDBF_CUDA_TRY(cudaGetLastError());
-    return IDBF_OK;
-  }
-}
+// The fault injection of idbf_batch_debug_set_wait needs the persistent launch's waits: while it is
+// set, tiles of level launches run as a persistent one.
+bool level_launched(const idbf_batch_s* b) { return bat::kTiles[b->tile].nt == 0 && b->debug_extra == 0; }
+int persistent_threads(const idbf_batch_s* b) { return bat::kTiles[b->tile].nt ? bat::kTiles[b->tile].nt : bat::NTMAX; }
 
-// shared memory per CTA: the largest node of any level of any operator (0 if the tile is not
-// instantiated for this precision)
-template <class P, int T>
-size_t smem_for(idbf_batch_s* b) {
-  constexpr int RB = bat::kTiles[T].rb, RPT = bat::kTiles[T].rpt, TC = bat::kTiles[T].tc;
-  if constexpr (!bat::instantiated<P, T>()) {
-    return 0;
-  } else {
-    size_t sm = 0;
-    for (int o = 0; o < b->nops; ++o) {
-      if (b->sep[o]) continue;
-      for (const LevelInfo& li : b->plans[o]->p.lv)
-        sm = std::max(sm, bat::node_smem<P, RB, RPT, TC>(li, li.max_rows > b->mix_rows));
+// The launches of every width and level and their items, for the current tile.
+template <class P>
+idbf_status plan_levels(idbf_batch_s* b, std::vector<bat::LevelItem>& items) {
+  const int cap = std::min(b->rb, bat::pass_rb<P>());
+  std::vector<int> widths;  // instance widths in use
+  std::vector<int> cls(b->nops, 0);
+  int maxL = 0;
+  for (int o = 0; o < b->nops; ++o) {
+    if (b->sep[o]) continue;
+    int w = 0;
+    bat::at_level_width<P>(node::even_block(b->R[o], cap), b->rb > 8, [&](auto rb, auto, auto, auto, auto) { w = decltype(rb)::value; });
+    cls[o] = w;
+    if (std::find(widths.begin(), widths.end(), w) == widths.end()) widths.push_back(w);
+    maxL = std::max(maxL, b->plans[o]->p.L);
+  }
+  std::sort(widths.begin(), widths.end(), [](int x, int y) { return x > y; });
+  // few nodes on a level over the whole batch: cut them as the single apply does
+  std::vector<int64_t> nodes(maxL + 1, 0);
+  for (int o = 0; o < b->nops; ++o)
+    for (int l = 0; !b->sep[o] && l <= b->plans[o]->p.L; ++l)
+      nodes[l] += (int64_t)b->plans[o]->p.m * ((b->R[o] + cls[o] - 1) / cls[o]);
+  for (const int w : widths)
+    for (int l = 0; l <= maxL; ++l) {
+      idbf_batch_s::LevelLaunch q{w, l, (int)items.size(), 0, 0, 0};
+      for (int o = 0; o < b->nops; ++o) {
+        const Plan& p = b->plans[o]->p;
+        if (b->sep[o] || cls[o] != w || l > p.L) continue;
+        const LevelInfo& li = p.lv[l];
+        const int nsl = node::slices(nodes[l], node::fwd_span(li), 4);
+        bat::at_level_width<P>(w, b->rb > 8, [&](auto rb, auto tr, auto, auto ntl, auto) {
+          q.smem = std::max(q.smem, node::fwd_smem<P, decltype(rb)::value>(li.max_in, li.max_out, li.max_rows, li.max_cols,
+                                                                            li.max_rows_pair, li.kind == KIND_U));
+          q.nt = std::max(q.nt, node::fwd_threads(li, decltype(tr)::value, nsl, decltype(ntl)::value));
+        });
+        // the right-hand-side blocks of a slice are adjacent, so that their reads meet in L2
+        const int npi = nsl > 1 ? 1 : b->npi;
+        for (int n0 = 0; n0 < p.m; n0 += npi)
+          for (int sl = 0; sl < nsl; ++sl)
+            for (int64_t r0 = 0; r0 < b->R[o]; r0 += w)
+              items.push_back({o, n0, std::min(npi, p.m - n0), (int)r0, sl, nsl});
+      }
+      q.count = (int)items.size() - q.first;
+      if (q.smem > 200 * 1024) return IDBF_EUNSUPPORTED;
+      if (q.count > 0) b->level_launches.push_back(q);
     }
-    return sm;
-  }
+  return IDBF_OK;
 }
 
-template <class P, int T>
+template <class P>
+idbf_status launch_levels(idbf_batch_s* b, cudaStream_t st) {
+  const void* const* xs = (const void* const*)b->d_ptrs;
+  void* const* ys = (void* const*)(b->d_ptrs + b->nops);
+  const int64_t* lds = (const int64_t*)(b->d_ptrs + 2 * b->nops);
+  IDBF_CUDA_TRY(cudaEventRecord(b->ev_fork, st));
+  int chain = -1, width = 0;
+  cudaStream_t cs = st;
+  auto join = [&]() -> cudaError_t {  // the chain that just ended rejoins the main stream
+    if (chain <= 0) return cudaSuccess;
+    const cudaError_t e = cudaEventRecord(b->ev_join[chain - 1], cs);
+    return e != cudaSuccess ? e : cudaStreamWaitEvent(st, b->ev_join[chain - 1], 0);
+  };
+  for (size_t k = 0; k < b->level_launches.size(); ++k) {
+    const auto& q = b->level_launches[k];
+    const bool first = q.width != width;
+    if (first) {
+      if (++chain > 0) {
+        if ((int)b->side.size() < chain) {
+          cudaStream_t s = nullptr;
+          cudaEvent_t ev = nullptr;
+          IDBF_CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+          b->side.push_back(s);
+          IDBF_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+          b->ev_join.push_back(ev);
+        }
+        cs = b->side[chain - 1];
+        IDBF_CUDA_TRY(cudaStreamWaitEvent(cs, b->ev_fork, 0));
+      }
+      width = q.width;
+    }
+    cudaError_t e = cudaSuccess;
+    bat::at_level_width<P>(q.width, b->rb > 8, [&](auto rb, auto tr, auto u, auto ntl, auto mb) {
+      auto kern = bat::k_batch_level<P, decltype(rb)::value, decltype(tr)::value, decltype(u)::value, decltype(ntl)::value,
+                                     decltype(mb)::value>;
+      if (q.smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if (e == cudaSuccess)
+        e = node::launch_after(kern, !first, (int64_t)q.count, q.nt, q.smem, cs, (const bat::LevelItem*)b->d_litems + q.first,
+                               (const bat::OpDesc*)b->d_ops, (const bat::OpLevel*)b->d_lv, q.level, xs, ys, lds);
+    });
+    IDBF_CUDA_TRY(e);
+    const bool last = k + 1 == b->level_launches.size() || b->level_launches[k + 1].width != width;
+    if (last) IDBF_CUDA_TRY(join());
+  }
+  return IDBF_OK;
+}
+
+template <class P>
+idbf_status launch_batch(idbf_batch_s* b, cudaStream_t st) {
+  if (b->smem > 48 * 1024)
+    IDBF_CUDA_TRY(cudaFuncSetAttribute(bat::k_batch<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
+  const void* const* xs = (const void* const*)b->d_ptrs;
+  void* const* ys = (void* const*)(b->d_ptrs + b->nops);
+  const int64_t* lds = (const int64_t*)(b->d_ptrs + 2 * b->nops);
+  IDBF_CUDA_TRY(cudaMemsetAsync(b->d_counters, 0, sizeof(int) * (1 + b->nlevels_total), st));
+  bat::k_batch<P><<<b->ctas, persistent_threads(b), b->smem, st>>>(b->d_ops, b->d_lv, b->d_items, b->nitems, xs, ys, lds,
+                                                                    b->d_counters, b->d_counters + 1, b->d_target,
+                                                                    b->d_status, b->limit_ns);
+  IDBF_CUDA_TRY(cudaGetLastError());
+  return IDBF_OK;
+}
+
+// shared memory per CTA: the largest node of any level of any operator
+template <class P>
+size_t smem_for(idbf_batch_s* b) {
+  size_t sm = 0;
+  for (int o = 0; o < b->nops; ++o) {
+    if (b->sep[o]) continue;
+    const int w = b->h_ops[o].width, passes = (w + bat::pass_rb<P>() - 1) / bat::pass_rb<P>();
+    for (const LevelInfo& li : b->plans[o]->p.lv) sm = std::max(sm, bat::node_smem<P>(li, (w + passes - 1) / passes));
+  }
+  return sm;
+}
+
+template <class P>
 int occupancy(idbf_batch_s* b) {
-  constexpr int RB = bat::kTiles[T].rb, RPT = bat::kTiles[T].rpt, TC = bat::kTiles[T].tc;
-  if constexpr (!bat::instantiated<P, T>()) {
-    return 1;
-  } else {
-    int n = 0;
-    if (b->smem > 48 * 1024)
-      cudaFuncSetAttribute(bat::k_batch<P, RB, RPT, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bat::k_batch<P, RB, RPT, TC>, bat::NT, b->smem);
-    return std::max(n, 1);
-  }
+  int n = 0;
+  if (b->smem > 48 * 1024)
+    cudaFuncSetAttribute(bat::k_batch<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bat::k_batch<P>, persistent_threads(b), b->smem);
+  return std::max(n, 1);
 }
 
-// calls F<P, tile>::run(b, args...) for the batch's precision and current tile
-#define IDBF_BATCH_DISPATCH(FN, RET_ON_BAD, ...)                                               \
-  [&]() {                                                                                      \
-    switch (b->mode) {                                                                         \
-      case IDBF_MODE_FP64: switch (b->tile) {                                                  \
-          case 0: return FN<FP64P, 0>(__VA_ARGS__); case 1: return FN<FP64P, 1>(__VA_ARGS__);  \
-          case 2: return FN<FP64P, 2>(__VA_ARGS__); case 3: return FN<FP64P, 3>(__VA_ARGS__);  \
-          case 4: return FN<FP64P, 4>(__VA_ARGS__); case 5: return FN<FP64P, 5>(__VA_ARGS__);  \
-          case 6: return FN<FP64P, 6>(__VA_ARGS__); case 7: return FN<FP64P, 7>(__VA_ARGS__);  \
-          default: return RET_ON_BAD; }                                                        \
-      case IDBF_MODE_DF64: switch (b->tile) {                                                  \
-          case 0: return FN<DF64P, 0>(__VA_ARGS__); case 1: return FN<DF64P, 1>(__VA_ARGS__);  \
-          case 2: return FN<DF64P, 2>(__VA_ARGS__); case 3: return FN<DF64P, 3>(__VA_ARGS__);  \
-          case 4: return FN<DF64P, 4>(__VA_ARGS__); case 5: return FN<DF64P, 5>(__VA_ARGS__);  \
-          case 6: return FN<DF64P, 6>(__VA_ARGS__); case 7: return FN<DF64P, 7>(__VA_ARGS__);  \
-          default: return RET_ON_BAD; }                                                        \
-      default: switch (b->tile) {                                                              \
-          case 0: return FN<FP32P, 0>(__VA_ARGS__); case 1: return FN<FP32P, 1>(__VA_ARGS__);  \
-          case 2: return FN<FP32P, 2>(__VA_ARGS__); case 3: return FN<FP32P, 3>(__VA_ARGS__);  \
-          case 4: return FN<FP32P, 4>(__VA_ARGS__); case 5: return FN<FP32P, 5>(__VA_ARGS__);  \
-          case 6: return FN<FP32P, 6>(__VA_ARGS__); case 7: return FN<FP32P, 7>(__VA_ARGS__);  \
-          default: return RET_ON_BAD; }                                                        \
-    }                                                                                          \
-  }()
+// calls FN<P>(args...) for the batch's arithmetic
+#define IDBF_BATCH_DISPATCH(FN, ...)                            \
+  (b->mode == IDBF_MODE_FP64   ? FN<FP64P>(__VA_ARGS__)         \
+   : b->mode == IDBF_MODE_DF64 ? FN<DF64P>(__VA_ARGS__)         \
+                               : FN<FP32P>(__VA_ARGS__))
 
 idbf_status launch(idbf_batch_s* b, cudaStream_t st) {
-  return IDBF_BATCH_DISPATCH(launch_batch, IDBF_EINVAL, b, st);
+  return level_launched(b) ? IDBF_BATCH_DISPATCH(launch_levels, b, st) : IDBF_BATCH_DISPATCH(launch_batch, b, st);
 }
 
 bool tile_valid(int mode, int tile) {
@@ -295,9 +475,22 @@ bool tile_valid(int mode, int tile) {
   const bat::Tile t = bat::kTiles[tile];
   switch (mode) {
     case IDBF_MODE_FP64: return t.rb <= bat::max_rb<FP64P>();
-    case IDBF_MODE_DF64: return t.rb <= bat::max_rb<DF64P>() && t.tc == 0;
+    case IDBF_MODE_DF64: return t.rb <= bat::max_rb<DF64P>() && !t.wide;
     default: return t.rb <= bat::max_rb<FP32P>();
   }
+}
+
+// The launches of one batch apply as a graph.
+idbf_status capture(idbf_batch_s* b) {
+  IDBF_CUDA_TRY(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
+  idbf_status s = launch(b, b->cap);
+  cudaGraph_t g = nullptr;
+  const cudaError_t e = cudaStreamEndCapture(b->cap, &g);
+  if (s != IDBF_OK) { if (g) cudaGraphDestroy(g); return s; }
+  if (e != cudaSuccess) { set_cuda_error(e); return IDBF_ECUDA; }
+  b->graph = g;
+  IDBF_CUDA_TRY(cudaGraphInstantiate(&b->exec, g, 0));
+  return IDBF_OK;
 }
 
 // Queue of items, completion targets and the captured graph for the current (rb, npi).
@@ -305,13 +498,22 @@ idbf_status layout(idbf_batch_s* b) {
   free_layout(b);
   if (!tile_valid(b->mode, b->tile)) return IDBF_EUNSUPPORTED;
   b->rb = bat::kTiles[b->tile].rb;
-  const bool mixed = bat::kTiles[b->tile].tc < 0;
   b->sep.assign(b->nops, 0);
   for (int o = 0; o < b->nops; ++o) b->sep[o] = b->plans[o]->p.N >= b->split_n ? 1 : 0;
-  // level bodies of the mixed tiling (ignored by the others)
-  for (int o = 0, li = 0; o < b->nops; ++o)
-    for (const LevelInfo& lvi : b->plans[o]->p.lv) b->h_lv[li++].body = lvi.max_rows > b->mix_rows ? 1 : 0;
-  IDBF_CUDA_TRY(cudaMemcpy(b->d_lv, b->h_lv.data(), sizeof(bat::OpLevel) * b->h_lv.size(), cudaMemcpyHostToDevice));
+  for (int o = 0; o < b->nops; ++o) b->h_ops[o].width = node::even_block(b->R[o], b->rb);
+  IDBF_CUDA_TRY(cudaMemcpy(b->d_ops, b->h_ops.data(), sizeof(bat::OpDesc) * b->nops, cudaMemcpyHostToDevice));
+  if (level_launched(b)) {
+    std::vector<bat::LevelItem> li;
+    const idbf_status s = IDBF_BATCH_DISPATCH(plan_levels, b, li);
+    if (s != IDBF_OK) return s;
+    b->nitems = (int)li.size();
+    b->smem = 0;
+    b->ctas = b->nitems;
+    if (b->nitems == 0) return IDBF_OK;
+    IDBF_CUDA_TRY(cudaMalloc((void**)&b->d_litems, sizeof(bat::LevelItem) * li.size()));
+    IDBF_CUDA_TRY(cudaMemcpy(b->d_litems, li.data(), sizeof(bat::LevelItem) * li.size(), cudaMemcpyHostToDevice));
+    return capture(b);
+  }
   std::vector<bat::Item> items;
   std::vector<int> target(b->nlevels_total, 0);
   int maxL = 0, base = 0;
@@ -327,7 +529,7 @@ idbf_status layout(idbf_batch_s* b) {
       if (l > p.L || b->sep[o]) continue;
       // the right-hand-side blocks of a run of nodes are neighbours in the queue, so the
       // blocks' second and later reads of the factors come from L2
-      const int rbl = mixed && !b->h_lv[lbase[o] + l].body ? bat::kMixedSmallRB : b->rb;
+      const int rbl = b->h_ops[o].width;
       for (int n0 = 0; n0 < p.m; n0 += b->npi)
         for (int r0 = 0; r0 < b->R[o]; r0 += rbl) {
           bat::Item it;
@@ -349,9 +551,9 @@ idbf_status layout(idbf_batch_s* b) {
     b->ctas = 0;
     return IDBF_OK;
   }
-  b->smem = IDBF_BATCH_DISPATCH(smem_for, (size_t)0, b);
+  b->smem = IDBF_BATCH_DISPATCH(smem_for, b);
   if (b->smem == 0 || b->smem > 200 * 1024) return IDBF_EUNSUPPORTED;
-  const int occ = IDBF_BATCH_DISPATCH(occupancy, 1, b);
+  const int occ = IDBF_BATCH_DISPATCH(occupancy, b);
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
   b->ctas = std::max(1, std::min(occ * sms, b->nitems));
@@ -360,16 +562,7 @@ idbf_status layout(idbf_batch_s* b) {
   IDBF_CUDA_TRY(cudaMalloc((void**)&b->d_counters, sizeof(int) * (1 + b->nlevels_total)));
   IDBF_CUDA_TRY(cudaMemcpy(b->d_items, items.data(), sizeof(bat::Item) * b->nitems, cudaMemcpyHostToDevice));
   IDBF_CUDA_TRY(cudaMemcpy(b->d_target, target.data(), sizeof(int) * b->nlevels_total, cudaMemcpyHostToDevice));
-  // capture: reset the counters, run the persistent kernel
-  IDBF_CUDA_TRY(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-  idbf_status s = launch(b, b->cap);
-  cudaGraph_t g = nullptr;
-  const cudaError_t e = cudaStreamEndCapture(b->cap, &g);
-  if (s != IDBF_OK) { if (g) cudaGraphDestroy(g); return s; }
-  if (e != cudaSuccess) { set_cuda_error(e); return IDBF_ECUDA; }
-  b->graph = g;
-  IDBF_CUDA_TRY(cudaGraphInstantiate(&b->exec, g, 0));
-  return IDBF_OK;
+  return capture(b);
 }
 
 }  // namespace
@@ -409,7 +602,7 @@ idbf_status idbf_batch_create(const idbf_plan* plans, int32_t nops, const int64_
     ods[o].L = p.L;
     ods[o].R = (int)nrhs[o];
     ods[o].level_base = (int)lvs.size();
-    ods[o].pad = 0;
+    ods[o].width = 1;
     ods[o].ws0 = w;
     ods[o].ws1 = (char*)w + half;
     for (int l = 0; l <= p.L; ++l) {
@@ -417,12 +610,12 @@ idbf_status idbf_batch_create(const idbf_plan* plans, int32_t nops, const int64_
       bat::OpLevel ol;
       ol.d = p.level(l);
       ol.mat = p.lmat[fmt][l];
-      ol.gcap = std::max(std::max(li.max_cols, li.max_rows), li.max_in);
-      ol.rcap = std::max(li.max_rows, li.max_cols);
       ol.max_in = li.max_in;
       ol.max_out = li.max_out;
       ol.max_rows = li.max_rows;
-      ol.body = 1;
+      ol.max_cols = li.max_cols;
+      ol.max_rows_pair = li.max_rows_pair;
+      ol.pad = 0;
       lvs.push_back(ol);
     }
   }
@@ -432,11 +625,11 @@ idbf_status idbf_batch_create(const idbf_plan* plans, int32_t nops, const int64_
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_lv, sizeof(bat::OpLevel) * lvs.size());
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_ptrs, sizeof(void*) * 3 * nops);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_status, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_ops, ods.data(), sizeof(bat::OpDesc) * nops, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_lv, lvs.data(), sizeof(bat::OpLevel) * lvs.size(), cudaMemcpyHostToDevice);
-    b->h_lv = lvs;
+    b->h_ops = ods;
     if (e == cudaSuccess) e = cudaMemset(b->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
     if (e != cudaSuccess) { set_cuda_error(e); s = e == cudaErrorMemoryAllocation ? IDBF_ENOMEM : IDBF_ECUDA; }
   }
   if (s == IDBF_OK) {
@@ -493,7 +686,7 @@ idbf_status idbf_batch_autotune(idbf_batch b, const void* const* x, void* const*
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   float best = 1e30f;
-  int btile = b->tile, bnpi = b->npi, bmix = b->mix_rows;
+  int btile = b->tile, bnpi = b->npi;
   int64_t bsplit = b->split_n;
   idbf_status s = IDBF_OK;
   // time the current layout (a warm-up launch, then reps launches); EUNSUPPORTED layouts are skipped
@@ -513,23 +706,17 @@ idbf_status idbf_batch_autotune(idbf_batch b, const void* const* x, void* const*
       best = ms;
       btile = b->tile;
       bnpi = b->npi;
-      bmix = b->mix_rows;
       bsplit = b->split_n;
     }
   };
   // every tiling at the current split
   auto tilings = [&]() {
     const int npis[3] = {1, 2, 4};
-    const int mixes[5] = {32, 64, 96, 128, 192};  // mixed tiling: row threshold of the per-thread body
-    const int mix0 = bmix;
     for (int a = 0; a < bat::kNumTiles && s == IDBF_OK; ++a)
-      for (int c = 0; c < 3 * 5 && s == IDBF_OK; ++c) {
+      for (int c = 0; c < 3 && s == IDBF_OK; ++c) {
         if (!tile_valid(b->mode, a)) continue;
-        const bool mixed = bat::kTiles[a].tc < 0;
-        if (!mixed && c >= 3) continue;
         b->tile = a;
-        b->npi = npis[c % 3];
-        b->mix_rows = mixed ? mixes[c / 3] : mix0;
+        b->npi = npis[c];
         trial();
       }
   };
@@ -551,7 +738,6 @@ idbf_status idbf_batch_autotune(idbf_batch b, const void* const* x, void* const*
       if (s != IDBF_OK) break;
       b->tile = btile;
       b->npi = bnpi;
-      b->mix_rows = bmix;
       b->split_n = c;
       trial();
     }
@@ -564,7 +750,6 @@ idbf_status idbf_batch_autotune(idbf_batch b, const void* const* x, void* const*
   cudaEventDestroy(e1);
   b->tile = btile;
   b->npi = bnpi;
-  b->mix_rows = bmix;
   b->split_n = bsplit;
   if (s == IDBF_OK) s = layout(b);
   if (best_ms) *best_ms = best;
@@ -668,6 +853,9 @@ void idbf_batch_destroy(idbf_batch b) {
   if (b->d_ptrs) cudaFree(b->d_ptrs);
   if (b->d_status) cudaFree(b->d_status);
   if (b->cap) cudaStreamDestroy(b->cap);
+  for (cudaStream_t q : b->side) cudaStreamDestroy(q);
+  for (cudaEvent_t q : b->ev_join) cudaEventDestroy(q);
+  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   if (cur != b->device) cudaSetDevice(cur);
   delete b;
 }

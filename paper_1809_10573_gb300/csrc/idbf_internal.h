@@ -54,6 +54,7 @@ struct LevelInfo {
   int max_out = 0;       // max summed output length of a node
   int max_rows_pair = 0; // max rows_0 + rows_1 of a node
   int max_cols_pair = 0; // max cols_0 + cols_1 of a node
+  int64_t sum_rows = 0, sum_cols = 0;  // over all blocks of the level
   int kmin = 0, kmax = 0;  // output segment lengths
 };
 
@@ -139,6 +140,9 @@ struct LevelIO {
   const void* win;
   void* wout;
   int R;
+  // the stream's previous launch is a level kernel that lets its successor begin early (it has
+  // passed its own wait before this launch's can return, so the boundary it read is free)
+  bool after;
 };
 // level l with the node kernels (node.cu), R right-hand sides
 idbf_status node_fwd(Plan* p, Arith a, int l, const LevelIO& io, cudaStream_t st);

@@ -29,28 +29,136 @@ __host__ __device__ constexpr int op_pitch() {
   return (RB * sizeof(G)) % 64 == 0 && RB > 1 ? RB + (int)(16 / sizeof(G)) : RB;
 }
 
-// RB operands of one element
-template <class P, int RB>
-__device__ __forceinline__ void load_ops(const typename P::gv_t* p, typename P::gv_t (&g)[RB]) {
-  if constexpr (sizeof(typename P::gv_t) == 8 && RB % 2 == 0) {
+// The RB operands of one element and the sums they enter. In general operand rb is element rb of the
+// row and a sum is the policy's accumulator; complex64 with an even RB packs the right-hand sides in
+// pairs, a row holding (re, re, im, im) per pair and a sum being two f32x2: each complex
+// multiply-add of a pair is four packed FMAs, in the order of FP32P::mac on either lane, and the
+// pairs' real and imaginary parts come out of one 16-byte load as packed registers.
+template <class P, int RB, bool PACKED = std::is_same<P, FP32P>::value && RB % 2 == 0>
+struct Sums {
+  using G = typename P::gv_t;
+  using M = typename P::mat_t;
+  struct ops_t { G g[RB]; };
+  typename P::acc_t a[RB];
+  __device__ static __forceinline__ void put(G* row, int rb, const G& v) { row[rb] = v; }
+  __device__ static __forceinline__ G get(const G* row, int rb) { return row[rb]; }
+  __device__ static __forceinline__ void load(ops_t& o, const G* row) {
 #pragma unroll
-    for (int i = 0; i < RB; i += 2) {
-      const float4 v = *reinterpret_cast<const float4*>(p + i);
-      g[i] = make_float2(v.x, v.y);
-      g[i + 1] = make_float2(v.z, v.w);
+    for (int i = 0; i < RB; ++i) o.g[i] = row[i];
+  }
+  __device__ __forceinline__ void init() {
+#pragma unroll
+    for (int i = 0; i < RB; ++i) P::init(a[i]);
+  }
+  __device__ __forceinline__ void mac(const M& m, const ops_t& o) {
+#pragma unroll
+    for (int i = 0; i < RB; ++i) P::mac(a[i], m, o.g[i]);
+  }
+  __device__ __forceinline__ void macc(const M& m, const ops_t& o) {  // conj(m)
+#pragma unroll
+    for (int i = 0; i < RB; ++i) P::macc(a[i], m, o.g[i]);
+  }
+  __device__ __forceinline__ void flush() {
+#pragma unroll
+    for (int i = 0; i < RB; ++i) P::flush(a[i]);
+  }
+  __device__ __forceinline__ void parts(typename P::part_t (&pr)[RB]) {
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      P::flush(a[i]);
+      pr[i] = P::part(a[i]);
     }
-  } else {
+  }
+};
+template <class P, int RB>
+struct Sums<P, RB, true> {
+  using G = float2;
+  struct ops_t { ulonglong2 g[RB / 2]; };
+  f32x2 re[RB / 2], im[RB / 2];
+  __device__ static __forceinline__ void put(G* row, int rb, const G& v) {
+    float* f = (float*)row + (rb >> 1) * 4 + (rb & 1);
+    f[0] = v.x;
+    f[2] = v.y;
+  }
+  __device__ static __forceinline__ G get(const G* row, int rb) {
+    const float* f = (const float*)row + (rb >> 1) * 4 + (rb & 1);
+    return make_float2(f[0], f[2]);
+  }
+  __device__ static __forceinline__ void load(ops_t& o, const G* row) {
 #pragma unroll
-    for (int i = 0; i < RB; ++i) g[i] = p[i];
+    for (int i = 0; i < RB / 2; ++i) o.g[i] = ((const ulonglong2*)row)[i];
+  }
+  __device__ __forceinline__ void init() {
+#pragma unroll
+    for (int i = 0; i < RB / 2; ++i) re[i] = im[i] = 0ull;
+  }
+  __device__ __forceinline__ void mac(const float2& m, const ops_t& o) {
+    const f32x2 mx = pk2(m.x, m.x), my = pk2(m.y, m.y), ny = pk2(-m.y, -m.y);
+#pragma unroll
+    for (int i = 0; i < RB / 2; ++i) {
+      re[i] = fma2(mx, o.g[i].x, re[i]);
+      im[i] = fma2(mx, o.g[i].y, im[i]);
+      re[i] = fma2(ny, o.g[i].y, re[i]);
+      im[i] = fma2(my, o.g[i].x, im[i]);
+    }
+  }
+  __device__ __forceinline__ void macc(const float2& m, const ops_t& o) { mac(make_float2(m.x, -m.y), o); }
+  __device__ __forceinline__ void flush() {}
+  __device__ __forceinline__ void parts(float2 (&pr)[RB]) {
+#pragma unroll
+    for (int i = 0; i < RB / 2; ++i) {
+      const float2 r = upk2(re[i]), m = upk2(im[i]);
+      pr[2 * i] = make_float2(r.x, m.x);
+      pr[2 * i + 1] = make_float2(r.y, m.y);
+    }
+  }
+};
+
+// Asks for `bytes` at p (rounded out to 16-byte granules, which the arenas' tails allow) in L2: one
+// instruction streams a whole block from HBM while the CTA is still loading its index lists and
+// inputs, so that the product loop's loads meet L2 latency instead of HBM latency.
+__device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
+  const uintptr_t a = (uintptr_t)p & ~(uintptr_t)15;
+  const uint32_t n = (uint32_t)((((uintptr_t)p + bytes + 15) & ~(uintptr_t)15) - a);
+  if (bytes > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(n) : "memory");
+}
+// A level's launch may begin while the previous level still runs (launch_after in node.cu): what
+// comes before wait_for_inputs reads the factors only. next_may_begin lets the following launch
+// begin once every CTA of this one has started.
+__device__ __forceinline__ void wait_for_inputs() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void next_may_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// the share of slice sl of nsl of both blocks of a node, by two threads of the CTA
+template <class M>
+__device__ __forceinline__ void prefetch_blocks(const M* mat, const int64_t (&mov)[2], const int (&rows)[2],
+                                                const int (&cols)[2], int sl, int nsl) {
+  if (threadIdx.x < 2) {
+    const int c = threadIdx.x;
+    const int64_t n = (int64_t)(c ? rows[1] : rows[0]) * (c ? cols[1] : cols[0]);
+    const int64_t a = n * sl / nsl, b = n * (sl + 1) / nsl;
+    prefetch_l2(mat + (c ? mov[1] : mov[0]) + a, (b - a) * (int64_t)sizeof(M));
   }
 }
 
-// sum of the accumulators of lanes that differ in the lane bits below `n` (a power of two); every
-// one of those lanes gets the sum
-template <class P>
-__device__ __forceinline__ void lane_sum(typename P::acc_t& a, int n) {
-  P::flush(a);
-  for (int o = 1; o < n; o <<= 1) P::shfl_add(a, o);
+// Sums the partial sums pr[0 .. RB-1] of the S (1, 2, 4 or 8) neighbouring lanes of a group: lane s
+// ends with the sums of the right-hand sides rb = s mod S, in slots rb & ~(S-1). Each step trades
+// half of what is left with the lane one bit away, so S lanes exchange RB (1 - 1/S) values each
+// instead of RB log2 S (shuffles run at a quarter of the FMA rate). Where a slot has no partner
+// (RB odd, or fewer right-hand sides than lanes) both lanes keep the sum.
+template <class P, int RB>
+__device__ __forceinline__ void lane_sum(typename P::part_t (&pr)[RB], int S, int s) {
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    if (o >= S) break;
+    const bool up = s & o;
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      if (i & (2 * o - 1)) continue;
+      const int q = i + o;
+      if (q < RB) pr[i] = P::add_lane(up ? pr[q < RB ? q : 0] : pr[i], up ? pr[i] : pr[q < RB ? q : 0], o);
+      else pr[i] = P::add_lane(pr[i], pr[i], o);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -77,14 +185,15 @@ template <class P, int RB, int TR, int U, bool STREAM>
 __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::mat_t* __restrict__ mat,
                                          const IO<typename P::vec_t>& io, int max_in, int max_out, int max_rows,
                                          int max_cols, int max_rows_pair, int64_t j, int sl, int nsl, int r0,
-                                         unsigned char* smem) {
+                                         int r1, unsigned char* smem) {
   using G = typename P::gv_t;
   using M = typename P::mat_t;
   using BP = BndOf<P>;
   using B = typename BP::b_t;
+  using SM = Sums<P, RB>;
   constexpr int PITCH = op_pitch<P, RB>();
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-  const int nrb = min(RB, io.R - r0);
+  const int nrb = min(RB, r1 - r0);  // right-hand sides r0 .. r1-1
   const bool ulev = d.kind == KIND_U;
   G* opd = (G*)smem;
   B* res = (B*)(smem + (((size_t)max_in * PITCH * sizeof(G) + 15) & ~(size_t)15));
@@ -96,6 +205,7 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
   const int rowsv[2] = {d.rows[2 * j], d.rows[2 * j + 1]};
   const int colsv[2] = {d.cols[2 * j], d.cols[2 * j + 1]};
   const int64_t mov[2] = {d.moff[2 * j], d.moff[2 * j + 1]};
+  if (!STREAM && r0 == 0) prefetch_blocks(mat, mov, rowsv, colsv, sl, nsl);
   int l0, l1;
   int64_t i0 = 0, i1 = 0;
   if (d.lev == 0) {
@@ -158,30 +268,14 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
       for (int k = tid; k < colsv[c]; k += nt) kix[c * max_cols + k] = ((c ? l0 : 0) + k) * PITCH;
     }
   }
-  // ---- inputs -> operands
-  if (d.lev == 0) {
-    for (int i = tid; i < l0 * RB; i += nt) {
-      const int rb = i / l0, e = i - rb * l0;
-      opd[e * PITCH + rb] = P::cvt(rb < nrb ? io.x[i0 + e + (int64_t)(r0 + rb) * io.ldx] : P::zero());
-    }
-  } else {
-    const B* winb = (const B*)io.win;
-    for (int i = tid; i < (l0 + l1) * RB; i += nt) {
-      const int e = i / RB, rb = i - e * RB;
-      const int64_t off = e < l0 ? i0 + e : i1 + (e - l0);
-      opd[e * PITCH + rb] = BP::g_of(rb < nrb ? winb[off * io.R + r0 + rb] : BP::zero());
-    }
-  }
-  __syncthreads();
   if (ulev) {
+    __syncthreads();
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       ra[c] = nsl > 1 ? s_ra[c] : 0;
       rn[c] = (nsl > 1 ? s_rb[c] : rowsv[c]) - ra[c];
     }
   }
-
-  // ---- block products
   const int nt0 = (rn[0] + TR - 1) / TR, T = nt0 + (rn[1] + TR - 1) / TR;
   const int maxc = max(colsv[0], colsv[1]);
   int S = 1;
@@ -191,86 +285,108 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
     obv[0] = d.out_off[out_seg_id(d, j, 0)];
     obv[1] = d.out_off[out_seg_id(d, j, 1)];
   }
-  B* woutb = (B*)io.wout;
-  for (int w = tid; w - lane < T * S; w += nt) {
+
+  // ---- this thread's row tile and its first columns
+  const int s = tid & (S - 1);
+  int c, rt, ntc, cols, rbeg, rcnt, step, off;
+  const M* Mc;
+  int roff[TR];
+  M mv[U][TR];
+  auto load = [&](int u, M (&m)[TR]) {
+#pragma unroll
+    for (int i = 0; i < TR; ++i) {
+      const M* q = Mc + (off + u * step + roff[i]);
+      m[i] = STREAM ? __ldcs(q) : __ldg(q);
+    }
+  };
+  auto begin = [&](int w) {  // tile w / S (none past the last: no columns); the entries of its first U columns
     const bool active = w < T * S;
-    const int tile = active ? w / S : 0, s = w & (S - 1);
-    const int c = tile >= nt0;
-    const int rt = tile - (c ? nt0 : 0);
-    const int ntc = c ? T - nt0 : nt0;
+    const int tile = active ? w / S : 0;
+    c = tile >= nt0;
+    rt = tile - (c ? nt0 : 0);
+    ntc = c ? T - nt0 : nt0;
     const int rows = c ? rowsv[1] : rowsv[0];
-    const int cols = active ? (c ? colsv[1] : colsv[0]) : 0;
-    const int rbeg = c ? ra[1] : ra[0], rcnt = c ? rn[1] : rn[0];
-    const M* Mc = mat + (c ? mov[1] : mov[0]) + rbeg;
-    const int32_t* kc = kix + c * max_cols;
-    int roff[TR];
+    cols = active ? (c ? colsv[1] : colsv[0]) : 0;
+    rbeg = c ? ra[1] : ra[0];
+    rcnt = active ? (c ? rn[1] : rn[0]) : 0;
+    Mc = mat + (c ? mov[1] : mov[0]) + rbeg;
 #pragma unroll
     for (int i = 0; i < TR; ++i) roff[i] = min(rt + i * ntc, max(rcnt - 1, 0));
-    typename P::acc_t acc[TR][RB];
+    step = S * rows;
+    off = s * rows;
 #pragma unroll
-    for (int i = 0; i < TR; ++i)
+    for (int u = 0; u < U; ++u)
+      if (s + u * S < cols) load(u, mv[u]);
+  };
+  begin(tid);
+
+  // ---- inputs -> operands
+  wait_for_inputs();
+  if (d.lev == 0) {
+    for (int i = tid; i < l0 * RB; i += nt) {
+      const int rb = i / l0, e = i - rb * l0;
+      SM::put(opd + e * PITCH, rb, P::cvt(rb < nrb ? io.x[i0 + e + (int64_t)(r0 + rb) * io.ldx] : P::zero()));
+    }
+  } else {
+    const B* winb = (const B*)io.win;
+    for (int i = tid; i < (l0 + l1) * RB; i += nt) {
+      const int e = i / RB, rb = i - e * RB;
+      const int64_t o = e < l0 ? i0 + e : i1 + (e - l0);
+      SM::put(opd + e * PITCH, rb, BP::g_of(rb < nrb ? winb[o * io.R + r0 + rb] : BP::zero()));
+    }
+  }
+  __syncthreads();
+
+  // ---- block products
+  B* woutb = (B*)io.wout;
+  for (int w = tid; w - lane < T * S; w += nt) {
+    if (w != tid) begin(w);
+    const int32_t* kc = kix + c * max_cols;
+    SM acc[TR];
 #pragma unroll
-      for (int rb = 0; rb < RB; ++rb) P::init(acc[i][rb]);
-    // U columns per step: all their entries are loaded before the first is used
-    const int step = S * rows;
-    int k = s, off = s * rows, since = 0;
-    auto load = [&](int u, M (&mv)[TR]) {
+    for (int i = 0; i < TR; ++i) acc[i].init();
+    auto mac = [&](int k, const M (&m)[TR]) {
+      typename SM::ops_t g;
+      SM::load(g, opd + kc[k]);
 #pragma unroll
-      for (int i = 0; i < TR; ++i) {
-        const M* q = Mc + (off + u * step + roff[i]);
-        mv[i] = STREAM ? __ldcs(q) : __ldg(q);
+      for (int i = 0; i < TR; ++i) acc[i].mac(m[i], g);
+    };
+    int k = s, since = 0;
+    for (; k + (U - 1) * S < cols; k += U * S) {
+      // an entry's register takes the entry U columns on as soon as it is consumed
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        mac(k + u * S, mv[u]);
+        if (k + (U + u) * S < cols) load(U + u, mv[u]);
       }
-    };
-    auto mac = [&](int u, const M (&mv)[TR]) {
-      G g[RB];
-      load_ops<P, RB>(opd + kc[k + u * S], g);
-#pragma unroll
-      for (int i = 0; i < TR; ++i)
-#pragma unroll
-        for (int rb = 0; rb < RB; ++rb) P::mac(acc[i][rb], mv[i], g[rb]);
-    };
-    for (; k + (U - 1) * S < cols; k += U * S, off += U * step) {
-      M mv[U][TR];
-#pragma unroll
-      for (int u = 0; u < U; ++u) load(u, mv[u]);
-#pragma unroll
-      for (int u = 0; u < U; ++u) mac(u, mv[u]);
+      off += U * step;
       since += U;
       if (since >= P::CHUNK) {
 #pragma unroll
-        for (int i = 0; i < TR; ++i)
-#pragma unroll
-          for (int rb = 0; rb < RB; ++rb) P::flush(acc[i][rb]);
+        for (int i = 0; i < TR; ++i) acc[i].flush();
         since = 0;
       }
     }
-    {
-      M mv[U - 1][TR];
 #pragma unroll
-      for (int u = 0; u < U - 1; ++u)
-        if (k + u * S < cols) load(u, mv[u]);
-#pragma unroll
-      for (int u = 0; u < U - 1; ++u)
-        if (k + u * S < cols) mac(u, mv[u]);
-    }
-#pragma unroll
-    for (int i = 0; i < TR; ++i)
-#pragma unroll
-      for (int rb = 0; rb < RB; ++rb) lane_sum<P>(acc[i][rb], S);
-    if (!active) continue;
-    // every lane of the S has the sums: lane s writes the right-hand sides rb = s mod S
+    for (int u = 0; u < U - 1; ++u)
+      if (k + u * S < cols) mac(k + u * S, mv[u]);
 #pragma unroll
     for (int i = 0; i < TR; ++i) {
+      typename P::part_t pr[RB];
+      acc[i].parts(pr);
+      lane_sum<P, RB>(pr, S, s);
       const int rr = rt + i * ntc;
       if (rr >= rcnt) continue;
 #pragma unroll
-      for (int rb = 0; rb < RB; ++rb) {
-        if ((rb & (S - 1)) != s) continue;
-        B v = BP::of_acc(acc[i][rb]);
+      for (int ib = 0; ib < RB; ++ib) {
+        if (ib & (S - 1)) continue;
+        const int rb = ib | s;
+        if (rb >= RB) continue;
+        B v = BP::of_part(pr[ib]);
         if (ulev) {
           res[((size_t)(c ? rn[0] : 0) + rr) * RB + rb] = v;
         } else if (rb < nrb) {
-          if (d.kind == KIND_V) v = BP::add(v, BP::b_of_g(opd[aux[c * max_rows + rbeg + rr] * PITCH + rb]));
+          if (d.kind == KIND_V) v = BP::add(v, BP::b_of_g(SM::get(opd + aux[c * max_rows + rbeg + rr] * PITCH, rb)));
           woutb[((c ? obv[1] : obv[0]) + rbeg + rr) * io.R + r0 + rb] = v;
         }
       }
@@ -283,7 +399,7 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
   const int ne = e1 - e0;
   auto term = [&](int c, int e, int rb) -> B {
     const int t = aux[c * max_out + e];
-    return t >= 0 ? BP::b_of_g(opd[((c ? l0 : 0) + t) * PITCH + rb]) : res[((c ? rn[0] : 0) + ~t - ra[c]) * RB + rb];
+    return t >= 0 ? BP::b_of_g(SM::get(opd + ((c ? l0 : 0) + t) * PITCH, rb)) : res[((c ? rn[0] : 0) + ~t - ra[c]) * RB + rb];
   };
   if (d.lev == d.L) {
     const int64_t y0 = leaf_start(d, j) + e0;
@@ -328,6 +444,7 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
   using M = typename P::mat_t;
   using BP = BndOf<P>;
   using B = typename BP::b_t;
+  using SM = Sums<P, RB>;
   constexpr int PITCH = op_pitch<P, RB>();
   constexpr int CG = 32 / LR, CT = CG * TC;  // lane groups of a warp, columns of a warp's tile
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
@@ -343,6 +460,7 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
   const int rowsv[2] = {d.rows[2 * j], d.rows[2 * j + 1]};
   const int colsv[2] = {d.cols[2 * j], d.cols[2 * j + 1]};
   const int64_t mov[2] = {d.moff[2 * j], d.moff[2 * j + 1]};
+  if (!STREAM && r0 == 0) prefetch_blocks(mat, mov, rowsv, colsv, sl, nsl);
   int o0len, o1len = 0;
   int64_t b0, b1 = 0;
   if (d.lev == d.L) {
@@ -398,17 +516,18 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
     }
   }
   // ---- inputs -> operands
+  wait_for_inputs();
   if (d.lev == d.L) {
     for (int i = tid; i < o0len * RB; i += nt) {
       const int rb = i / o0len, e = i - rb * o0len;
-      opd[e * PITCH + rb] = P::cvt(rb < nrb ? io.x[b0 + e + (int64_t)(r0 + rb) * io.ldx] : P::zero());
+      SM::put(opd + e * PITCH, rb, P::cvt(rb < nrb ? io.x[b0 + e + (int64_t)(r0 + rb) * io.ldx] : P::zero()));
     }
   } else {
     const B* winb = (const B*)io.win;
     for (int i = tid; i < (o0len + o1len) * RB; i += nt) {
       const int e = i / RB, rb = i - e * RB;
       const int64_t off = e < o0len ? b0 + e : b1 + (e - o0len);
-      opd[e * PITCH + rb] = BP::g_of(rb < nrb ? winb[off * io.R + r0 + rb] : BP::zero());
+      SM::put(opd + e * PITCH, rb, BP::g_of(rb < nrb ? winb[off * io.R + r0 + rb] : BP::zero()));
     }
   }
   __syncthreads();
@@ -433,11 +552,9 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
     const int c = w >= nt0;
     const int i_first = (w - (c ? nt0 : 0)) * CT + cg;  // this lane's first column within the slice
     const int icnt = c ? in[1] : in[0], ibeg = c ? ia[1] : ia[0];
-    typename P::acc_t acc[TC][RB];
+    SM acc[TC];
 #pragma unroll
-    for (int t = 0; t < TC; ++t)
-#pragma unroll
-      for (int rb = 0; rb < RB; ++rb) P::init(acc[t][rb]);
+    for (int t = 0; t < TC; ++t) acc[t].init();
     int coff[TC];
 #pragma unroll
     for (int t = 0; t < TC; ++t) coff[t] = ibeg + min(i_first + t * CG, icnt - 1);
@@ -457,52 +574,51 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
         }
       };
       auto mac = [&](int u, const M (&mv)[TC]) {
-        G g[RB];
-        load_ops<P, RB>(opd + gc[r + u * LR], g);
+        typename SM::ops_t g;
+        SM::load(g, opd + gc[r + u * LR]);
 #pragma unroll
-        for (int t = 0; t < TC; ++t)
-#pragma unroll
-          for (int rb = 0; rb < RB; ++rb) P::macc(acc[t][rb], mv[t], g[rb]);
+        for (int t = 0; t < TC; ++t) acc[t].macc(mv[t], g);
       };
+      M mv[U][TC];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (r + u * LR < rows) load(u, mv[u]);
       for (; r + (U - 1) * LR < rows; r += U * LR) {
-        M mv[U][TC];
 #pragma unroll
-        for (int u = 0; u < U; ++u) load(u, mv[u]);
-#pragma unroll
-        for (int u = 0; u < U; ++u) mac(u, mv[u]);
+        for (int u = 0; u < U; ++u) {
+          mac(u, mv[u]);
+          if (r + (U + u) * LR < rows) load(U + u, mv[u]);
+        }
         since += U;
         if (since >= P::CHUNK) {
 #pragma unroll
-          for (int t = 0; t < TC; ++t)
-#pragma unroll
-            for (int rb = 0; rb < RB; ++rb) P::flush(acc[t][rb]);
+          for (int t = 0; t < TC; ++t) acc[t].flush();
           since = 0;
         }
       }
-      if constexpr (U > 1) {
-        M mv[U - 1][TC];
 #pragma unroll
-        for (int u = 0; u < U - 1; ++u)
-          if (r + u * LR < rows) load(u, mv[u]);
-#pragma unroll
-        for (int u = 0; u < U - 1; ++u)
-          if (r + u * LR < rows) mac(u, mv[u]);
-      }
+      for (int u = 0; u < U - 1; ++u)
+        if (r + u * LR < rows) mac(u, mv[u]);
     }
     __syncwarp();
 #pragma unroll
-    for (int t = 0; t < TC; ++t)
-#pragma unroll
-      for (int rb = 0; rb < RB; ++rb) lane_sum<P>(acc[t][rb], LR);
-#pragma unroll
     for (int t = 0; t < TC; ++t) {
-      const int ii = i_first + t * CG;
-      if (ii >= icnt) continue;
-      const int i = ibeg + ii;
+      typename P::part_t pr[RB];
+      acc[t].parts(pr);
+      lane_sum<P, RB>(pr, LR < 8 ? LR : 8, lr & 7);
+      if constexpr (LR == 16) {
 #pragma unroll
-      for (int rb = 0; rb < RB; ++rb) {
-        if ((rb & (LR - 1)) != lr) continue;
-        B v = BP::of_acc(acc[t][rb]);
+        for (int rb = 0; rb < RB; ++rb) pr[rb] = P::add_lane(pr[rb], pr[rb], 8);
+      }
+      const int ii = i_first + t * CG;
+      if (ii >= icnt || lr >= 8) continue;
+      const int i = ibeg + ii;
+      constexpr int LS = LR < 8 ? LR : 8;
+#pragma unroll
+      for (int ib = 0; ib < RB; ib += LS) {
+        const int rb = ib | lr;
+        if (rb >= RB) continue;
+        B v = BP::of_part(pr[ib]);
         if (vlev) {
           res[((c ? in[0] : 0) + ii) * RB + rb] = v;
         } else if (rb < nrb) {
@@ -510,7 +626,7 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
             woutb[(i < len0 ? ib0 + i : ib1 + (i - len0)) * io.R + r0 + rb] = v;
           } else {  // U: forward input segment c gets v[q_c] + res_c
             const int q = d.idx[d.ioff[2 * j + c] + i];
-            woutb[((c ? ib1 : ib0) + i) * io.R + r0 + rb] = BP::add(BP::b_of_g(opd[q * PITCH + rb]), v);
+            woutb[((c ? ib1 : ib0) + i) * io.R + r0 + rb] = BP::add(BP::b_of_g(SM::get(opd + q * PITCH, rb)), v);
           }
         }
       }
@@ -523,7 +639,7 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
   const int ne = e1 - e0;
   auto term = [&](int c, int e, int rb) -> B {
     const int t = aux[c * max_in + e];
-    return t >= 0 ? BP::b_of_g(opd[((c ? o0len : 0) + t) * PITCH + rb]) : res[((c ? in[0] : 0) + ~t - ia[c]) * RB + rb];
+    return t >= 0 ? BP::b_of_g(SM::get(opd + ((c ? o0len : 0) + t) * PITCH, rb)) : res[((c ? in[0] : 0) + ~t - ia[c]) * RB + rb];
   };
   if (d.lev == 0) {
     const int64_t y0 = leaf_start(d, j) + e0;
