@@ -14,6 +14,7 @@
 
 #include "idbf_internal.h"
 #include "level_kernels.cuh"
+#include "node_launch.h"
 
 namespace idbf {
 
@@ -182,6 +183,11 @@ __global__ void __launch_bounds__(RG::NTHREADS, RG::CTAS)
   constexpr int STAGES = RG::STAGES, STAGE_BYTES = RG::STAGE_BYTES;
   constexpr int TEAMS = RG::TEAMS, NCT = RG::NCT;
   constexpr int NSUB = PAIR ? 4 : 1;  // nodes per work unit
+  // Complex64, bound by HBM: the next launch's CTAs take over as slots free up and ask for their
+  // first nodes' blocks while this launch drains (FIO, variant 1: N = 2^14 108 -> 87 us, 2^16 296 ->
+  // 262 us). Double-float, bound by issue and the FMA pipe, loses by that (2^16: 699 -> 728 us); there
+  // only the launch itself overlaps (724 -> 699 us).
+  constexpr bool EARLY = sizeof(M) == 8;
   extern __shared__ __align__(128) unsigned char smem[];
   static_assert(RPT == 1 || !SPLIT, "the column split is for one output row per thread");
   const Geo geo = geometry<P, RG>(max_in, max_out, max_cols_pair, RPT, SPLIT, PAIR ? mid_elems : 0);
@@ -204,6 +210,7 @@ __global__ void __launch_bounds__(RG::NTHREADS, RG::CTAS)
   __shared__ NodeMeta nmeta[2];  // description of the node in input buffer b
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t nunits = PAIR ? d.m / 2 : d.m;
+  if constexpr (EARLY) node::next_may_begin();
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) {
       mbar_init(&full[i], 1);
@@ -272,6 +279,12 @@ __global__ void __launch_bounds__(RG::NTHREADS, RG::CTAS)
     int64_t un = blockIdx.x;
     int v = 0;
     NodeMeta nxt = meta(un < nunits ? un : 0, 0);
+    if constexpr (EARLY) {
+      if (un < nunits)
+        for (int c = 0; c < 2; ++c)
+          node::prefetch_l2((nxt.sel ? mat1 : mat) + nxt.mo[c], (int64_t)nxt.rows[c] * nxt.cols[c] * ES);
+    }
+    node::wait_for_inputs();
     for (; un < nunits && ok; ++nn) {
       const NodeMeta cur = nxt;
       const bool second = PAIR && cur.sel;
@@ -358,6 +371,7 @@ __global__ void __launch_bounds__(RG::NTHREADS, RG::CTAS)
   const int tr = tc - team * TCT;       // row index within the team
   uint32_t it = 0, nn = 0;
   bool failed = false;
+  node::wait_for_inputs();
   for (int64_t un = blockIdx.x; un < nunits; un += gridDim.x) {
   for (int sub = 0; sub < NSUB; ++sub, ++nn) {
     consumer_sync<NCT>();
@@ -610,13 +624,23 @@ constexpr Arith arith_of() {
   return std::is_same<P, FP64P>::value ? ARITH_FP64 : std::is_same<P, DF64P>::value ? ARITH_DF64 : ARITH_FP32;
 }
 
-static int default_variant(int fmt) { return fmt == IDBF_STORE_C128 ? 0 : 1; }
+// Level l of a plan that was not tuned. FP64 runs the node kernel. Double-float and FP32 run the
+// streaming kernel where tall blocks come in numbers that fill its persistent CTAs, the node
+// kernel elsewhere (one vector, us, node / streaming; double-float: FIO N = 2^16 689 / 725, 2^18
+// 2850 / 2654, J_0 N = 2^17 541 / 761; FP32: FIO 2^12 42 / 57, 2^14 125 / 108, 2^16 303 / 296, J_0
+// 250 / 349). The fault injection of idbf_debug_set_wait needs the streaming kernel's waits.
+static int default_variant(const Plan* p, int l, int fmt) {
+  if (fmt == IDBF_STORE_C128) return 0;
+  if (!p->producer_enabled) return 1;
+  const bool tall = p->lv[l].max_rows > 64;
+  return tall && p->m >= (fmt == IDBF_STORE_DF64 ? 4096 : 256) ? 1 : 0;
+}
 
 // One level l (pair = false) or the fused pair of levels l, l + 1 (pair = true) with the
 // streaming kernel and ring layout RG.
 template <class P, class RG>
 static idbf_status launch_stream(Plan* p, int l, bool pair, bool bulk, bool split_short, const void* x,
-                                 IO<typename P::vec_t> io, cudaStream_t st) {
+                                 IO<typename P::vec_t> io, cudaStream_t st, bool after) {
   using V = typename P::vec_t;
   if (pair && (l + 1 > p->L)) return IDBF_EUNSUPPORTED;
   const LevelInfo& li = p->lv[l];
@@ -655,8 +679,9 @@ static idbf_status launch_stream(Plan* p, int l, bool pair, bool bulk, bool spli
   const typename P::mat_t* mat1 = (const typename P::mat_t*)p->lmat[fmt_of<P>()][pair ? l + 1 : l];
   auto go = [&](auto kern) -> idbf_status {
     IDBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)geo.total));
-    kern<<<ctas, RG::NTHREADS, geo.total, st>>>(d, mat, d1, mat1, io, max_in, max_out, max_cols_pair, mid_elems,
-                                                use_bulk, p->d_status, p->wait_limit_ns, p->producer_enabled);
+    IDBF_CUDA_TRY(node::launch_after(kern, after, ctas, RG::NTHREADS, geo.total, st, d, mat, d1, mat1, io, max_in, max_out,
+                                     max_cols_pair, mid_elems, use_bulk, p->d_status, p->wait_limit_ns,
+                                     p->producer_enabled));
     return IDBF_OK;
   };
   idbf_status s;
@@ -707,21 +732,21 @@ static idbf_status launch_fwd_variant(Plan* p, int l, int v, const void* x, void
   if (v != 0 && fmt == IDBF_STORE_C128) return IDBF_EUNSUPPORTED;  // FP64: per-node or warp-per-node kernel
   if (v >= kFirstPairVariant) {  // levels l and l + 1 fused (win: boundary l - 1, wout: boundary l + 1)
     switch (v - kFirstPairVariant) {
-      case 0: return launch_stream<P, strm::RingA>(p, l, true, true, true, x, io, st);
-      case 1: return launch_stream<P, strm::RingB>(p, l, true, true, true, x, io, st);
-      case 2: return launch_stream<P, strm::RingC>(p, l, true, true, true, x, io, st);
-      default: return launch_stream<P, strm::RingD>(p, l, true, true, true, x, io, st);
+      case 0: return launch_stream<P, strm::RingA>(p, l, true, true, true, x, io, st, after);
+      case 1: return launch_stream<P, strm::RingB>(p, l, true, true, true, x, io, st, after);
+      case 2: return launch_stream<P, strm::RingC>(p, l, true, true, true, x, io, st, after);
+      default: return launch_stream<P, strm::RingD>(p, l, true, true, true, x, io, st, after);
     }
   }
-  if (v == 14 || v == 15) return launch_stream<P, strm::RingD>(p, l, false, v == 14, true, x, io, st);
+  if (v == 14 || v == 15) return launch_stream<P, strm::RingD>(p, l, false, v == 14, true, x, io, st, after);
   const bool split = v >= 8;
   switch (split ? v - 7 : v) {
-    case 1: return launch_stream<P, strm::RingA>(p, l, false, true, split, x, io, st);
-    case 2: return launch_stream<P, strm::RingA>(p, l, false, false, split, x, io, st);
-    case 3: return launch_stream<P, strm::RingB>(p, l, false, true, split, x, io, st);
-    case 4: return launch_stream<P, strm::RingB>(p, l, false, false, split, x, io, st);
-    case 5: return launch_stream<P, strm::RingC>(p, l, false, true, split, x, io, st);
-    case 6: return launch_stream<P, strm::RingC>(p, l, false, false, split, x, io, st);
+    case 1: return launch_stream<P, strm::RingA>(p, l, false, true, split, x, io, st, after);
+    case 2: return launch_stream<P, strm::RingA>(p, l, false, false, split, x, io, st, after);
+    case 3: return launch_stream<P, strm::RingB>(p, l, false, true, split, x, io, st, after);
+    case 4: return launch_stream<P, strm::RingB>(p, l, false, false, split, x, io, st, after);
+    case 5: return launch_stream<P, strm::RingC>(p, l, false, true, split, x, io, st, after);
+    case 6: return launch_stream<P, strm::RingC>(p, l, false, false, split, x, io, st, after);
     default: break;
   }
   return node_fwd(p, arith_of<P>(), l, LevelIO{x, p->N, y, p->N, win, wout, 1, after}, st);
@@ -751,18 +776,18 @@ static idbf_status run_fwd1(Plan* p, const void* x, void* y, int64_t ld, cudaStr
   V* wb[2] = {(V*)p->d_ws, (V*)((char*)p->d_ws + (size_t)p->max_seg_total * 16)};
   int cur = 1;  // buffer holding the last boundary written (boundary b in b % 2 without pairs)
   for (int l = 0; l <= p->L;) {
-    int v = p->tuned[fmt].size() > (size_t)l && p->tuned[fmt][l] >= 0 ? p->tuned[fmt][l] : default_variant(fmt);
+    int v = p->tuned[fmt].size() > (size_t)l && p->tuned[fmt][l] >= 0 ? p->tuned[fmt][l] : default_variant(p, l, fmt);
     const bool pair = is_pair_variant(v) && l < p->L;
     const int last = pair ? l + 1 : l;  // level whose outputs this launch writes
     const V* win = l > 0 ? wb[cur] : nullptr;
     V* wout = last < p->L ? wb[cur ^ 1] : nullptr;
     (void)ld;
     idbf_status s = IDBF_EUNSUPPORTED;
-    if (is_pair_variant(v) && !pair) v = default_variant(fmt);  // a pair variant on level L: one level
+    if (is_pair_variant(v) && !pair) v = default_variant(p, l, fmt);  // a pair variant on level L: one level
     s = launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt, l > 0);
     if (s == IDBF_EUNSUPPORTED && pair) {  // the pair does not fit: level l alone, into the next buffer
       V* wout1 = wb[cur ^ 1];               // l < L here, so level l writes a workspace boundary
-      s = launch_fwd_variant<P>(p, l, default_variant(fmt), x, y, win, wout1, st, fmt, l > 0);
+      s = launch_fwd_variant<P>(p, l, default_variant(p, l, fmt), x, y, win, wout1, st, fmt, l > 0);
       if (s == IDBF_EUNSUPPORTED) s = launch_fwd_variant<P>(p, l, 0, x, y, win, wout1, st, fmt, l > 0);
       if (s != IDBF_OK) return s;
       if (l < p->L) cur ^= 1;
@@ -927,7 +952,8 @@ static idbf_status autotune_fmt(Plan* p, int fmt, cudaStream_t st, int reps, flo
     idbf_status r = launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt, false);
     if (r != IDBF_OK) return r;
     cudaEventRecord(e0, st);
-    for (int k = 0; k < reps; ++k) launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt, false);
+    // as in an apply: every launch may begin while its predecessor drains
+    for (int k = 0; k < reps; ++k) launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt, true);
     cudaEventRecord(e1, st);
     if (cudaEventSynchronize(e1) != cudaSuccess) return IDBF_ECUDA;
     cudaEventElapsedTime(ms_out, e0, e1);
@@ -935,7 +961,7 @@ static idbf_status autotune_fmt(Plan* p, int fmt, cudaStream_t st, int reps, flo
   };
   const int nl = p->L + 1;
   std::vector<float> one(nl, 1e30f), two(nl, 1e30f);
-  std::vector<int> one_v(nl, default_variant(fmt)), two_v(nl, -1);
+  std::vector<int> one_v(nl, 0), two_v(nl, -1);
   for (int l = 0; l < nl && s == IDBF_OK; ++l) {
     for (int v = 0; v < kNumFwdVariants && s == IDBF_OK; ++v) {
       if (is_pair_variant(v) && l == p->L) continue;

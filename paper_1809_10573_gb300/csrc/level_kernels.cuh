@@ -46,7 +46,7 @@ struct FP64P {
   using vec_t = double2;
   using gv_t = double2;
   struct acc_t { double re, im; };
-  static constexpr int CHUNK = 16;
+  static constexpr int CHUNK = 16, ADJ_CHUNK = 16;
   __device__ static __forceinline__ mat_t ld(const mat_t* p) { return __ldcs(p); }
   __device__ static __forceinline__ gv_t cvt(vec_t v) { return v; }
   __device__ static __forceinline__ void init(acc_t& a) { a.re = 0.0; a.im = 0.0; }
@@ -88,7 +88,7 @@ struct FP32P {
   using vec_t = float2;
   using gv_t = float2;
   struct acc_t { float re, im; };
-  static constexpr int CHUNK = 16;
+  static constexpr int CHUNK = 16, ADJ_CHUNK = 16;
   __device__ static __forceinline__ mat_t ld(const mat_t* p) { return __ldcs(p); }
   __device__ static __forceinline__ gv_t cvt(vec_t v) { return v; }
   __device__ static __forceinline__ void init(acc_t& a) { a.re = 0.f; a.im = 0.f; }
@@ -162,7 +162,10 @@ struct DF64P {
   using vec_t = double2;
   using gv_t = float4;
   struct acc_t { float sr, cr, si, ci, hr, lr, hi, li; };
-  static constexpr int CHUNK = 16;
+  // terms between two folds of (s, c), whose error grows with the terms they hold; the adjoint cuts a
+  // column over 8 lanes and folds often, so that its error stays that of 32 short chains (FIO
+  // N = 2^16: 1.8e-14 against 3.6e-14 with 16 terms)
+  static constexpr int CHUNK = 16, ADJ_CHUNK = 2;
   __device__ static __forceinline__ mat_t ld(const mat_t* p) { return __ldcs(p); }
   __device__ static __forceinline__ gv_t cvt(vec_t v) {
     const float rh = (float)v.x, ih = (float)v.y;
@@ -323,6 +326,22 @@ struct IO {
 __device__ __forceinline__ int64_t out_seg_id(const DevLevel& d, int64_t j, int c) {
   return (j / d.H) * 2 * d.H + j % d.H + c * d.H;
 }
+
+namespace node {
+// Asks for `bytes` at p (rounded out to 16-byte granules, which the arenas' tails allow) in L2: one
+// instruction streams a whole block from HBM while the CTA is still loading its index lists and
+// inputs, so that the product loop's loads meet L2 latency instead of HBM latency.
+__device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
+  const uintptr_t a = (uintptr_t)p & ~(uintptr_t)15;
+  const uint32_t n = (uint32_t)((((uintptr_t)p + bytes + 15) & ~(uintptr_t)15) - a);
+  if (bytes > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(n) : "memory");
+}
+// A level's launch may begin while the previous level still runs (launch_after in node.cu): what
+// comes before wait_for_inputs reads the factors only. next_may_begin lets the following launch
+// begin once every CTA of this one has started.
+__device__ __forceinline__ void wait_for_inputs() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void next_may_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+}  // namespace node
 
 // ---------------------------------------------------------------------------------------------
 // Warp-per-node forward body, one right-hand side, for levels of short blocks (the outer levels

@@ -114,20 +114,6 @@ struct Sums<P, RB, true> {
   }
 };
 
-// Asks for `bytes` at p (rounded out to 16-byte granules, which the arenas' tails allow) in L2: one
-// instruction streams a whole block from HBM while the CTA is still loading its index lists and
-// inputs, so that the product loop's loads meet L2 latency instead of HBM latency.
-__device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
-  const uintptr_t a = (uintptr_t)p & ~(uintptr_t)15;
-  const uint32_t n = (uint32_t)((((uintptr_t)p + bytes + 15) & ~(uintptr_t)15) - a);
-  if (bytes > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"(n) : "memory");
-}
-// A level's launch may begin while the previous level still runs (launch_after in node.cu): what
-// comes before wait_for_inputs reads the factors only. next_may_begin lets the following launch
-// begin once every CTA of this one has started.
-__device__ __forceinline__ void wait_for_inputs() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void next_may_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // the share of slice sl of nsl of both blocks of a node, by two threads of the CTA
 template <class M>
 __device__ __forceinline__ void prefetch_blocks(const M* mat, const int64_t (&mov)[2], const int (&rows)[2],
@@ -590,7 +576,7 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
           if (r + (U + u) * LR < rows) load(U + u, mv[u]);
         }
         since += U;
-        if (since >= P::CHUNK) {
+        if (since >= P::ADJ_CHUNK) {
 #pragma unroll
           for (int t = 0; t < TC; ++t) acc[t].flush();
           since = 0;
