@@ -81,7 +81,7 @@ struct IDDesc {
   int64_t n_c;
   int32_t ns;        // samples
   int32_t kmax;      // max rank (min(ns, b, k))
-  int32_t pad0;
+  int32_t order;     // QR: the batch's IDs by falling cost (entry i: the ID that CTA i factors)
   int32_t pad;
   uint64_t key;      // random sampling stream
   // scratch offsets (batch-relative)
@@ -119,17 +119,20 @@ __device__ __forceinline__ int hs_find(const int32_t* keys, int cap, int32_t k) 
 }
 
 // Mock-Chebyshev (sampling == 0), random (1), all (2). Output: sorted global indices.
-// Shared memory per warp: keys[cap], vals[cap], picks[nsmax]; cap is a power of two larger than
-// twice the number of keys inserted (ns for Mock-Chebyshev, up to 2 ns for the shuffle).
+// Shared memory per warp: keys[cap], vals[cap], picks[nsmax] and the distances of every node to the
+// candidates on either side, near[nsmax][2]; cap is a power of two larger than twice the number of keys inserted (ns
+// for Mock-Chebyshev, up to 2 ns for the shuffle). The serial choice of lane 0 then reads global
+// memory only where a neighbour is taken already (FIO N = 2^15: 13.1 -> 8.5 ms of the build).
 __global__ void k_sample(const IDDesc* __restrict__ D, int64_t nid, const int32_t* __restrict__ list,
                          const double* __restrict__ coord, int32_t* __restrict__ samp, int sampling, int cap,
                          int nsmax) {
-  extern __shared__ int32_t sm[];
+  extern __shared__ __align__(16) int32_t sm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwarps = blockDim.x >> 5;
   const int64_t id = (int64_t)blockIdx.x * nwarps + warp;
   if (id >= nid) return;
-  int32_t* keys = sm + (size_t)warp * (cap * 2 + nsmax);
+  double* near = (double*)sm + (size_t)warp * 2 * nsmax;
+  int32_t* keys = sm + (size_t)nwarps * 4 * nsmax + (size_t)warp * (cap * 2 + nsmax);
   int32_t* vals = keys + cap;
   int32_t* picks = vals + cap;
   const IDDesc d = D[id];
@@ -153,12 +156,12 @@ __global__ void k_sample(const IDDesc* __restrict__ D, int64_t nid, const int32_
         if (coord[cand_index(d, list, mid)] < y) a = mid + 1; else b = mid;
       }
       picks[j] = (int32_t)a;
+      near[2 * j] = a > 0 ? y - coord[cand_index(d, list, a - 1)] : 0.0;
+      near[2 * j + 1] = a < d.n_c ? coord[cand_index(d, list, a)] - y : 0.0;
     }
     __syncwarp();
     if (lane == 0) {
       for (int j = 0; j < ns; ++j) {
-        const double t = (1.0 - cospi((2.0 * j + 1.0) / (2.0 * ns))) * 0.5;
-        const double y = lo + t * (hi - lo);
         const int64_t pos = picks[j];
         int64_t left = pos - 1, right = pos;
         while (left >= 0 && keys[hs_find(keys, cap, (int32_t)left)] != 0) --left;
@@ -166,7 +169,12 @@ __global__ void k_sample(const IDDesc* __restrict__ D, int64_t nid, const int32_
         int64_t pick;
         if (left < 0) pick = right;
         else if (right >= d.n_c) pick = left;
-        else pick = (y - coord[cand_index(d, list, left)]) <= (coord[cand_index(d, list, right)] - y) ? left : right;
+        else if (left == pos - 1 && right == pos) pick = near[2 * j] <= near[2 * j + 1] ? left : right;
+        else {
+          const double t = (1.0 - cospi((2.0 * j + 1.0) / (2.0 * ns))) * 0.5;
+          const double y = lo + t * (hi - lo);
+          pick = (y - coord[cand_index(d, list, left)]) <= (coord[cand_index(d, list, right)] - y) ? left : right;
+        }
         keys[hs_find(keys, cap, (int32_t)pick)] = (int32_t)pick + 1;
         picks[j] = (int32_t)pick;
       }
@@ -287,7 +295,8 @@ __global__ void __launch_bounds__(NT) k_qr(const IDDesc* __restrict__ D, double2
                                            int32_t* __restrict__ pscr, int32_t* __restrict__ kout,
                                            int32_t* __restrict__ satur, double eps) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const IDDesc d = D[blockIdx.x];
+  const int id = D[blockIdx.x].order;  // the longest first, so that the last wave is of short ones
+  const IDDesc d = D[id];
   const int ns = d.ns, b = d.b, kmax = d.kmax;
   double2* A = Aall + d.a_off;
   double2* v = (double2*)smraw;               // Householder vector, ns
@@ -391,9 +400,9 @@ __global__ void __launch_bounds__(NT) k_qr(const IDDesc* __restrict__ D, double2
     for (int c = 1 + tid; c < b; c += NT) A[(int64_t)c * ns] = make_double2(0.0, 0.0);
   }
   if (tid == 0) {
-    kout[blockIdx.x] = k;
+    kout[id] = k;
     // stopped at the cap, not by eps (an empty block, kmax = 0, has rank 0 by definition)
-    satur[blockIdx.x] = (!zero_block && kmax > 0 && k == kmax && kmax < b) ? 1 : 0;
+    satur[id] = (!zero_block && kmax > 0 && k == kmax && kmax < b) ? 1 : 0;
   }
   __syncthreads();
   if (zero_block) return;
@@ -490,12 +499,19 @@ __device__ __forceinline__ double block_sum_d(double v, double* rv) {
 }
 
 // As k_qr, on double-float entries (float4); same outputs: kout, perm in pscr, T in A(0:k, k:b).
-template <int NT>
-__global__ void __launch_bounds__(NT) k_qr_df(const IDDesc* __restrict__ D, double2* __restrict__ Araw,
+//
+// Bound by latency (each step waits for its loads) and, before the columns were taken NC at a time,
+// by the FP64 pipe (47 % busy with one column's scalars on all 32 lanes). Two shapes, by the batch's
+// blocks: 512 threads, one CTA per SM, for blocks of more than 128 columns (FIO N = 2^15: build 265
+// ms against 280 with 256 threads), else 256 threads, three CTAs per SM (NUFFT N = 50000: 89 against
+// 117 ms). One column at a time: 453 and 150 ms.
+template <int NT, int NC, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_qr_df(const IDDesc* __restrict__ D, double2* __restrict__ Araw,
                                               int32_t* __restrict__ pscr, int32_t* __restrict__ kout,
                                               int32_t* __restrict__ satur, double eps) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const IDDesc d = D[blockIdx.x];
+  const int id = D[blockIdx.x].order;  // the longest first, so that the last wave is of short ones
+  const IDDesc d = D[id];
   const int ns = d.ns, b = d.b, kmax = d.kmax;
   float4* A = (float4*)(Araw + d.a_off);
   float4* v = (float4*)smraw;                 // Householder vector, ns (double-float complex)
@@ -591,36 +607,75 @@ __global__ void __launch_bounds__(NT) k_qr_df(const IDDesc* __restrict__ D, doub
     for (int i = j + 1 + tid; i < ns; i += NT) v[i - j] = cj[i];
     __syncthreads();
     const double coef = sh_coef;
-    // trailing columns: a -= coef v (v^* a); FP32 norms of rows j+1.. recomputed
-    for (int c = j + 1 + warp; c < b; c += NW) {
-      float4* col = A + (int64_t)c * ns;
-      float dr = 0.f, er = 0.f, di = 0.f, ei = 0.f;  // v^* a: (sum, compensation) per part
+    // trailing columns: a -= coef v (v^* a); FP32 norms of rows j+1.. recomputed. A warp takes NC
+    // columns at a time: one read of v serves them all, their loads are in flight together, and
+    // the FP64 scalars of the NC columns are one pass of the FP64 pipe (group g of 32 / NC lanes
+    // computes column g's).
+    for (int c0 = j + 1 + warp * NC; c0 < b; c0 += NW * NC) {
+      float4* col[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) col[q] = A + (int64_t)min(c0 + q, b - 1) * ns;
+      const int nc = min(NC, b - c0);
+      float dr[NC], er[NC], di[NC], ei[NC];  // v^* a: (sum, compensation) per part
+#pragma unroll
+      for (int q = 0; q < NC; ++q) dr[q] = er[q] = di[q] = ei[q] = 0.f;
+#pragma unroll 2
       for (int i = j + lane; i < ns; i += 32) {
-        const float4 z = col[i], w = v[i - j];
-        df2_dot(dr, er, w.x, w.y, z.x, z.y);   // Re: wr zr + wi zi
-        df2_dot(dr, er, w.z, w.w, z.z, z.w);
-        df2_dot(di, ei, w.x, w.y, z.z, z.w);   // Im: wr zi - wi zr
-        df2_dot(di, ei, -w.z, -w.w, z.x, z.y);
+        const float4 w = v[i - j];
+        float4 z[NC];
+#pragma unroll
+        for (int q = 0; q < NC; ++q) z[q] = col[q][i];
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          df2_dot(dr[q], er[q], w.x, w.y, z[q].x, z[q].y);   // Re: wr zr + wi zi
+          df2_dot(dr[q], er[q], w.z, w.w, z[q].z, z[q].w);
+          df2_dot(di[q], ei[q], w.x, w.y, z[q].z, z[q].w);   // Im: wr zi - wi zr
+          df2_dot(di[q], ei[q], -w.z, -w.w, z[q].x, z[q].y);
+        }
       }
-      float hr, lr, hi, li;
-      df2_fast(dr, er, hr, lr);
-      df2_fast(di, ei, hi, li);
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ohr = __shfl_xor_sync(0xffffffffu, hr, o), olr = __shfl_xor_sync(0xffffffffu, lr, o);
-        const float ohi = __shfl_xor_sync(0xffffffffu, hi, o), oli = __shfl_xor_sync(0xffffffffu, li, o);
-        df2_acc(hr, lr, ohr, olr);
-        df2_acc(hi, li, ohi, oli);
+      float hr = 0.f, lr = 0.f, hi = 0.f, li = 0.f;  // the sums of column lane / (32 / NC)
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        float ar, br, ai, bi2;
+        df2_fast(dr[q], er[q], ar, br);
+        df2_fast(di[q], ei[q], ai, bi2);
+        for (int o = 16; o > 0; o >>= 1) {
+          const float ohr = __shfl_xor_sync(0xffffffffu, ar, o), olr = __shfl_xor_sync(0xffffffffu, br, o);
+          const float ohi = __shfl_xor_sync(0xffffffffu, ai, o), oli = __shfl_xor_sync(0xffffffffu, bi2, o);
+          df2_acc(ar, br, ohr, olr);
+          df2_acc(ai, bi2, ohi, oli);
+        }
+        if (lane / (32 / NC) == q) { hr = ar; lr = br; hi = ai; li = bi2; }
       }
-      const double2 f = make_double2(coef * ((double)hr + (double)lr), coef * ((double)hi + (double)li));
-      const float4 fd = df_split(f);
-      float s = 0.f;
+      const float4 fl = df_split(make_double2(coef * ((double)hr + (double)lr), coef * ((double)hi + (double)li)));
+      float4 fd[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        const int src = q * (32 / NC);
+        fd[q] = make_float4(__shfl_sync(0xffffffffu, fl.x, src), __shfl_sync(0xffffffffu, fl.y, src),
+                            __shfl_sync(0xffffffffu, fl.z, src), __shfl_sync(0xffffffffu, fl.w, src));
+      }
+      float s[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) s[q] = 0.f;
+#pragma unroll 2
       for (int i = j + lane; i < ns; i += 32) {
-        const float4 z = df_cmsub(col[i], fd, v[i - j]);
-        col[i] = z;
-        if (i > j) s = fmaf(z.x, z.x, fmaf(z.z, z.z, s));
+        const float4 w = v[i - j];
+        float4 z[NC];
+#pragma unroll
+        for (int q = 0; q < NC; ++q) z[q] = col[q][i];
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          z[q] = df_cmsub(z[q], fd[q], w);
+          if (q < nc) col[q][i] = z[q];
+          if (i > j) s[q] = fmaf(z[q].x, z[q].x, fmaf(z[q].z, z[q].z, s[q]));
+        }
       }
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) nrm[c] = s;
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+        if (lane == 0 && q < nc) nrm[c0 + q] = s[q];
+      }
     }
     if (tid == 0) cj[j] = sh_beta;
     __syncthreads();
@@ -633,27 +688,54 @@ __global__ void __launch_bounds__(NT) k_qr_df(const IDDesc* __restrict__ D, doub
     for (int c = 1 + tid; c < b; c += NT) A[(int64_t)c * ns] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   if (tid == 0) {
-    kout[blockIdx.x] = k;
+    kout[id] = k;
     // stopped at the cap, not by eps (an empty block, kmax = 0, has rank 0 by definition)
-    satur[blockIdx.x] = (!zero_block && kmax > 0 && k == kmax && kmax < b) ? 1 : 0;
+    satur[id] = (!zero_block && kmax > 0 && k == kmax && kmax < b) ? 1 : 0;
   }
   __syncthreads();
   if (zero_block) return;
-  // T = R11^{-1} R12 by column-oriented back substitution, a warp per column of R12; the
-  // quotient in FP64, the updates in double-float
-  for (int c = k + warp; c < b; c += NW) {
-    float4* col = A + (int64_t)c * ns;
+  // T = R11^{-1} R12 by column-oriented back substitution, a warp per NC columns of R12: the
+  // quotients in FP64 (the reciprocals of the diagonal once per ID, in v's space), the updates in
+  // double-float
+  double2* rinv = (double2*)v;
+  for (int i = tid; i < k; i += NT) {
+    const double2 r = df_join(A[(int64_t)i * ns + i]);
+    const double den = r.x * r.x + r.y * r.y;
+    rinv[i] = make_double2(r.x / den, -r.y / den);
+  }
+  __syncthreads();
+  for (int c0 = k + warp * NC; c0 < b; c0 += NW * NC) {
+    float4* col[NC];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) col[q] = A + (int64_t)min(c0 + q, b - 1) * ns;
+    const int nc = min(NC, b - c0);
+    const int mine = lane / (32 / NC);  // column whose quotient this lane computes
+    float4* cm = A + (int64_t)min(c0 + mine, b - 1) * ns;
     for (int i = k - 1; i >= 0; --i) {
       __syncwarp();
-      const double2 rii = df_join(A[(int64_t)i * ns + i]);
-      const double2 num = df_join(col[i]);
-      const double den = rii.x * rii.x + rii.y * rii.y;
-      const double2 t = make_double2((num.x * rii.x + num.y * rii.y) / den, (num.y * rii.x - num.x * rii.y) / den);
-      const float4 td = df_split(t);
+      const double2 num = df_join(cm[i]), ri = rinv[i];
+      const float4 tl = df_split(make_double2(num.x * ri.x - num.y * ri.y, num.x * ri.y + num.y * ri.x));
+      float4 td[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        const int src = q * (32 / NC);
+        td[q] = make_float4(__shfl_sync(0xffffffffu, tl.x, src), __shfl_sync(0xffffffffu, tl.y, src),
+                            __shfl_sync(0xffffffffu, tl.z, src), __shfl_sync(0xffffffffu, tl.w, src));
+      }
       const float4* ci = A + (int64_t)i * ns;
-      for (int l = lane; l < i; l += 32) col[l] = df_cmsub(col[l], ci[l], td);
+      for (int l = lane; l < i; l += 32) {
+        const float4 r = ci[l];
+        float4 z[NC];
+#pragma unroll
+        for (int q = 0; q < NC; ++q) z[q] = col[q][l];
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          z[q] = df_cmsub(z[q], r, td[q]);
+          if (q < nc) col[q][l] = z[q];
+        }
+      }
       __syncwarp();
-      if (lane == 0) col[i] = td;
+      if (lane % (32 / NC) == 0 && mine < nc) cm[i] = tl;
     }
   }
 }
@@ -936,6 +1018,13 @@ idbf_status Builder::run_step(int side, int s) {
       maxns = std::max(maxns, d.ns);
       maxb = std::max(maxb, d.b);
     }
+    {
+      std::vector<int32_t> ord(nb);
+      for (int64_t i = 0; i < nb; ++i) ord[i] = (int32_t)i;
+      auto cost = [&](int32_t i) { return (int64_t)Db[i].ns * Db[i].b * std::max(Db[i].kmax, 1); };
+      std::stable_sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) { return cost(x) > cost(y); });
+      for (int64_t i = 0; i < nb; ++i) Db[i].order = ord[i];
+    }
     cudaError_t e;
     if ((e = A.ensure(std::max<int64_t>(a, 1) * 16)) != cudaSuccess ||
         (e = blist.ensure(std::max<int64_t>(bo, 1) * 4)) != cudaSuccess ||
@@ -954,10 +1043,11 @@ idbf_status Builder::run_step(int side, int s) {
     // sampling: one ID per warp; hash capacity a power of two >= 4 ns (load factor <= 1/2)
     int cap = 64;
     while (cap < 4 * maxns) cap <<= 1;
-    const size_t per_warp = ((size_t)cap * 2 + maxns) * 4;
+    const size_t tables = ((size_t)cap * 2 + maxns) * 4;
+    if (tables > 200 * 1024) { free_res(); return IDBF_EUNSUPPORTED; }
+    const size_t per_warp = tables + (size_t)maxns * 16;  // at most 216 KB: cap <= 16384 within the limit above
     const int wpb = (int)std::max<size_t>(1, std::min<size_t>(4, (200u * 1024) / per_warp));
     const size_t smS = (size_t)wpb * per_warp;
-    if (smS > 200 * 1024) { free_res(); return IDBF_EUNSUPPORTED; }
     TRY_CUDA(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smS));
     k_sample<<<(unsigned)((nb + wpb - 1) / wpb), wpb * 32, smS, st>>>(dD, nb, cand_list, cand_coord, (int32_t*)samp.p,
                                                                     prm.sampling, cap, maxns);
@@ -970,9 +1060,11 @@ idbf_status Builder::run_step(int side, int s) {
     const size_t smQ = (size_t)maxns * 16 + (size_t)maxb * 12 + 16;
     if (smQ > 200 * 1024) { free_res(); return IDBF_EUNSUPPORTED; }
     if (df) {
-      TRY_CUDA(cudaFuncSetAttribute(k_qr_df<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smQ));
-      k_qr_df<256><<<(unsigned)nb, 256, smQ, st>>>(dD, (double2*)A.p, (int32_t*)pscr.p, (int32_t*)kbuf.p,
-                                                  (int32_t*)satbuf.p, prm.eps);
+      const bool big = maxb > 128;
+      auto qr = big ? k_qr_df<512, 4, 1> : k_qr_df<256, 4, 3>;
+      TRY_CUDA(cudaFuncSetAttribute(qr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smQ));
+      qr<<<(unsigned)nb, big ? 512 : 256, smQ, st>>>(dD, (double2*)A.p, (int32_t*)pscr.p, (int32_t*)kbuf.p,
+                                                     (int32_t*)satbuf.p, prm.eps);
     } else {
       TRY_CUDA(cudaFuncSetAttribute(k_qr<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smQ));
       k_qr<256><<<(unsigned)nb, 256, smQ, st>>>(dD, (double2*)A.p, (int32_t*)pscr.p, (int32_t*)kbuf.p,
