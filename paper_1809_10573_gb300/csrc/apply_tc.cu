@@ -29,6 +29,8 @@
 #include <algorithm>
 
 #include "idbf_internal.h"
+#include "level_kernels.cuh"
+#include "node_launch.h"
 
 namespace idbf {
 namespace tc {
@@ -453,6 +455,290 @@ __global__ void __launch_bounds__(NT + 32, 1)
 
 }  // namespace tc
 
+// ---------------------------------------------------------------------------------------------
+// The default split (three products) with warp-level MMAs (mma.sync m16n8k8, TF32 operands, FP32
+// accumulation), operands split in registers. The tcgen05 kernel above has to write every operand
+// to shared memory twice over (hi and lo, once per pass of 64 rows) and read it back for the MMAs,
+// and shared-memory bandwidth and that staging, not the tensor pipe, set its time (its pipe is 17 %
+// busy). Here a warp reads its factor entries from global memory and the vectors from a tile shared
+// by the CTA, splits both in registers and feeds them straight to the MMAs: the slower tensor path (302
+// TFLOP/s measured, against ~1000 for tcgen05 TF32) is kept busier than the fast one was.
+//
+// One CTA (NT threads) takes node j and RB = 8 NTL right-hand sides; a warp's task is 16 rows of a block times
+// the RB right-hand sides. Complex products are four real ones: Re += Mr Gr + (-Mi) Gi, Im += Mr Gi +
+// Mi Gr. The tensor core rounds every accumulation downwards a little, so the main products hi hi
+// run in chains of two k-steps (four accumulations) that are then added to a total in
+// round-to-nearest FP32; the two correction products, 2^-11 of the main ones, keep an accumulator
+// of their own. Columns past the block's end multiply zero entries with a row of zeros.
+// U levels: block 0 writes its term of every output position, block 1 adds its own after a barrier
+// (two terms: the order of the addition cannot change the sum).
+namespace wmma3 {
+__host__ __device__ constexpr int pitch(int RB) { return RB + 4; }  // rows 32 bytes apart modulo the banks
+__host__ __device__ constexpr int cols8(int cols) { return (cols + 7) & ~7; }
+inline size_t smem_bytes(int RB, int max_in, int max_cols, int max_rows) {
+  return (size_t)(max_in + 1) * pitch(RB) * sizeof(float2) + 2 * (size_t)(cols8(max_cols) + max_rows) * sizeof(int32_t);
+}
+
+__device__ __forceinline__ void mma(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+// d = a b
+__device__ __forceinline__ void mma0(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.f));
+}
+// x = hi + lo: hi is x rounded to TF32, ties away from zero, in integer arithmetic (the value of
+// cvt.rna.tf32.f32, whose conversion pipe is slower: S^h at N = 2^16, 256 vectors, tensor pipe 50 %);
+// the tensor core narrows lo
+__device__ __forceinline__ void split(float x, uint32_t& hi, uint32_t& lo) {
+  hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+  lo = __float_as_uint(x - __uint_as_float(hi));
+}
+
+template <int NTL, int NT>
+__global__ void __launch_bounds__(NT, 4)
+    k_level_mma(DevLevel d, const float2* __restrict__ mat, IO<float2> io, int max_in, int max_cols, int max_rows,
+                int nblk) {
+  constexpr int RB = 8 * NTL, PITCH = pitch(RB);
+  extern __shared__ __align__(16) unsigned char smem[];
+  node::next_may_begin();
+  float2* opd = (float2*)smem;                                   // [max_in + 1][PITCH], the last row zero
+  int32_t* kix = (int32_t*)(opd + (size_t)(max_in + 1) * PITCH);  // operand of every column, [2][cols8(max_cols)]
+  int32_t* aux = kix + 2 * cols8(max_cols);                       // V: operand passed through, U: position; per row
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  const int64_t j = blockIdx.x / (unsigned)nblk;
+  const int r0 = (int)(blockIdx.x % (unsigned)nblk) * RB, nr = min(RB, io.R - r0);
+  const int rowsv[2] = {d.rows[2 * j], d.rows[2 * j + 1]};
+  const int colsv[2] = {d.cols[2 * j], d.cols[2 * j + 1]};
+  const int64_t mov[2] = {d.moff[2 * j], d.moff[2 * j + 1]};
+  if (r0 == 0 && tid < 2)
+    node::prefetch_l2(mat + (tid ? mov[1] : mov[0]),
+                      (int64_t)(tid ? rowsv[1] : rowsv[0]) * (tid ? colsv[1] : colsv[0]) * (int64_t)sizeof(float2));
+  int l0, l1 = 0;
+  int64_t i0;
+  if (d.lev == 0) {
+    l0 = d.n0;
+    i0 = j * d.n0;
+  } else {
+    l0 = d.in_len[2 * j];
+    l1 = d.in_len[2 * j + 1];
+    i0 = d.in_off[2 * j];  // segments 2j and 2j + 1 are adjacent
+  }
+  int len0 = 0;
+  int64_t ob0 = 0, ob1 = 0;
+  if (d.lev < d.L) {
+    const int64_t s0 = out_seg_id(d, j, 0), s1 = out_seg_id(d, j, 1);
+    len0 = d.out_len[s0];
+    ob0 = d.out_off[s0];
+    ob1 = d.out_off[s1];
+  }
+  const int32_t* ixv[2] = {d.idx + d.ioff[2 * j], d.idx + d.ioff[2 * j + 1]};
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    int32_t* kc = kix + c * cols8(max_cols);
+    const int base = d.kind == KIND_U && c ? l0 : 0;
+    for (int k = tid; k < cols8(colsv[c]); k += NT)
+      kc[k] = k >= colsv[c] ? max_in * PITCH : (d.kind == KIND_V ? ixv[c][rowsv[c] + k] : base + k) * PITCH;
+    if (d.kind != KIND_S)
+      for (int r = tid; r < rowsv[c]; r += NT)
+        aux[c * max_rows + r] = d.kind == KIND_V ? ixv[c][r] * PITCH : ixv[c][(c ? l1 : l0) + r];
+  }
+  node::wait_for_inputs();
+  for (int i = tid; i < PITCH; i += NT) opd[(size_t)max_in * PITCH + i] = make_float2(0.f, 0.f);
+  if (d.lev == 0) {
+    for (int i = tid; i < l0 * RB; i += NT) {
+      const int rb = i / l0, e = i - rb * l0;
+      opd[e * PITCH + rb] = rb < nr ? io.x[i0 + e + (int64_t)(r0 + rb) * io.ldx] : make_float2(0.f, 0.f);
+    }
+  } else {
+    for (int i = tid; i < (l0 + l1) * RB; i += NT) {
+      const int e = i / RB, rb = i - e * RB;
+      opd[e * PITCH + rb] = rb < nr ? io.win[(i0 + e) * io.R + r0 + rb] : make_float2(0.f, 0.f);
+    }
+  }
+  __syncthreads();
+  // output element e of t = concat(out_0, out_1) (or of the leaf of y), right-hand side n of the block
+  auto out_ptr = [&](int e, int n) -> float2* {
+    if (d.lev == d.L) return io.y + (j * d.n0 + e) + (int64_t)(r0 + n) * io.ldy;
+    return io.wout + (e < len0 ? ob0 + e : ob1 + (e - len0)) * io.R + r0 + n;
+  };
+
+  auto task = [&](int c, int tile) {
+    const int rows = c ? rowsv[1] : rowsv[0], cols = c ? colsv[1] : colsv[0];
+    const int32_t* kc = kix + c * cols8(max_cols);
+    const int ra = tile * 16 + g, rb2 = ra + 8;
+    const float2* Ma = mat + (c ? mov[1] : mov[0]) + min(ra, rows - 1);
+    const int up = min(rb2, rows - 1) - min(ra, rows - 1);  // entries to the row 8 below
+    float tot[2][NTL][4], acc[2][NTL][4], cor[2][NTL][4];   // [re, im]
+#pragma unroll
+    for (int z = 0; z < 2; ++z)
+#pragma unroll
+      for (int n = 0; n < NTL; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) tot[z][n][e] = cor[z][n][e] = 0.f;
+    auto load = [&](int k0, float2 (&m)[4]) {  // entries (ra, k), (ra + 8, k), (ra, k + 4), (ra + 8, k + 4)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = k0 + t + 4 * h;
+        m[2 * h] = m[2 * h + 1] = make_float2(0.f, 0.f);
+        if (k < cols) {
+          m[2 * h] = __ldg(Ma + k * rows);
+          m[2 * h + 1] = __ldg(Ma + k * rows + up);
+        }
+      }
+    };
+    auto step = [&](int k0, const float2 (&m)[4], bool first) {
+      uint32_t rh[4], rl[4], ih[4], il[4], nh[4], nl[4];  // Mr, Mi, -Mi
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        split(m[e].x, rh[e], rl[e]);
+        split(m[e].y, ih[e], il[e]);
+        nh[e] = ih[e] ^ 0x80000000u;
+        nl[e] = il[e] ^ 0x80000000u;
+      }
+      const float2* g0 = opd + kc[k0 + t] + g;
+      const float2* g1 = opd + kc[k0 + t + 4] + g;
+#pragma unroll
+      for (int n = 0; n < NTL; ++n) {
+        const float2 a = g0[8 * n], b = g1[8 * n];
+        uint32_t grh[2], grl[2], gih[2], gil[2];
+        split(a.x, grh[0], grl[0]);
+        split(b.x, grh[1], grl[1]);
+        split(a.y, gih[0], gil[0]);
+        split(b.y, gih[1], gil[1]);
+        if (first) {
+          mma0(acc[0][n], rh, grh);
+          mma0(acc[1][n], rh, gih);
+        } else {
+          mma(acc[0][n], rh, grh);
+          mma(acc[1][n], rh, gih);
+        }
+        mma(cor[0][n], rh, grl);
+        mma(cor[1][n], rh, gil);
+        mma(acc[0][n], nh, gih);
+        mma(acc[1][n], ih, grh);
+        mma(cor[0][n], rl, grh);
+        mma(cor[1][n], rl, gih);
+        mma(cor[0][n], nh, gil);
+        mma(cor[1][n], ih, grl);
+        mma(cor[0][n], nl, gih);
+        mma(cor[1][n], il, grh);
+      }
+    };
+    float2 m0[4], m1[4];
+    load(0, m0);
+    load(8, m1);
+    for (int k0 = 0; k0 < cols; k0 += 16) {  // two k-steps: one chain of the main products
+      step(k0, m0, true);
+      load(k0 + 16, m0);
+      if (k0 + 8 < cols) step(k0 + 8, m1, false);
+      load(k0 + 24, m1);
+#pragma unroll
+      for (int z = 0; z < 2; ++z)
+#pragma unroll
+        for (int n = 0; n < NTL; ++n)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) tot[z][n][e] += acc[z][n][e];
+    }
+    // lane (g, t) holds rows ra, ra + 8 and right-hand sides 8 n + 2 t, + 1
+    // (a U level's block 1 loads block 0's terms of all its outputs before it stores the first)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = h ? rb2 : ra;
+      if (r >= rows) continue;
+      const int x = d.kind == KIND_S ? 0 : aux[c * max_rows + r];
+      float2 add[NTL][2];
+#pragma unroll
+      for (int n = 0; n < NTL; ++n)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int rb = 8 * n + 2 * t + q;
+          add[n][q] = make_float2(0.f, 0.f);
+          if (rb < nr) {
+            if (d.kind == KIND_V) add[n][q] = opd[x + rb];
+            else if (d.kind == KIND_U && c) add[n][q] = *out_ptr(x, rb);
+          }
+        }
+#pragma unroll
+      for (int n = 0; n < NTL; ++n)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int rb = 8 * n + 2 * t + q, e = 2 * h + q;
+          if (rb >= nr) continue;
+          *out_ptr(d.kind == KIND_U ? x : (c ? len0 : 0) + r, rb) =
+              make_float2(tot[0][n][e] + cor[0][n][e] + add[n][q].x, tot[1][n][e] + cor[1][n][e] + add[n][q].y);
+        }
+    }
+  };
+  const int t0 = (rowsv[0] + 15) / 16, t1 = (rowsv[1] + 15) / 16;
+  if (d.kind != KIND_U) {
+    for (int w = warp; w < t0 + t1; w += NT / 32) task(w >= t0, w >= t0 ? w - t0 : w);
+    return;
+  }
+  for (int c = 0; c < 2; ++c) {
+    for (int w = warp; w < (c ? t1 : t0); w += NT / 32) task(c, w);
+    const int lc = c ? l1 : l0;
+    // the inputs pass through to positions q_c, four at a time per thread (consecutive threads:
+    // consecutive right-hand sides of the workspace, consecutive positions of a column of y)
+    for (int i0p = tid; i0p < lc * RB; i0p += 4 * NT) {
+      float2* o[4];
+      float2 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0p + u * NT;
+        const int e = d.lev == d.L ? i % lc : i / RB, rb = d.lev == d.L ? i / lc : i % RB;
+        o[u] = nullptr;
+        if (i < lc * RB && rb < nr) {
+          o[u] = out_ptr(ixv[c][e], rb);
+          v[u] = opd[((c ? l0 : 0) + e) * PITCH + rb];
+          if (c) {
+            const float2 w = *o[u];
+            v[u] = make_float2(w.x + v[u].x, w.y + v[u].y);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (o[u]) *o[u] = v[u];
+    }
+    if (c == 0) __syncthreads();
+  }
+}
+
+template <int NTL, int NT>
+static cudaError_t launch(Plan* p, int l, const IO<float2>& io, bool after, cudaStream_t st) {
+  const LevelInfo& li = p->lv[l];
+  const size_t sm = smem_bytes(8 * NTL, li.max_in, li.max_cols, li.max_rows);
+  const cudaError_t e = cudaFuncSetAttribute(k_level_mma<NTL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const int nblk = (io.R + 8 * NTL - 1) / (8 * NTL);
+  return node::launch_after(k_level_mma<NTL, NT>, after, (int64_t)p->m * nblk, NT, sm, st, p->level(l),
+                            (const float2*)p->lmat[IDBF_STORE_C64][l], io, li.max_in, li.max_cols, li.max_rows, nblk);
+}
+// 32 right-hand sides and three warps per CTA where blocks are short (at most 64 rows: four 16-row
+// tiles), 16 and four warps where they are tall, whose operands would leave one CTA per SM else; 8
+// where the level has too few nodes to fill the GPU or the operands do not fit. 256 vectors: DFT N =
+// 40960 2.76 ms with the first, 3.20 with the second; FIO N = 2^16 11.5 and 9.07 ms. False if not even
+// eight right-hand sides fit.
+static bool level(Plan* p, int l, const IO<float2>& io, bool after, cudaStream_t st, cudaError_t* e) {
+  const LevelInfo& li = p->lv[l];
+  auto ok = [&](int rb) {
+    return smem_bytes(rb, li.max_in, li.max_cols, li.max_rows) <= 220 * 1024 && io.R > rb / 2 &&
+           (int64_t)p->m * ((io.R + rb - 1) / rb) >= 2 * node::num_sms();
+  };
+  if (li.max_rows <= 64 && ok(32)) *e = launch<4, 96>(p, l, io, after, st);
+  else if (ok(16)) *e = launch<2, 128>(p, l, io, after, st);
+  else if (smem_bytes(8, li.max_in, li.max_cols, li.max_rows) <= 220 * 1024) *e = launch<1, 128>(p, l, io, after, st);
+  else return false;
+  return true;
+}
+}  // namespace wmma3
+
 // the 3xTF32 apply of all levels (forward); returns EUNSUPPORTED if a block is too large. With
 // wide_middle the middle factor S^h runs on the CUDA cores in FP64 or double-float instead.
 idbf_status apply_tf32x3(Plan* p, const void* x, void* y, int64_t R, int64_t ld, cudaStream_t st, bool wide_middle) {
@@ -476,6 +762,16 @@ idbf_status apply_tf32x3(Plan* p, const void* x, void* y, int64_t R, int64_t ld,
       const idbf_status s = apply_middle_wide(p, win, wout, R, st);
       if (s != IDBF_OK) return s;
       continue;
+    }
+    if (p->tc_split_mode == 0) {
+      IO<float2> io;
+      io.x = (const float2*)x; io.ldx = ld; io.y = (float2*)y; io.ldy = ld; io.R = (int)R;
+      io.win = win; io.wout = wout;
+      cudaError_t e = cudaSuccess;
+      if (wmma3::level(p, l, io, l > 0, st, &e)) {
+        IDBF_CUDA_TRY(e);
+        continue;
+      }
     }
     const unsigned ctas = (unsigned)std::min<int64_t>(p->m, sms);
     tc::k_level_tc<<<ctas, tc::NT + 32, tc::SMEM, st>>>(d, (const float2*)p->lmat[IDBF_STORE_C64][l], (const float2*)x, ld,

@@ -66,3 +66,20 @@ def test_unsorted_redundant_lists_are_reordered_with_their_blocks(kind):
     xd = torch.from_numpy(X).cuda()
     assert rel(plan.apply(xd).cpu().numpy(), idbf.apply(c["F"], X)) < 1e-12
     assert rel(plan.apply_adjoint(xd).cpu().numpy(), idbf.apply_adjoint(c["F"], X)) < 1e-12
+
+
+@pytest.mark.parametrize("case", ["dft_1024", "fio_base_4096", "fio_base_8192_oddL"])
+def test_split_precision_widths_and_split_modes(case):
+    """3xTF32: every width of the warp-level MMA kernel, ragged last tiles, and the two split modes that
+    run the tcgen05 kernel. FP32-class results: the 2e-5 bar of the FP32 apply."""
+    from paper_1809_10573_gb300 import _lib
+    c = oracle_case(case)
+    plan = P.Plan.import_factors(c["ex"], storage=P.STORE_C64)
+    for R in (1, 7, 8, 9, 17, 33, 100):
+        X = inputs.complex_gaussian(c["N"], R, seed=R)
+        xd = torch.from_numpy(X.astype(np.complex64)).cuda()
+        ref = idbf.apply(c["F"], X)
+        for mode in (0, 1, 2) if R in (1, 33) else (0,):
+            assert _lib.lib().idbf_set_tc_split(plan._h, mode) == _lib.OK
+            assert rel(plan.apply(xd, mode=P.MODE_TF32X3).cpu().numpy(), ref) < 2e-5, (R, mode)
+    plan.sync_status()
