@@ -239,10 +239,14 @@ void at_level_width(int w, bool few, F f) {
     if (w > 1) IDBF_W(2, 1, 8, 256, 3);
     IDBF_W(1, 1, 6, 256, 4);
   } else if constexpr (std::is_same<P, FP64P>::value) {
-    if (w > 4) IDBF_W(8, 1, 2, 256, 2);
-    if (w > 2) IDBF_W(4, 1, 4, 256, 2);
+    if (w > 7) IDBF_W(8, 1, 2, 256, 2);
+    if (w > 6) IDBF_W(7, 1, 2, 256, 2);
+    if (w > 5) IDBF_W(6, 1, 2, 256, 2);
+    if (w > 4) IDBF_W(5, 1, 4, 256, 2);
+    if (w > 3) IDBF_W(4, 1, 4, 256, 2);
+    if (w > 2) IDBF_W(3, 1, 4, 256, 2);
     if (w > 1) IDBF_W(2, 1, 4, 256, 2);
-    IDBF_W(1, 1, 4, 256, 3);
+    IDBF_W(1, 1, 8, 256, 3);
   } else {
     if (w > 3) IDBF_W(4, 1, 2, 256, 2);
     if (w > 2) IDBF_W(3, 1, 2, 256, 2);
@@ -333,19 +337,24 @@ int persistent_threads(const idbf_batch_s* b) { return bat::kTiles[b->tile].nt ?
 template <class P>
 idbf_status plan_levels(idbf_batch_s* b, std::vector<bat::LevelItem>& items) {
   const int cap = std::min(b->rb, bat::pass_rb<P>());
+  constexpr bool kFp64 = std::is_same<P, FP64P>::value;
   std::vector<int> widths;  // instance widths in use
   std::vector<int> cls(b->nops, 0);
   int maxL = 0;
   for (int o = 0; o < b->nops; ++o) {
     if (b->sep[o]) continue;
     int w = 0;
-    bat::at_level_width<P>(node::even_block(b->R[o], cap), b->rb > 8, [&](auto rb, auto, auto, auto, auto) { w = decltype(rb)::value; });
+    const int want = kFp64 ? node::fitting_block(b->R[o]) : node::even_block(b->R[o], cap);
+    bat::at_level_width<P>(want, b->rb > 8, [&](auto rb, auto, auto, auto, auto) { w = decltype(rb)::value; });
     cls[o] = w;
     if (std::find(widths.begin(), widths.end(), w) == widths.end()) widths.push_back(w);
     maxL = std::max(maxL, b->plans[o]->p.L);
   }
   std::sort(widths.begin(), widths.end(), [](int x, int y) { return x > y; });
-  // few nodes on a level over the whole batch: cut them as the single apply does
+  // few nodes on a level over the whole batch: cut them as the single apply does. FP64 counts each
+  // operator's nodes alone: its chains share one slow pipe and end together only in small items (five
+  // operators of N = 1024..8192, 18 vectors in all: 483 us against 783; double-float, whose chains
+  // fill one another's gaps, 316 against 421, complex64 154 against 199 the other way round)
   std::vector<int64_t> nodes(maxL + 1, 0);
   for (int o = 0; o < b->nops; ++o)
     for (int l = 0; !b->sep[o] && l <= b->plans[o]->p.L; ++l)
@@ -357,7 +366,7 @@ idbf_status plan_levels(idbf_batch_s* b, std::vector<bat::LevelItem>& items) {
         const Plan& p = b->plans[o]->p;
         if (b->sep[o] || cls[o] != w || l > p.L) continue;
         const LevelInfo& li = p.lv[l];
-        const int nsl = node::slices(nodes[l], node::fwd_span(li), 4);
+        const int nsl = node::slices(kFp64 ? (int64_t)p.m * ((b->R[o] + w - 1) / w) : nodes[l], node::fwd_span(li), 4);
         bat::at_level_width<P>(w, b->rb > 8, [&](auto rb, auto tr, auto, auto ntl, auto) {
           q.smem = std::max(q.smem, node::fwd_smem<P, decltype(rb)::value>(li.max_in, li.max_out, li.max_rows, li.max_cols,
                                                                             li.max_rows_pair, li.kind == KIND_U));
