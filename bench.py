@@ -503,7 +503,7 @@ def _gpu_headline(args, rank, world, np, torch, P, inputs, team):
                 "peak_kind": peak_kind,
                 "traffic": (ratio * ab / nlaunch) if ratio is not None else None,
                 "kernel": "double-float level kernels (per level or fused level pair the autotuned "
-                          "k_level_stream ring, k_level_warp or k_level_fwd; every launch of the timed "
+                          "k_level_stream ring, k_level_warp or k_node_fwd; every launch of the timed "
                           "region is one of them)",
                 "algorithmic_bytes_per_launch": ab / nlaunch, "launches_per_apply": nlaunch}
     # end to end through the C call: pinned host x -> device, apply, device -> host y

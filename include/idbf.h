@@ -186,7 +186,7 @@ typedef struct {
  * with no columns contribute zeros. Plans with leaves of uneven size run the per-node level
  * kernels (FP64, double-float and FP32, any number of right-hand sides, forward and adjoint,
  * idbf_apply_noalloc) and, for one right-hand side, the streaming kernels and fused level
- * pairs; the warp-per-node, register-tiled and tensor-core kernels, batches and checkpoints
+ * pairs; the warp-per-node and tensor-core kernels, batches and checkpoints
  * refuse them (EUNSUPPORTED; an apply then uses the per-node kernel). Offsets that are all equal
  * are the uniform case. Synchronous. */
 idbf_status idbf_import_factors(const idbf_host_factors* f, int32_t storage, void* stream,
@@ -197,7 +197,7 @@ idbf_status idbf_import_factors(const idbf_host_factors* f, int32_t storage, voi
 #define IDBF_MODE_DF64 1   /* DF64 storage, complex128 vectors, double-float (FP32 pair) arithmetic */
 #define IDBF_MODE_FP32 2   /* C64 storage, complex64 vectors, FP32 FMA */
 #define IDBF_MODE_TF32X3 3 /* C64 storage, complex64 vectors, 3xTF32 tensor-core block products
-                           * (tcgen05, FP32 accumulation; forward only; blocks of <= 256 rows) */
+                           * (FP32 accumulation; forward only; blocks of <= 256 rows) */
 #define IDBF_MODE_TF32X3_S64 4 /* as IDBF_MODE_TF32X3 on every level but the middle factor S^h
                                * (Eq. finishIDBF), whose products and sums run on the CUDA cores
                                * in double-float (DF64 storage of that level, preferred) or FP64
@@ -225,7 +225,7 @@ idbf_status idbf_apply_adjoint(idbf_plan plan, const void* x, void* y, int64_t n
  * has to know its full device footprint when the library loads.
  *   Scope: forward apply only, modes IDBF_MODE_FP64, IDBF_MODE_DF64 and IDBF_MODE_FP32 (same
  *   arguments as idbf_apply). Every level runs the per-node level kernel (variant 0 of
- *   idbf_autotune), not the autotuned streaming or register-tiled kernels, so a call is slower
+ *   idbf_autotune), not the autotuned streaming kernels, so a call is slower
  *   than idbf_apply and its double-float / FP32 results differ from idbf_apply's in the summation
  *   order only: they agree within that mode's rounding error (FP64: to ~1e-15 relative).
  *   Workspace: a fixed array of IDBF_NOALLOC_SCRATCH_BYTES compiled into the library. Every GPU
@@ -277,7 +277,7 @@ idbf_status idbf_set_level_variants(idbf_plan plan, int32_t mode, const int32_t*
 
 /* idbf_set_tc_split - operand splitting of the 3xTF32 tensor-core mode: 0 = x_hi + x_lo with
  * x_hi = tf32(x) and three products (default), 1 = x_lo also rounded to TF32, 2 = four products
- * (adds x_lo y_lo). */
+ * (adds x_lo y_lo). Mode 0 runs the warp-level MMA kernel, modes 1 and 2 the tcgen05 one. */
 idbf_status idbf_set_tc_split(idbf_plan plan, int32_t split_mode);
 
 /* idbf_reserve - allocate the apply workspace for up to nrhs right-hand sides now. */
