@@ -28,6 +28,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "batch_items.cuh"
 #include "idbf_internal.h"
 #include "node_kernels.cuh"
 #include "node_launch.h"
@@ -73,32 +74,6 @@ struct Tile {
 constexpr Tile kTiles[] = {{1, 256, false}, {4, 256, false}, {8, 128, false}, {8, 0, false},
                            {8, 256, true},  {16, 0, true},   {32, 256, true}, {16, 128, true}};
 constexpr int kNumTiles = 8;
-template <class P>
-__host__ __device__ constexpr int max_rb() {
-  return std::is_same<P, FP32P>::value ? 32 : std::is_same<P, FP64P>::value ? 16 : 8;
-}
-// right-hand sides that one pass of the body holds in registers
-template <class P>
-__host__ __device__ constexpr int pass_rb() {
-  return std::is_same<P, DF64P>::value ? 4 : 8;
-}
-
-// The body's width for an item of at most w right-hand sides in one pass: calls f with it.
-template <class P, class F>
-__host__ __device__ __forceinline__ void at_width(int w, F f) {
-  using std::integral_constant;
-  if constexpr (std::is_same<P, FP32P>::value) {
-    if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 2>(), integral_constant<int, 2>());
-  } else if constexpr (std::is_same<P, FP64P>::value) {
-    if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 1>(), integral_constant<int, 2>());
-  } else {
-    if (w == 3) return f(integral_constant<int, 3>(), integral_constant<int, 1>(), integral_constant<int, 2>());
-  }
-  if (w > 2) return f(integral_constant<int, 4>(), integral_constant<int, 1>(), integral_constant<int, 2>());
-  if (w > 1) return f(integral_constant<int, 2>(), integral_constant<int, 1>(), integral_constant<int, 4>());
-  return f(integral_constant<int, 1>(), integral_constant<int, 1>(), integral_constant<int, 4>());
-}
-
 // One node at one width. Not inlined: the widths of a precision share the kernel's registers.
 template <class P, int RB, int TR, int U>
 __device__ __noinline__ void batch_node(const OpLevel& ol, const IO<typename P::vec_t>& io, int64_t j, int r, int r1,
@@ -169,7 +144,7 @@ __global__ void __launch_bounds__(NTMAX, 2) k_batch(const OpDesc* __restrict__ o
     __syncthreads();
     if (!sfail) {
       const int r1 = min(od.R, w.r0 + od.width);
-      const int passes = (r1 - w.r0 + pass_rb<P>() - 1) / pass_rb<P>(), pw = (r1 - w.r0 + passes - 1) / passes;
+      const int pw = pass_width<P>(r1 - w.r0);
       for (int n = 0; n < w.nodes; ++n)
         for (int r = w.r0; r < r1; r += pw) {
           if (n || r != w.r0) __syncthreads();
@@ -254,16 +229,6 @@ void at_level_width(int w, bool few, F f) {
     IDBF_W(1, 1, 4, 256, 3);
   }
 #undef IDBF_W
-}
-
-template <class P>
-size_t node_smem(const LevelInfo& li, int pw) {
-  size_t n = 0;
-  at_width<P>(pw, [&](auto rb, auto, auto) {
-    n = node::fwd_smem<P, decltype(rb)::value>(li.max_in, li.max_out, li.max_rows, li.max_cols, li.max_rows_pair,
-                                               li.kind == KIND_U);
-  });
-  return n;
 }
 
 }  // namespace bat
@@ -454,8 +419,7 @@ size_t smem_for(idbf_batch_s* b) {
   size_t sm = 0;
   for (int o = 0; o < b->nops; ++o) {
     if (b->sep[o]) continue;
-    const int w = b->h_ops[o].width, passes = (w + bat::pass_rb<P>() - 1) / bat::pass_rb<P>();
-    for (const LevelInfo& li : b->plans[o]->p.lv) sm = std::max(sm, bat::node_smem<P>(li, (w + passes - 1) / passes));
+    for (const LevelInfo& li : b->plans[o]->p.lv) sm = std::max(sm, bat::items_smem<P>(li, b->R[o], b->h_ops[o].width));
   }
   return sm;
 }
