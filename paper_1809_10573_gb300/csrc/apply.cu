@@ -678,7 +678,7 @@ static idbf_status launch_stream(Plan* p, int l, bool pair, bool bulk, bool spli
   const typename P::mat_t* mat = (const typename P::mat_t*)p->lmat[fmt_of<P>()][l];
   const typename P::mat_t* mat1 = (const typename P::mat_t*)p->lmat[fmt_of<P>()][pair ? l + 1 : l];
   auto go = [&](auto kern) -> idbf_status {
-    IDBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)geo.total));
+    IDBF_CUDA_TRY(allow_smem(kern, cap));
     IDBF_CUDA_TRY(node::launch_after(kern, after, ctas, RG::NTHREADS, geo.total, st, d, mat, d1, mat1, io, max_in, max_out,
                                      max_cols_pair, mid_elems, use_bulk, p->d_status, p->wait_limit_ns,
                                      p->producer_enabled));
@@ -704,13 +704,14 @@ static idbf_status launch_warp_node(Plan* p, int l, IO<typename P::vec_t> io, cu
   const LevelInfo& li = p->lv[l];
   const int gcap = std::max(li.max_cols, li.max_in);
   const size_t per = warp_node_smem<P>(li.max_in, gcap, li.max_out);
-  if (li.max_rows > 128 || per > 24 * 1024) return IDBF_EUNSUPPORTED;
+  constexpr size_t kPerWarpCap = 24 * 1024;
+  if (li.max_rows > 128 || per > kPerWarpCap) return IDBF_EUNSUPPORTED;
   const size_t sm = per * kWarpNodeWarps;
   const DevLevel d = p->level(l);
   const typename P::mat_t* mat = (const typename P::mat_t*)p->lmat[fmt][l];
   const unsigned grid = (unsigned)((p->m + kWarpNodeWarps - 1) / kWarpNodeWarps);
   auto go = [&](auto kern) -> idbf_status {
-    if (sm > 48 * 1024) IDBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024) IDBF_CUDA_TRY(allow_smem(kern, kPerWarpCap * kWarpNodeWarps));
     kern<<<grid, kWarpNodeWarps * 32, sm, st>>>(d, mat, io, li.max_in, gcap, li.max_out);
     IDBF_CUDA_TRY(cudaGetLastError());
     return IDBF_OK;

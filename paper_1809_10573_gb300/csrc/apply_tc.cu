@@ -475,6 +475,7 @@ __global__ void __launch_bounds__(NT + 32, 1)
 namespace wmma3 {
 __host__ __device__ constexpr int pitch(int RB) { return RB + 4; }  // rows 32 bytes apart modulo the banks
 __host__ __device__ constexpr int cols8(int cols) { return (cols + 7) & ~7; }
+constexpr size_t kSmemCap = 220 * 1024;
 inline size_t smem_bytes(int RB, int max_in, int max_cols, int max_rows) {
   return (size_t)(max_in + 1) * pitch(RB) * sizeof(float2) + 2 * (size_t)(cols8(max_cols) + max_rows) * sizeof(int32_t);
 }
@@ -714,7 +715,7 @@ template <int NTL, int NT>
 static cudaError_t launch(Plan* p, int l, const IO<float2>& io, bool after, cudaStream_t st) {
   const LevelInfo& li = p->lv[l];
   const size_t sm = smem_bytes(8 * NTL, li.max_in, li.max_cols, li.max_rows);
-  const cudaError_t e = cudaFuncSetAttribute(k_level_mma<NTL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const cudaError_t e = sm > 48 * 1024 ? allow_smem(k_level_mma<NTL, NT>, kSmemCap) : cudaSuccess;
   if (e != cudaSuccess) return e;
   const int nblk = (io.R + 8 * NTL - 1) / (8 * NTL);
   return node::launch_after(k_level_mma<NTL, NT>, after, (int64_t)p->m * nblk, NT, sm, st, p->level(l),
@@ -728,12 +729,12 @@ static cudaError_t launch(Plan* p, int l, const IO<float2>& io, bool after, cuda
 static bool level(Plan* p, int l, const IO<float2>& io, bool after, cudaStream_t st, cudaError_t* e) {
   const LevelInfo& li = p->lv[l];
   auto ok = [&](int rb) {
-    return smem_bytes(rb, li.max_in, li.max_cols, li.max_rows) <= 220 * 1024 && io.R > rb / 2 &&
+    return smem_bytes(rb, li.max_in, li.max_cols, li.max_rows) <= kSmemCap && io.R > rb / 2 &&
            (int64_t)p->m * ((io.R + rb - 1) / rb) >= 2 * node::num_sms();
   };
   if (li.max_rows <= 64 && ok(32)) *e = launch<4, 96>(p, l, io, after, st);
   else if (ok(16)) *e = launch<2, 128>(p, l, io, after, st);
-  else if (smem_bytes(8, li.max_in, li.max_cols, li.max_rows) <= 220 * 1024) *e = launch<1, 128>(p, l, io, after, st);
+  else if (smem_bytes(8, li.max_in, li.max_cols, li.max_rows) <= kSmemCap) *e = launch<1, 128>(p, l, io, after, st);
   else return false;
   return true;
 }
@@ -747,7 +748,7 @@ idbf_status apply_tf32x3(Plan* p, const void* x, void* y, int64_t R, int64_t ld,
     if (wide_middle && l == p->hV) continue;
     if (p->lv[l].max_rows > tc::MAXROWS || p->lv[l].max_cols > tc::GIXCAP) return IDBF_EUNSUPPORTED;
   }
-  IDBF_CUDA_TRY(cudaFuncSetAttribute(tc::k_level_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::SMEM));
+  IDBF_CUDA_TRY(allow_smem(tc::k_level_tc, tc::SMEM));
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -61,6 +61,7 @@ __device__ __forceinline__ uint64_t gtimer() {
 }
 
 constexpr int NTMAX = 256;
+constexpr size_t kSmemCap = 200 * 1024;  // per CTA
 
 // Tiles: right-hand sides per work item (rb; above the body's width in several passes), threads per
 // CTA of the persistent launch, or 0 for level launches, one chain of launches per width of the
@@ -345,7 +346,7 @@ idbf_status plan_levels(idbf_batch_s* b, std::vector<bat::LevelItem>& items) {
               items.push_back({o, n0, std::min(npi, p.m - n0), (int)r0, sl, nsl});
       }
       q.count = (int)items.size() - q.first;
-      if (q.smem > 200 * 1024) return IDBF_EUNSUPPORTED;
+      if (q.smem > bat::kSmemCap) return IDBF_EUNSUPPORTED;
       if (q.count > 0) b->level_launches.push_back(q);
     }
   return IDBF_OK;
@@ -386,7 +387,7 @@ idbf_status launch_levels(idbf_batch_s* b, cudaStream_t st) {
     bat::at_level_width<P>(q.width, b->rb > 8, [&](auto rb, auto tr, auto u, auto ntl, auto mb) {
       auto kern = bat::k_batch_level<P, decltype(rb)::value, decltype(tr)::value, decltype(u)::value, decltype(ntl)::value,
                                      decltype(mb)::value>;
-      if (q.smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if (q.smem > 48 * 1024) e = allow_smem(kern, bat::kSmemCap);
       if (e == cudaSuccess)
         e = node::launch_after(kern, !first, (int64_t)q.count, q.nt, q.smem, cs, (const bat::LevelItem*)b->d_litems + q.first,
                                (const bat::OpDesc*)b->d_ops, (const bat::OpLevel*)b->d_lv, q.level, xs, ys, lds);
@@ -401,7 +402,7 @@ idbf_status launch_levels(idbf_batch_s* b, cudaStream_t st) {
 template <class P>
 idbf_status launch_batch(idbf_batch_s* b, cudaStream_t st) {
   if (b->smem > 48 * 1024)
-    IDBF_CUDA_TRY(cudaFuncSetAttribute(bat::k_batch<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
+    IDBF_CUDA_TRY(allow_smem(bat::k_batch<P>, bat::kSmemCap));
   const void* const* xs = (const void* const*)b->d_ptrs;
   void* const* ys = (void* const*)(b->d_ptrs + b->nops);
   const int64_t* lds = (const int64_t*)(b->d_ptrs + 2 * b->nops);
@@ -428,7 +429,7 @@ template <class P>
 int occupancy(idbf_batch_s* b) {
   int n = 0;
   if (b->smem > 48 * 1024)
-    cudaFuncSetAttribute(bat::k_batch<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
+    allow_smem(bat::k_batch<P>, bat::kSmemCap);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bat::k_batch<P>, persistent_threads(b), b->smem);
   return std::max(n, 1);
 }
@@ -525,7 +526,7 @@ idbf_status layout(idbf_batch_s* b) {
     return IDBF_OK;
   }
   b->smem = IDBF_BATCH_DISPATCH(smem_for, b);
-  if (b->smem == 0 || b->smem > 200 * 1024) return IDBF_EUNSUPPORTED;
+  if (b->smem == 0 || b->smem > bat::kSmemCap) return IDBF_EUNSUPPORTED;
   const int occ = IDBF_BATCH_DISPATCH(occupancy, b);
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);

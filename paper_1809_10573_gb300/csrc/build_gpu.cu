@@ -1048,7 +1048,7 @@ idbf_status Builder::run_step(int side, int s) {
     const size_t per_warp = tables + (size_t)maxns * 16;  // at most 216 KB: cap <= 16384 within the limit above
     const int wpb = (int)std::max<size_t>(1, std::min<size_t>(4, (200u * 1024) / per_warp));
     const size_t smS = (size_t)wpb * per_warp;
-    TRY_CUDA(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smS));
+    TRY_CUDA(allow_smem(k_sample, 216 * 1024));
     k_sample<<<(unsigned)((nb + wpb - 1) / wpb), wpb * 32, smS, st>>>(dD, nb, cand_list, cand_coord, (int32_t*)samp.p,
                                                                     prm.sampling, cap, maxns);
     TRY_CUDA(cudaGetLastError());
@@ -1062,11 +1062,11 @@ idbf_status Builder::run_step(int side, int s) {
     if (df) {
       const bool big = maxb > 128;
       auto qr = big ? k_qr_df<512, 4, 1> : k_qr_df<256, 4, 3>;
-      TRY_CUDA(cudaFuncSetAttribute(qr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smQ));
+      TRY_CUDA(allow_smem(qr, 200 * 1024));
       qr<<<(unsigned)nb, big ? 512 : 256, smQ, st>>>(dD, (double2*)A.p, (int32_t*)pscr.p, (int32_t*)kbuf.p,
                                                      (int32_t*)satbuf.p, prm.eps);
     } else {
-      TRY_CUDA(cudaFuncSetAttribute(k_qr<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smQ));
+      TRY_CUDA(allow_smem(k_qr<256>, 200 * 1024));
       k_qr<256><<<(unsigned)nb, 256, smQ, st>>>(dD, (double2*)A.p, (int32_t*)pscr.p, (int32_t*)kbuf.p,
                                                (int32_t*)satbuf.p, prm.eps);
     }
@@ -1099,7 +1099,7 @@ idbf_status Builder::run_step(int side, int s) {
     auto emit = df ? k_emit<true> : k_emit<false>;
     const size_t smE = (size_t)maxb * 8;
     if (smE > 200 * 1024) { free_res(); return IDBF_EUNSUPPORTED; }  // never above the QR's own need
-    if (smE > 48 * 1024) TRY_CUDA(cudaFuncSetAttribute(emit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smE));
+    if (smE > 48 * 1024) TRY_CUDA(allow_smem(emit, 200 * 1024));
     emit<<<(unsigned)nb, 256, smE, st>>>(dD, (EmitDesc*)emits.p, (double2*)A.p, (int32_t*)pscr.p,
                                                     (int32_t*)blist.p, (int32_t*)kbuf.p, (double2*)res.back().T,
                                                     res.back().I, res.back().S, side);

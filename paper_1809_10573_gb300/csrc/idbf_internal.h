@@ -117,6 +117,15 @@ void set_cuda_error(cudaError_t e);
     }                                             \
   } while (0)
 
+// Lets kernel `kern` take up to `limit` bytes of dynamic shared memory per CTA. The limit belongs to the
+// kernel in its whole context, not to a launch: it is the same constant at every launch of one kernel,
+// because a limit of the launch's own size would be lowered by another host thread (another plan, a
+// smaller level) between this thread's call and its launch.
+template <class K>
+cudaError_t allow_smem(K kern, size_t limit) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
+}
+
 // Level infos and segment offsets from the host structure (h_rows, h_cols, h_seg_len).
 idbf_status finalize_structure(Plan* p);
 // Copy the host structure (block shapes and offsets, segment lengths and offsets) to the device.

@@ -50,7 +50,7 @@ static idbf_status fwd_launch(Plan* p, int l, const void* mat, const IO<typename
   const int nsl = slices((int64_t)p->m * nblk, fwd_span(li), 4);
   const int nt = fwd_threads(li, TR, nsl, NTMAX);
   auto go = [&](auto kern) -> idbf_status {
-    if (sm > 48 * 1024) IDBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024) IDBF_CUDA_TRY(allow_smem(kern, kSmemCap));
     IDBF_CUDA_TRY(launch_after(kern, after, (int64_t)p->m * nsl * nblk, nt, sm, st, p->level(l),
                                (const typename P::mat_t*)mat, io, li.max_in, li.max_out, li.max_rows, li.max_cols,
                                li.max_rows_pair, nblk, nsl));
@@ -73,7 +73,7 @@ static idbf_status adj_launch(Plan* p, int l, const void* mat, const IO<typename
   int nt = ((cols + tile - 1) / tile + 2) / 3 * 32;
   nt = std::max(nsl > 1 ? NTMAX : 64, std::min(NTMAX, nt));
   auto go = [&](auto kern) -> idbf_status {
-    if (sm > 48 * 1024) IDBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > 48 * 1024) IDBF_CUDA_TRY(allow_smem(kern, kSmemCap));
     IDBF_CUDA_TRY(launch_after(kern, after, (int64_t)p->m * nsl * nblk, nt, sm, st, p->level(l),
                                (const typename P::mat_t*)mat, io, li.max_in, li.max_out, li.max_rows, li.max_cols_pair,
                                nblk, nsl));
