@@ -208,8 +208,8 @@ void at_level_width(int w, bool few, F f) {
   return f(std::integral_constant<int, RB>(), std::integral_constant<int, TR>(), std::integral_constant<int, U>(), \
            std::integral_constant<int, NT>(), std::integral_constant<int, MB>())
   if constexpr (std::is_same<P, FP32P>::value) {
-    if (w > 6 && few) IDBF_W(8, 2, 2, 256, 2);
-    if (w > 6) IDBF_W(8, 2, 4, 192, 4);
+    if (w > 6 && few) IDBF_W(8, 1, 4, 256, 2);
+    if (w > 6) IDBF_W(8, 1, 4, 256, 3);
     if (w > 4) IDBF_W(6, 1, 4, 256, 3);
     if (w > 2) IDBF_W(4, 1, 4, 256, 3);
     if (w > 1) IDBF_W(2, 1, 8, 256, 3);

@@ -27,7 +27,7 @@ template <class P, class F>
 __host__ __device__ __forceinline__ void at_width(int w, F f) {
   using std::integral_constant;
   if constexpr (std::is_same<P, FP32P>::value) {
-    if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 2>(), integral_constant<int, 2>());
+    if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 1>(), integral_constant<int, 4>());
   } else if constexpr (std::is_same<P, FP64P>::value) {
     if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 1>(), integral_constant<int, 2>());
   } else {

@@ -38,6 +38,11 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 
 // ---------------------------------------------------------------------------------------------
 // arithmetic policies
@@ -46,7 +51,7 @@ struct FP64P {
   using vec_t = double2;
   using gv_t = double2;
   struct acc_t { double re, im; };
-  static constexpr int CHUNK = 16, ADJ_CHUNK = 16;
+  static constexpr int CHUNK = 16;
   __device__ static __forceinline__ mat_t ld(const mat_t* p) { return __ldcs(p); }
   __device__ static __forceinline__ gv_t cvt(vec_t v) { return v; }
   __device__ static __forceinline__ void init(acc_t& a) { a.re = 0.0; a.im = 0.0; }
@@ -87,11 +92,13 @@ struct FP32P {
   using mat_t = float2;
   using vec_t = float2;
   using gv_t = float2;
-  struct acc_t { float re, im; };
-  static constexpr int CHUNK = 16, ADJ_CHUNK = 16;
+  // (re, im) takes the running terms; flush folds it into the total (tr, ti), so that a long sum rounds
+  // like a sum of short ones
+  struct acc_t { float re, im, tr, ti; };
+  static constexpr int CHUNK = 16;
   __device__ static __forceinline__ mat_t ld(const mat_t* p) { return __ldcs(p); }
   __device__ static __forceinline__ gv_t cvt(vec_t v) { return v; }
-  __device__ static __forceinline__ void init(acc_t& a) { a.re = 0.f; a.im = 0.f; }
+  __device__ static __forceinline__ void init(acc_t& a) { a.re = a.im = a.tr = a.ti = 0.f; }
   __device__ static __forceinline__ void mac(acc_t& a, const mat_t& m, const gv_t& g) {
     a.re = fmaf(m.x, g.x, a.re);
     a.re = fmaf(-m.y, g.y, a.re);
@@ -104,8 +111,12 @@ struct FP32P {
     a.im = fmaf(m.x, g.y, a.im);
     a.im = fmaf(-m.y, g.x, a.im);
   }
-  __device__ static __forceinline__ void flush(acc_t&) {}
-  __device__ static __forceinline__ vec_t fin(const acc_t& a) { return make_float2(a.re, a.im); }
+  __device__ static __forceinline__ void flush(acc_t& a) {
+    a.tr += a.re;
+    a.ti += a.im;
+    a.re = a.im = 0.f;
+  }
+  __device__ static __forceinline__ vec_t fin(const acc_t& a) { return make_float2(a.tr, a.ti); }
   __device__ static __forceinline__ void warp_sum(acc_t& a) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -116,13 +127,13 @@ struct FP32P {
   __device__ static __forceinline__ vec_t add(vec_t a, vec_t b) { return make_float2(a.x + b.x, a.y + b.y); }
   __device__ static __forceinline__ vec_t zero() { return make_float2(0.f, 0.f); }
   using part_t = float2;
-  __device__ static __forceinline__ part_t part(const acc_t& a) { return make_float2(a.re, a.im); }
+  __device__ static __forceinline__ part_t part(const acc_t& a) { return make_float2(a.tr, a.ti); }
   // a partial sum plus one of lane (lane xor o)
   __device__ static __forceinline__ part_t add_lane(const part_t& keep, const part_t& send, int o) {
     return make_float2(keep.x + __shfl_xor_sync(0xffffffffu, send.x, o), keep.y + __shfl_xor_sync(0xffffffffu, send.y, o));
   }
   __device__ static __forceinline__ vec_t fin_part(const part_t& p) { return p; }
-  __device__ static __forceinline__ void combine(acc_t& a, const part_t& b) { a.re += b.x; a.im += b.y; }
+  __device__ static __forceinline__ void combine(acc_t& a, const part_t& b) { a.tr += b.x; a.ti += b.y; }
 };
 
 // ---- double-float helpers (round-to-nearest intrinsics: never contracted into FMA) ----------
@@ -143,9 +154,32 @@ __device__ __forceinline__ void dw_accumulate(float& hi, float& lo, float s, flo
   e = __fadd_rn(e, __fadd_rn(lo, c));
   fast_two_sum(t, e, hi, lo);
 }
-// s + c += a * b for double-float a = (ah, al), b = (bh, bl): the product of the high parts is
-// split exactly (p + e, e = fma(ah, bh, -p)); the cross terms ah bl + al bh enter the
-// compensation; p enters the running sum through TwoSum whose error also goes to c.
+// The same with the error of the low parts' sum kept too (the "accurate" double-word addition), for
+// the additions that are few: lanes' partial sums and the two terms of an output.
+__device__ __forceinline__ void dw_add(float& hi, float& lo, float s, float c) {
+  float t, e, u, v;
+  two_sum(hi, s, t, e);
+  two_sum(lo, c, u, v);
+  fast_two_sum(t, __fadd_rn(e, u), hi, lo);
+  fast_two_sum(hi, __fadd_rn(lo, v), hi, lo);
+}
+// s + c + d += a * b for double-float a = (ah, al), b = (bh, bl): the product of the high parts is
+// split exactly (p + e, e = fma(ah, bh, -p)), the cross terms ah bl + al bh enter e, and p enters the
+// running sum through TwoSum. The errors of the sum (c) and of the products (d) are added up apart:
+// one rounding per term less than in a common sum.
+__device__ __forceinline__ void dot2_step(float& s, float& c, float& d, float ah, float al, float bh, float bl) {
+  const float p = __fmul_rn(ah, bh);
+  float e = __fmaf_rn(ah, bh, -p);
+  e = __fmaf_rn(ah, bl, e);
+  e = __fmaf_rn(al, bh, e);
+  float t, err;
+  two_sum(s, p, t, err);
+  s = t;
+  c = __fadd_rn(c, err);
+  d = __fadd_rn(d, e);
+}
+
+// The same with the errors of the sum and of the products in one sum c: a register less.
 __device__ __forceinline__ void dot2_step(float& s, float& c, float ah, float al, float bh, float bl) {
   const float p = __fmul_rn(ah, bh);
   float e = __fmaf_rn(ah, bh, -p);
@@ -161,36 +195,39 @@ struct DF64P {
   using mat_t = float4;   // (re_hi, re_lo, im_hi, im_lo)
   using vec_t = double2;
   using gv_t = float4;
-  struct acc_t { float sr, cr, si, ci, hr, lr, hi, li; };
-  // terms between two folds of (s, c), whose error grows with the terms they hold; the adjoint cuts a
-  // column over 8 lanes and folds often, so that its error stays that of 32 short chains (FIO
-  // N = 2^16: 1.8e-14 against 3.6e-14 with 16 terms)
-  static constexpr int CHUNK = 16, ADJ_CHUNK = 2;
+  struct acc_t { float sr, cr, dr, si, ci, di, hr, lr, hi, li; };
+  static constexpr int CHUNK = 16;  // terms between two folds of the warp-per-node kernel
   __device__ static __forceinline__ mat_t ld(const mat_t* p) { return __ldcs(p); }
   __device__ static __forceinline__ gv_t cvt(vec_t v) {
     const float rh = (float)v.x, ih = (float)v.y;
     return make_float4(rh, (float)(v.x - (double)rh), ih, (float)(v.y - (double)ih));
   }
   __device__ static __forceinline__ void init(acc_t& a) {
-    a.sr = a.cr = a.si = a.ci = 0.f;
+    a.sr = a.cr = a.dr = a.si = a.ci = a.di = 0.f;
     a.hr = a.lr = a.hi = a.li = 0.f;
   }
   __device__ static __forceinline__ void mac(acc_t& a, const mat_t& m, const gv_t& g) {
+    dot2_step(a.sr, a.cr, a.dr, m.x, m.y, g.x, g.y);
+    dot2_step(a.sr, a.cr, a.dr, -m.z, -m.w, g.z, g.w);
+    dot2_step(a.si, a.ci, a.di, m.x, m.y, g.z, g.w);
+    dot2_step(a.si, a.ci, a.di, m.z, m.w, g.x, g.y);
+  }
+  __device__ static __forceinline__ void mac_narrow(acc_t& a, const mat_t& m, const gv_t& g) {  // d is not used
     dot2_step(a.sr, a.cr, m.x, m.y, g.x, g.y);
     dot2_step(a.sr, a.cr, -m.z, -m.w, g.z, g.w);
     dot2_step(a.si, a.ci, m.x, m.y, g.z, g.w);
     dot2_step(a.si, a.ci, m.z, m.w, g.x, g.y);
   }
   __device__ static __forceinline__ void macc(acc_t& a, const mat_t& m, const gv_t& g) {
-    dot2_step(a.sr, a.cr, m.x, m.y, g.x, g.y);
-    dot2_step(a.sr, a.cr, m.z, m.w, g.z, g.w);
-    dot2_step(a.si, a.ci, m.x, m.y, g.z, g.w);
-    dot2_step(a.si, a.ci, -m.z, -m.w, g.x, g.y);
+    dot2_step(a.sr, a.cr, a.dr, m.x, m.y, g.x, g.y);
+    dot2_step(a.sr, a.cr, a.dr, m.z, m.w, g.z, g.w);
+    dot2_step(a.si, a.ci, a.di, m.x, m.y, g.z, g.w);
+    dot2_step(a.si, a.ci, a.di, -m.z, -m.w, g.x, g.y);
   }
   __device__ static __forceinline__ void flush(acc_t& a) {
-    dw_accumulate(a.hr, a.lr, a.sr, a.cr);
-    dw_accumulate(a.hi, a.li, a.si, a.ci);
-    a.sr = a.cr = a.si = a.ci = 0.f;
+    dw_accumulate(a.hr, a.lr, a.sr, __fadd_rn(a.cr, a.dr));
+    dw_accumulate(a.hi, a.li, a.si, __fadd_rn(a.ci, a.di));
+    a.sr = a.cr = a.dr = a.si = a.ci = a.di = 0.f;
   }
   __device__ static __forceinline__ vec_t fin(const acc_t& a) {
     return make_double2((double)a.hr + (double)a.lr, (double)a.hi + (double)a.li);
@@ -214,8 +251,8 @@ struct DF64P {
     part_t r = keep;
     const float hr = __shfl_xor_sync(0xffffffffu, send.x, o), lr = __shfl_xor_sync(0xffffffffu, send.y, o);
     const float hi = __shfl_xor_sync(0xffffffffu, send.z, o), li = __shfl_xor_sync(0xffffffffu, send.w, o);
-    dw_accumulate(r.x, r.y, hr, lr);
-    dw_accumulate(r.z, r.w, hi, li);
+    dw_add(r.x, r.y, hr, lr);
+    dw_add(r.z, r.w, hi, li);
     return r;
   }
   __device__ static __forceinline__ vec_t fin_part(const part_t& p) {
@@ -254,12 +291,13 @@ struct DF64S32P : DF64P {
   __device__ static __forceinline__ vec_t zero() { return make_float2(0.f, 0.f); }
 };
 
-// Vectors between levels of the single-vector forward path. With DF set the double-float
-// policy keeps them in its own format, (re_hi, re_lo, im_hi, im_lo) floats (16 bytes, like
-// complex128), so that gathering a level's operands, adding its pass-through terms and writing its
-// outputs take no FP64 arithmetic (GB300 issues FP64 at a small fraction of the FP32 rate); only
-// level 0 converts the complex128 x and level L the complex128 y. Otherwise the boundary vectors
-// are the policy's vec_t.
+// Vectors between levels. With DF set the double-float policy keeps them in its own format, (re_hi,
+// re_lo, im_hi, im_lo) floats (16 bytes, like complex128), so that gathering a level's operands, adding
+// its pass-through terms and writing its outputs take no FP64 arithmetic (GB300 issues FP64 at a small
+// fraction of the FP32 rate); only the first level converts the complex128 x and the last the
+// complex128 y. A pair holds 48 bits of the 53, as much as the operands of the products; with
+// complex128 between levels the errors are within 4 % of these, and nine vectors at N = 40960 take 880
+// us against 763. Otherwise the boundary vectors are the policy's vec_t.
 template <class P, bool DF>
 struct Bnd {
   using b_t = typename P::vec_t;
@@ -288,8 +326,8 @@ struct Bnd<DF64P, true> {
   __device__ static __forceinline__ b_t of_acc(const DF64P::acc_t& a) { return DF64P::part(a); }
   __device__ static __forceinline__ b_t of_part(const float4& a) { return a; }
   __device__ static __forceinline__ b_t add(b_t a, b_t b) {
-    dw_accumulate(a.x, a.y, b.x, b.y);
-    dw_accumulate(a.z, a.w, b.z, b.w);
+    dw_add(a.x, a.y, b.x, b.y);
+    dw_add(a.z, a.w, b.z, b.w);
     return a;
   }
   __device__ static __forceinline__ b_t zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }

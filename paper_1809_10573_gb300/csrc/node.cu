@@ -89,11 +89,11 @@ static idbf_status fwd_level(Plan* p, int l, const void* mat, const IO<typename 
   idbf_status s = IDBF_EUNSUPPORTED;
   // wide blocks whose operands do not fit in shared memory fall through to narrower ones
   if constexpr (std::is_same<P, FP32P>::value) {
-    // eight right-hand sides per CTA and four CTAs per SM: with sixteen, and twice the registers and
-    // shared memory, half as many warps hide the same latencies (32 vectors, N = 2^16: 1808 against
-    // 1729 us; 9 vectors as 5 + 4: 977 against 847 us)
+    // eight right-hand sides per CTA and one row per thread, three CTAs of 256 threads per SM: the sums
+    // and their totals fit in the registers (two rows per thread spill 532 bytes at 192 x 4 threads; 32
+    // vectors, N = 2^16: 1764 us, 2030 with two rows and 128 x 4, 2190 with 192 x 3)
     const int w = even_block(io.R, 8);
-    if (w > 6) s = fwd_launch<P, 8, 2, 4, 192, 4>(p, l, mat, io, after, st);
+    if (w > 6) s = fwd_launch<P, 8, 1, 4, 256, 3>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 4) s = fwd_launch<P, 6, 1, 4, 256, 3>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 2) s = fwd_launch<P, 4, 1, 4, 256, 3>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 1) s = fwd_launch<P, 2, 1, 8, 384, 2>(p, l, mat, io, after, st);
@@ -126,10 +126,13 @@ template <class P>
 static idbf_status adj_level(Plan* p, int l, const void* mat, const IO<typename P::vec_t>& io, bool after, cudaStream_t st) {
   idbf_status s = IDBF_EUNSUPPORTED;
   if constexpr (std::is_same<P, FP32P>::value) {
+    // sixteen right-hand sides, one column per lane: with the totals two columns need more than the 128
+    // registers of two CTAs (32 vectors, N = 2^16: 2115 us; 1815 without totals, with errors 10 to 50 %
+    // larger). Eight: a column over eight lanes without totals is 10 % faster, with errors 5 to 20 % larger
     const int w = even_block(io.R, 16);
-    if (w > 8) s = adj_launch<P, 16, 2, 4, 2, 256, 2>(p, l, mat, io, after, st);
-    if (s == IDBF_EUNSUPPORTED && w > 4) s = adj_launch<P, 8, 2, 4, 2, 192, 4>(p, l, mat, io, after, st);
-    if (s == IDBF_EUNSUPPORTED && w > 2) s = adj_launch<P, 4, 4, 8, 1, 256, 3>(p, l, mat, io, after, st);
+    if (w > 8) s = adj_launch<P, 16, 1, 4, 2, 256, 2>(p, l, mat, io, after, st);
+    if (s == IDBF_EUNSUPPORTED && w > 4) s = adj_launch<P, 8, 1, 4, 2, 192, 4>(p, l, mat, io, after, st);
+    if (s == IDBF_EUNSUPPORTED && w > 2) s = adj_launch<P, 4, 2, 8, 2, 256, 3>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 1) s = adj_launch<P, 2, 4, 8, 2, 256, 3>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED) s = adj_launch<P, 1, 4, 16, 2, 256, 4>(p, l, mat, io, after, st);
   } else if constexpr (std::is_same<P, FP64P>::value) {
@@ -141,7 +144,9 @@ static idbf_status adj_level(Plan* p, int l, const void* mat, const IO<typename 
     if (s == IDBF_EUNSUPPORTED && w > 3) s = adj_launch<P, 4, 2, 8, 2, 256, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 2) s = adj_launch<P, 3, 2, 8, 2, 256, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 1) s = adj_launch<P, 2, 2, 8, 2, 256, 2>(p, l, mat, io, after, st);
-    if (s == IDBF_EUNSUPPORTED) s = adj_launch<P, 1, 2, 8, 4, 256, 3>(p, l, mat, io, after, st);
+    // one vector: four sums of single columns (two columns of two sums are 2 % faster, N = 2^12..2^16, with
+    // 2-8 % larger errors)
+    if (s == IDBF_EUNSUPPORTED) s = adj_launch<P, 1, 1, 8, 4, 256, 3>(p, l, mat, io, after, st);
   } else {
     const int w = even_block(io.R, 4);
     if (w > 3) s = adj_launch<P, 4, 1, 8, 2, 256, 2>(p, l, mat, io, after, st);

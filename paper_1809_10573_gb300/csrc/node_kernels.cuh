@@ -29,17 +29,35 @@ __host__ __device__ constexpr int op_pitch() {
   return (RB * sizeof(G)) % 64 == 0 && RB > 1 ? RB + (int)(16 / sizeof(G)) : RB;
 }
 
+// How the terms of a row (or column) are added up, so that the rounding error does not grow with its
+// length:
+//   FOLD  terms after which the running sums are folded into totals beside them: double-float, and
+//         complex64, where a fold is a small part of the arithmetic;
+//   K     independent sums that take the columns (rows) in turn and meet at the end: FP64, whose pipe
+//         is the bound and which folds would load further, and the complex64 adjoint of one or two
+//         vectors, whose lanes hold few rows.
+// Errors against the FP64 apply, FIO N = 2^16, with single chains and now: complex64 4 vectors 7.8e-7
+// and 3.8e-7, 32 vectors 7.7e-7 and 3.9e-7, their adjoint 4.3e-7 and 3.5e-7, 5.5e-7 and 3.6e-7; double-float 4
+// vectors 4.1e-14 (folds of 16 terms) and 2.9e-14, adjoint 1.85e-14 and 1.72e-14.
+template <class P, int RB, bool ADJ>
+struct Chains {
+  static constexpr bool DF = std::is_same<typename P::part_t, float4>::value;
+  static constexpr bool F64 = std::is_same<typename P::part_t, double2>::value;
+  static constexpr int K = F64 ? (ADJ && RB == 1 ? 4 : 2) : !DF && ADJ && RB <= 2 ? 2 : 1;
+  static constexpr int FOLD = DF ? (ADJ ? 2 : RB <= 2 ? 4 : 8) : K > 1 ? 0 : !ADJ && RB == 4 ? 8 : 4;
+};
+
 // The RB operands of one element and the sums they enter. In general operand rb is element rb of the
 // row and a sum is the policy's accumulator; complex64 with an even RB packs the right-hand sides in
 // pairs, a row holding (re, re, im, im) per pair and a sum being two f32x2: each complex
 // multiply-add of a pair is four packed FMAs, in the order of FP32P::mac on either lane, and the
 // pairs' real and imaginary parts come out of one 16-byte load as packed registers.
-template <class P, int RB, bool PACKED = std::is_same<P, FP32P>::value && RB % 2 == 0>
+template <class P, int RB, int K, bool TOT, bool PACKED = std::is_same<P, FP32P>::value && RB % 2 == 0>
 struct Sums {
   using G = typename P::gv_t;
   using M = typename P::mat_t;
   struct ops_t { G g[RB]; };
-  typename P::acc_t a[RB];
+  typename P::acc_t a[K][RB];
   __device__ static __forceinline__ void put(G* row, int rb, const G& v) { row[rb] = v; }
   __device__ static __forceinline__ G get(const G* row, int rb) { return row[rb]; }
   __device__ static __forceinline__ void load(ops_t& o, const G* row) {
@@ -48,33 +66,47 @@ struct Sums {
   }
   __device__ __forceinline__ void init() {
 #pragma unroll
-    for (int i = 0; i < RB; ++i) P::init(a[i]);
-  }
-  __device__ __forceinline__ void mac(const M& m, const ops_t& o) {
+    for (int k = 0; k < K; ++k)
 #pragma unroll
-    for (int i = 0; i < RB; ++i) P::mac(a[i], m, o.g[i]);
+      for (int i = 0; i < RB; ++i) P::init(a[k][i]);
   }
-  __device__ __forceinline__ void macc(const M& m, const ops_t& o) {  // conj(m)
+  __device__ __forceinline__ void mac(int u, const M& m, const ops_t& o) {  // into sum u mod K
 #pragma unroll
-    for (int i = 0; i < RB; ++i) P::macc(a[i], m, o.g[i]);
+    for (int i = 0; i < RB; ++i) {
+      // double-float, three vectors and more: the registers of a second error sum cost 10 %
+      if constexpr (std::is_same<typename P::part_t, float4>::value && RB > 2) P::mac_narrow(a[u % K][i], m, o.g[i]);
+      else P::mac(a[u % K][i], m, o.g[i]);
+    }
   }
-  __device__ __forceinline__ void flush() {
+  __device__ __forceinline__ void macc(int u, const M& m, const ops_t& o) {  // conj(m)
 #pragma unroll
-    for (int i = 0; i < RB; ++i) P::flush(a[i]);
+    for (int i = 0; i < RB; ++i) P::macc(a[u % K][i], m, o.g[i]);
+  }
+  __device__ __forceinline__ void fold() {
+    if constexpr (K == 1) {
+#pragma unroll
+      for (int i = 0; i < RB; ++i) P::flush(a[0][i]);
+    }
   }
   __device__ __forceinline__ void parts(typename P::part_t (&pr)[RB]) {
 #pragma unroll
     for (int i = 0; i < RB; ++i) {
-      P::flush(a[i]);
-      pr[i] = P::part(a[i]);
+#pragma unroll
+      for (int k = 0; k < K; ++k) P::flush(a[k][i]);
+#pragma unroll
+      for (int h = 1; h < K; h *= 2)
+#pragma unroll
+        for (int k = 0; k + h < K; k += 2 * h) P::combine(a[k][i], P::part(a[k + h][i]));
+      pr[i] = P::part(a[0][i]);
     }
   }
 };
-template <class P, int RB>
-struct Sums<P, RB, true> {
+template <class P, int RB, int K, bool TOT>
+struct Sums<P, RB, K, TOT, true> {
   using G = float2;
   struct ops_t { ulonglong2 g[RB / 2]; };
-  f32x2 re[RB / 2], im[RB / 2];
+  f32x2 re[K][RB / 2], im[K][RB / 2];
+  f32x2 tre[TOT ? RB / 2 : 1], tim[TOT ? RB / 2 : 1];  // totals
   __device__ static __forceinline__ void put(G* row, int rb, const G& v) {
     float* f = (float*)row + (rb >> 1) * 4 + (rb & 1);
     f[0] = v.x;
@@ -90,24 +122,41 @@ struct Sums<P, RB, true> {
   }
   __device__ __forceinline__ void init() {
 #pragma unroll
-    for (int i = 0; i < RB / 2; ++i) re[i] = im[i] = 0ull;
-  }
-  __device__ __forceinline__ void mac(const float2& m, const ops_t& o) {
-    const f32x2 mx = pk2(m.x, m.x), my = pk2(m.y, m.y), ny = pk2(-m.y, -m.y);
-#pragma unroll
     for (int i = 0; i < RB / 2; ++i) {
-      re[i] = fma2(mx, o.g[i].x, re[i]);
-      im[i] = fma2(mx, o.g[i].y, im[i]);
-      re[i] = fma2(ny, o.g[i].y, re[i]);
-      im[i] = fma2(my, o.g[i].x, im[i]);
+#pragma unroll
+      for (int k = 0; k < K; ++k) re[k][i] = im[k][i] = 0ull;
+      if (TOT) tre[TOT ? i : 0] = tim[TOT ? i : 0] = 0ull;
     }
   }
-  __device__ __forceinline__ void macc(const float2& m, const ops_t& o) { mac(make_float2(m.x, -m.y), o); }
-  __device__ __forceinline__ void flush() {}
-  __device__ __forceinline__ void parts(float2 (&pr)[RB]) {
+  __device__ __forceinline__ void mac(int u, const float2& m, const ops_t& o) {
+    const f32x2 mx = pk2(m.x, m.x), my = pk2(m.y, m.y), ny = pk2(-m.y, -m.y);
+    const int k = u % K;
 #pragma unroll
     for (int i = 0; i < RB / 2; ++i) {
-      const float2 r = upk2(re[i]), m = upk2(im[i]);
+      re[k][i] = fma2(mx, o.g[i].x, re[k][i]);
+      im[k][i] = fma2(mx, o.g[i].y, im[k][i]);
+      re[k][i] = fma2(ny, o.g[i].y, re[k][i]);
+      im[k][i] = fma2(my, o.g[i].x, im[k][i]);
+    }
+  }
+  __device__ __forceinline__ void macc(int u, const float2& m, const ops_t& o) { mac(u, make_float2(m.x, -m.y), o); }
+  __device__ __forceinline__ void fold() {
+    if constexpr (TOT) {
+#pragma unroll
+      for (int i = 0; i < RB / 2; ++i) {
+        tre[i] = add2(tre[i], re[0][i]);
+        tim[i] = add2(tim[i], im[0][i]);
+        re[0][i] = im[0][i] = 0ull;
+      }
+    }
+  }
+  __device__ __forceinline__ void parts(float2 (&pr)[RB]) {
+    static_assert(K == 1 || (K == 2 && !TOT), "one sum, or two that meet in one addition");
+    fold();
+#pragma unroll
+    for (int i = 0; i < RB / 2; ++i) {
+      const float2 r = upk2(TOT ? tre[TOT ? i : 0] : K == 1 ? re[0][i] : add2(re[0][i], re[K - 1][i]));
+      const float2 m = upk2(TOT ? tim[TOT ? i : 0] : K == 1 ? im[0][i] : add2(im[0][i], im[K - 1][i]));
       pr[2 * i] = make_float2(r.x, m.x);
       pr[2 * i + 1] = make_float2(r.y, m.y);
     }
@@ -176,7 +225,8 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
   using M = typename P::mat_t;
   using BP = BndOf<P>;
   using B = typename BP::b_t;
-  using SM = Sums<P, RB>;
+  using CH = Chains<P, RB, false>;
+  using SM = Sums<P, RB, CH::K, CH::FOLD != 0>;
   constexpr int PITCH = op_pitch<P, RB>();
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   const int nrb = min(RB, r1 - r0);  // right-hand sides r0 .. r1-1
@@ -264,8 +314,10 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
   }
   const int nt0 = (rn[0] + TR - 1) / TR, T = nt0 + (rn[1] + TR - 1) / TR;
   const int maxc = max(colsv[0], colsv[1]);
+  // (four columns per lane at least; eight: double-float, FIO N = 2^12, one vector 68 us against 63, 2^14 221
+  // against 218)
   int S = 1;
-  while (S < 8 && 2 * S * T <= nt && maxc >= 16 * S) S *= 2;
+  while (S < 8 && 2 * S * T <= nt && maxc >= 8 * S) S *= 2;
   int64_t obv[2] = {0, 0};
   if (!ulev) {
     obv[0] = d.out_off[out_seg_id(d, j, 0)];
@@ -331,31 +383,31 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
     SM acc[TR];
 #pragma unroll
     for (int i = 0; i < TR; ++i) acc[i].init();
-    auto mac = [&](int k, const M (&m)[TR]) {
+    auto mac = [&](int k, int u, const M (&m)[TR]) {
       typename SM::ops_t g;
       SM::load(g, opd + kc[k]);
 #pragma unroll
-      for (int i = 0; i < TR; ++i) acc[i].mac(m[i], g);
+      for (int i = 0; i < TR; ++i) acc[i].mac(u, m[i], g);
     };
     int k = s, since = 0;
     for (; k + (U - 1) * S < cols; k += U * S) {
       // an entry's register takes the entry U columns on as soon as it is consumed
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        mac(k + u * S, mv[u]);
+        mac(k + u * S, u, mv[u]);
         if (k + (U + u) * S < cols) load(U + u, mv[u]);
       }
       off += U * step;
       since += U;
-      if (since >= P::CHUNK) {
+      if (CH::FOLD > 0 && since >= CH::FOLD) {
 #pragma unroll
-        for (int i = 0; i < TR; ++i) acc[i].flush();
+        for (int i = 0; i < TR; ++i) acc[i].fold();
         since = 0;
       }
     }
 #pragma unroll
     for (int u = 0; u < U - 1; ++u)
-      if (k + u * S < cols) mac(k + u * S, mv[u]);
+      if (k + u * S < cols) mac(k + u * S, u, mv[u]);
 #pragma unroll
     for (int i = 0; i < TR; ++i) {
       typename P::part_t pr[RB];
@@ -430,7 +482,8 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
   using M = typename P::mat_t;
   using BP = BndOf<P>;
   using B = typename BP::b_t;
-  using SM = Sums<P, RB>;
+  using CH = Chains<P, RB, true>;
+  using SM = Sums<P, RB, CH::K, CH::FOLD != 0>;
   constexpr int PITCH = op_pitch<P, RB>();
   constexpr int CG = 32 / LR, CT = CG * TC;  // lane groups of a warp, columns of a warp's tile
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
@@ -563,7 +616,7 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
         typename SM::ops_t g;
         SM::load(g, opd + gc[r + u * LR]);
 #pragma unroll
-        for (int t = 0; t < TC; ++t) acc[t].macc(mv[t], g);
+        for (int t = 0; t < TC; ++t) acc[t].macc(u, mv[t], g);
       };
       M mv[U][TC];
 #pragma unroll
@@ -576,9 +629,9 @@ __device__ __forceinline__ void adj_body(const DevLevel& d, const typename P::ma
           if (r + (U + u) * LR < rows) load(U + u, mv[u]);
         }
         since += U;
-        if (since >= P::ADJ_CHUNK) {
+        if (CH::FOLD > 0 && since >= CH::FOLD) {
 #pragma unroll
-          for (int t = 0; t < TC; ++t) acc[t].flush();
+          for (int t = 0; t < TC; ++t) acc[t].fold();
           since = 0;
         }
       }
