@@ -12,14 +12,15 @@ from paper_1809_10573_gb300 import inputs
 from tests.cases import oracle_case
 
 pytestmark = pytest.mark.gpu
-MODES = {"fp32": (P.MODE_FP32, torch.complex64), "df64": (P.MODE_DF64, torch.complex128)}
+MODES = {"fp32": (P.MODE_FP32, torch.complex64), "df64": (P.MODE_DF64, torch.complex128),
+         "tf32x3": (P.MODE_TF32X3, torch.complex64), "tf32x3_s64": (P.MODE_TF32X3_S64, torch.complex64)}
 # kernel, N, leaf: (mode, right-hand sides, adjoint, error)
 BARS = [
     ("fio", 1 << 14, 64, [("fp32", 2, False, 4.14e-7), ("fp32", 4, False, 4.13e-7), ("fp32", 8, True, 4.03e-7),
                           ("df64", 1, True, 1.67e-14), ("df64", 4, True, 1.67e-14)]),
     ("fio", 1 << 12, 64, [("fp32", 2, True, 3.05e-7), ("fp32", 8, True, 3.26e-7), ("fp32", 32, True, 3.84e-7)]),
     ("dft", 40960, 40, [("fp32", 4, False, 3.37e-7), ("fp32", 8, False, 3.91e-7), ("fp32", 32, False, 4.91e-7),
-                        ("df64", 4, True, 1.50e-14)]),
+                        ("df64", 4, True, 1.50e-14), ("tf32x3", 32, False, 5.80e-7), ("tf32x3_s64", 32, False, 4.90e-7)]),
 ]
 
 
