@@ -337,12 +337,12 @@ idbf_status idbf_batch_autotune(idbf_batch b, const void* const* x, void* const*
                                 int32_t reps, void* stream, float* best_ms);
 
 /* idbf_batch_set_tiling - choose the tiling by hand: `tile` indexes the autotuner's list above.
- * 0, 1, 2, 4, 6, 7: the persistent launch with 1, 4, 8, 8, 32 and 16 right-hand sides per item (128
- * threads per CTA for 2 and 7, else 256); 3, 5: level launches, most CTAs resident (3, reported as 8
- * right-hand sides per item) or most threads and registers per CTA (5, reported as 16). 4-7 in FP32
- * and FP64 only, 6 in FP32 only. nodes_per_item in {1, 2, 4}. IDBF_EUNSUPPORTED if the tile does not
- * exist for the batch's precision or its shared memory exceeds 200 KB (the previous tiling is then
- * kept), IDBF_EINVAL for other values. Synchronous. */
+ * 0, 1, 2, 4, 6, 7, 9: the persistent launch with 1, 4, 8, 8, 32, 16 and 1 right-hand sides per item (128
+ * threads per CTA for 2, 7 and 9, else 256); 3, 5, 8: level launches, most CTAs resident (3, reported as
+ * 8 right-hand sides per item), most registers per CTA (5, reported as 16) or at most four right-hand
+ * sides per CTA (8, reported as 4). 4-7 in FP32 and FP64 only, 6 in FP32 only. nodes_per_item in
+ * {1, 2, 4}. IDBF_EUNSUPPORTED if the tile does not exist for the batch's precision or its shared memory
+ * exceeds 200 KB (the previous tiling is then kept), IDBF_EINVAL for other values. Synchronous. */
 idbf_status idbf_batch_set_tiling(idbf_batch b, int32_t tile, int32_t nodes_per_item);
 
 /* idbf_batch_set_split - operators with N >= min_separate_n leave the persistent launch: each

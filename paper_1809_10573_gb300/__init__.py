@@ -286,7 +286,8 @@ class Batch:
 
     # tile indices of idbf_batch_set_tiling: (right-hand sides per item, threads per CTA of the
     # persistent launch or 0 for level launches, 1 if in FP32 and FP64 only)
-    TILES = ((1, 256, 0), (4, 256, 0), (8, 128, 0), (8, 0, 0), (8, 256, 1), (16, 0, 1), (32, 256, 1), (16, 128, 1))
+    TILES = ((1, 256, 0), (4, 256, 0), (8, 128, 0), (8, 0, 0), (8, 256, 1), (16, 0, 1), (32, 256, 1), (16, 128, 1),
+             (4, 0, 0), (1, 128, 0))
 
     def set_tiling(self, tile: int, nodes_per_item: int = 1):
         _lib.check(_lib.lib().idbf_batch_set_tiling(self._h, int(tile), int(nodes_per_item)), "idbf_batch_set_tiling")

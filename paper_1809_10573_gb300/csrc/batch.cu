@@ -14,12 +14,10 @@
 // already been taken by CTAs that are running, and the wait ends: there is no cycle, whatever the
 // number of resident CTAs. (A CTA holds one item ahead of the one it computes; of all unfinished items
 // the earliest in the queue is always one being computed.) Every wait is bounded in time; on a
-// timeout the item is counted as done (its results are invalid), bit 0 of the status word is set,
-// and idbf_batch_sync_status reports IDBF_ETIMEOUT.
+// timeout the item runs all the same (its results are invalid) and is counted as done, bit 0 of the
+// status word is set, and idbf_batch_sync_status reports IDBF_ETIMEOUT.
 //
 // Each node is computed by node::fwd_body, the body of the per-level kernels (node_kernels.cuh).
-// 24 operators of N = 2^10 .. 2^14, 1-32 right-hand sides, FP32: level launches 2.60 ms, persistent
-// launch 3.31 ms, one apply after the other 4.08 ms.
 #include <cuda_runtime.h>
 #include <string.h>
 
@@ -66,32 +64,61 @@ constexpr size_t kSmemCap = 200 * 1024;  // per CTA
 // Tiles: right-hand sides per work item (rb; above the body's width in several passes), threads per
 // CTA of the persistent launch, or 0 for level launches, one chain of launches per width of the
 // batch's operators: with rb = 8 in the instances of the per-level kernels (most CTAs resident),
-// with rb = 16 in instances of more threads and registers per CTA, whose tall nodes finish
-// sooner (batches of few nodes: 16 operators of N = 2^9 .. 2^12 in FP32 342 against 427 us).
+// with rb = 16 in instances of more registers per CTA, whose tall nodes finish sooner, with rb = 4 in
+// narrow ones, of which a small batch has fewer chains. In FP32 ten operators of N = 2^10 .. 2^11 take 149
+// us with rb = 4, 156 with 16, 169 with 8, and 24 of N = 2^9 .. 2^14 1475, 1195 and 1132 us. FP64, bound by
+// its pipe, prefers persistent launches of one right-hand side per item (the same batches: 1030 and
+// 10310 us with 128 threads, 1114 and 12150 with 256, 1090 and 10860 as level launches).
 struct Tile {
   int rb, nt;
   bool wide;  // FP32 and FP64 only
 };
 constexpr Tile kTiles[] = {{1, 256, false}, {4, 256, false}, {8, 128, false}, {8, 0, false},
-                           {8, 256, true},  {16, 0, true},   {32, 256, true}, {16, 128, true}};
-constexpr int kNumTiles = 8;
+                           {8, 256, true},  {16, 0, true},   {32, 256, true}, {16, 128, true},
+                           {4, 0, false},   {1, 128, false}};
+constexpr int kNumTiles = 10;
 // One node at one width. Not inlined: the widths of a precision share the kernel's registers.
+// dep: the completion counter that the item waits for (nullptr: no wait).
+struct Dep {
+  const volatile int* done;
+  int need;
+  uint64_t limit_ns;
+  int* status;
+};
 template <class P, int RB, int TR, int U>
 __device__ __noinline__ void batch_node(const OpLevel& ol, const IO<typename P::vec_t>& io, int64_t j, int r, int r1,
-                                        unsigned char* smem) {
-  node::fwd_body<P, RB, TR, U, false>(ol.d, (const typename P::mat_t*)ol.mat, io, ol.max_in, ol.max_out, ol.max_rows,
-                                      ol.max_cols, ol.max_rows_pair, j, 0, 1, r, r1, smem);
+                                        unsigned char* smem, const Dep& dep) {
+  node::fwd_body<P, RB, TR, U, false>(
+      ol.d, (const typename P::mat_t*)ol.mat, io, ol.max_in, ol.max_out, ol.max_rows, ol.max_cols, ol.max_rows_pair, j, 0, 1,
+      r, r1, smem, [&] {
+        if (!dep.done) return;
+        if (threadIdx.x == 0) {
+          if (*dep.done < dep.need) {
+            const uint64_t t0 = gtimer();
+            while (*dep.done < dep.need) {
+              if (gtimer() - t0 > dep.limit_ns) {
+                atomicOr(dep.status, 1);
+                break;
+              }
+            }
+          }
+          __threadfence();  // acquire: the previous level's outputs are visible
+        }
+        __syncthreads();
+      });
 }
 
-template <class P>
-__global__ void __launch_bounds__(NTMAX, 2) k_batch(const OpDesc* __restrict__ ops, const OpLevel* __restrict__ lv,
-                                                    const Item* __restrict__ items, int nitems, const void* const* xs,
-                                                    void* const* ys, const int64_t* lds, int* head, int* done,
-                                                    const int* __restrict__ target, int* status, uint64_t limit_ns) {
+// W: the widest pass, 1 for items of one right-hand side (three CTAs of 256 threads per SM) or the
+// policy's.
+template <class P, int W>
+__global__ void __launch_bounds__(NTMAX, W == 1 ? 3 : 2)
+    k_batch(const OpDesc* __restrict__ ops, const OpLevel* __restrict__ lv, const Item* __restrict__ items, int nitems,
+            const void* const* xs, void* const* ys, const int64_t* lds, int* head, int* done,
+            const int* __restrict__ target, int* status, uint64_t limit_ns) {
   using V = typename P::vec_t;
   using M = typename P::mat_t;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int sidx, sfail;
+  __shared__ int sidx;
   __shared__ OpLevel ol;  // the item's level and vectors
   __shared__ IO<V> io;
   if (threadIdx.x == 0) sidx = atomicAdd(head, 1);
@@ -106,7 +133,7 @@ __global__ void __launch_bounds__(NTMAX, 2) k_batch(const OpDesc* __restrict__ o
     static_assert(sizeof(OpLevel) % 4 == 0, "copied in words");
     if (threadIdx.x >= 32 && threadIdx.x < 64)
       for (int q = threadIdx.x - 32; q < (int)(sizeof(OpLevel) / 4); q += 32) ((uint32_t*)&ol)[q] = ((const uint32_t*)(lv + li))[q];
-    if (threadIdx.x == 64) {
+    if (threadIdx.x == 32) {
       io.x = (const V*)xs[w.op];
       io.ldx = lds[w.op];
       io.y = (V*)ys[w.op];
@@ -125,34 +152,25 @@ __global__ void __launch_bounds__(NTMAX, 2) k_batch(const OpDesc* __restrict__ o
         const int64_t n = nl.d.moff[e] + (int64_t)nl.d.rows[e] * nl.d.cols[e] - a;
         if (nw.r0 == 0 && n * (int64_t)sizeof(M) < (1 << 22)) node::prefetch_l2((const M*)nl.mat + a, n * (int64_t)sizeof(M));
       }
-      sfail = 0;
-      if (w.level > 0) {
-        volatile int* dp = done + (li - 1);
-        const int need = target[li - 1];
-        if (*dp < need) {
-          const uint64_t t0 = gtimer();
-          while (*dp < need) {
-            if (gtimer() - t0 > limit_ns) {
-              sfail = 1;
-              atomicOr(status, 1);
-              break;
-            }
-          }
-        }
-        __threadfence();  // acquire: the previous level's outputs are visible
-      }
     }
     __syncthreads();
-    if (!sfail) {
+    {
+      // only the item's first node and pass wait, after their index lists and first factor columns
+      // are on their way
+      Dep dep = {w.level > 0 ? done + (li - 1) : nullptr, w.level > 0 ? target[li - 1] : 0, limit_ns, status};
       const int r1 = min(od.R, w.r0 + od.width);
       const int pw = pass_width<P>(r1 - w.r0);
       for (int n = 0; n < w.nodes; ++n)
         for (int r = w.r0; r < r1; r += pw) {
           if (n || r != w.r0) __syncthreads();
-          at_width<P>(pw, [&](auto rb, auto tr, auto u) {
-            batch_node<P, decltype(rb)::value, decltype(tr)::value, decltype(u)::value>(
-                ol, io, (int64_t)(w.node0 + n), r, min(r + pw, r1), smem);
-          });
+          if constexpr (W == 1)
+            batch_node<P, 1, 1, 4>(ol, io, (int64_t)(w.node0 + n), r, r + 1, smem, dep);
+          else
+            at_width<P>(pw, [&](auto rb, auto tr, auto u) {
+              batch_node<P, decltype(rb)::value, decltype(tr)::value, decltype(u)::value>(
+                  ol, io, (int64_t)(w.node0 + n), r, min(r + pw, r1), smem, dep);
+            });
+          dep.done = nullptr;
         }
     }
     __threadfence();  // release: this item's outputs before its completion count
@@ -195,8 +213,14 @@ __global__ void __launch_bounds__(NTL, MINB)
     if (n) __syncthreads();
     node::fwd_body<P, RB, TR, U, false>(ol.d, (const typename P::mat_t*)ol.mat, io, ol.max_in, ol.max_out, ol.max_rows,
                                         ol.max_cols, ol.max_rows_pair, (int64_t)(it.node0 + n), it.sl, it.nsl, it.r0,
-                                        min(it.r0 + RB, io.R), smem);
+                                        min(it.r0 + RB, io.R), smem, [] { node::wait_for_inputs(); });
   }
+}
+
+// right-hand sides that a level launch's instance holds in registers
+template <class P>
+constexpr int level_rb() {
+  return std::is_same<P, DF64P>::value ? 4 : 8;
 }
 
 // The instances of the level launches, as the per-level kernels of node.cu: calls f with
@@ -302,7 +326,7 @@ int persistent_threads(const idbf_batch_s* b) { return bat::kTiles[b->tile].nt ?
 // The launches of every width and level and their items, for the current tile.
 template <class P>
 idbf_status plan_levels(idbf_batch_s* b, std::vector<bat::LevelItem>& items) {
-  const int cap = std::min(b->rb, bat::pass_rb<P>());
+  const int cap = std::min(b->rb, bat::level_rb<P>());
   constexpr bool kFp64 = std::is_same<P, FP64P>::value;
   std::vector<int> widths;  // instance widths in use
   std::vector<int> cls(b->nops, 0);
@@ -318,9 +342,11 @@ idbf_status plan_levels(idbf_batch_s* b, std::vector<bat::LevelItem>& items) {
   }
   std::sort(widths.begin(), widths.end(), [](int x, int y) { return x > y; });
   // few nodes on a level over the whole batch: cut them as the single apply does. FP64 counts each
-  // operator's nodes alone: its chains share one slow pipe and end together only in small items (five
-  // operators of N = 1024..8192, 18 vectors in all: 483 us against 783; double-float, whose chains
-  // fill one another's gaps, 316 against 421, complex64 154 against 199 the other way round)
+  // operator's nodes alone, and cuts to one CTA per SM: its chains share one slow pipe and end together
+  // only in small items, but every slice repeats a node's preparation (24 operators of N = 2^9 .. 2^14: 10860
+  // us, with two CTAs 11210, four 11680; double-float and complex64, whose chains fill one another's
+  // gaps, lose by counts of their own: 421 us against 316 and 199 against 154 for five operators of
+  // N = 1024 .. 8192)
   std::vector<int64_t> nodes(maxL + 1, 0);
   for (int o = 0; o < b->nops; ++o)
     for (int l = 0; !b->sep[o] && l <= b->plans[o]->p.L; ++l)
@@ -332,7 +358,7 @@ idbf_status plan_levels(idbf_batch_s* b, std::vector<bat::LevelItem>& items) {
         const Plan& p = b->plans[o]->p;
         if (b->sep[o] || cls[o] != w || l > p.L) continue;
         const LevelInfo& li = p.lv[l];
-        const int nsl = node::slices(kFp64 ? (int64_t)p.m * ((b->R[o] + w - 1) / w) : nodes[l], node::fwd_span(li), 4);
+        const int nsl = node::slices(kFp64 ? (int64_t)p.m * ((b->R[o] + w - 1) / w) : nodes[l], node::fwd_span(li), kFp64 ? 1 : 4);
         bat::at_level_width<P>(w, b->rb > 8, [&](auto rb, auto tr, auto, auto ntl, auto) {
           q.smem = std::max(q.smem, node::fwd_smem<P, decltype(rb)::value>(li.max_in, li.max_out, li.max_rows, li.max_cols,
                                                                             li.max_rows_pair, li.kind == KIND_U));
@@ -399,17 +425,22 @@ idbf_status launch_levels(idbf_batch_s* b, cudaStream_t st) {
   return IDBF_OK;
 }
 
+// the instance of the persistent kernel for the current tile
+template <class P>
+auto* batch_kernel(const idbf_batch_s* b) {
+  return b->rb == 1 ? bat::k_batch<P, 1> : bat::k_batch<P, bat::pass_rb<P>()>;
+}
+
 template <class P>
 idbf_status launch_batch(idbf_batch_s* b, cudaStream_t st) {
-  if (b->smem > 48 * 1024)
-    IDBF_CUDA_TRY(allow_smem(bat::k_batch<P>, bat::kSmemCap));
+  const auto kern = batch_kernel<P>(b);
+  if (b->smem > 48 * 1024) IDBF_CUDA_TRY(allow_smem(kern, bat::kSmemCap));
   const void* const* xs = (const void* const*)b->d_ptrs;
   void* const* ys = (void* const*)(b->d_ptrs + b->nops);
   const int64_t* lds = (const int64_t*)(b->d_ptrs + 2 * b->nops);
   IDBF_CUDA_TRY(cudaMemsetAsync(b->d_counters, 0, sizeof(int) * (1 + b->nlevels_total), st));
-  bat::k_batch<P><<<b->ctas, persistent_threads(b), b->smem, st>>>(b->d_ops, b->d_lv, b->d_items, b->nitems, xs, ys, lds,
-                                                                    b->d_counters, b->d_counters + 1, b->d_target,
-                                                                    b->d_status, b->limit_ns);
+  kern<<<b->ctas, persistent_threads(b), b->smem, st>>>(b->d_ops, b->d_lv, b->d_items, b->nitems, xs, ys, lds, b->d_counters,
+                                                        b->d_counters + 1, b->d_target, b->d_status, b->limit_ns);
   IDBF_CUDA_TRY(cudaGetLastError());
   return IDBF_OK;
 }
@@ -428,9 +459,9 @@ size_t smem_for(idbf_batch_s* b) {
 template <class P>
 int occupancy(idbf_batch_s* b) {
   int n = 0;
-  if (b->smem > 48 * 1024)
-    allow_smem(bat::k_batch<P>, bat::kSmemCap);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bat::k_batch<P>, persistent_threads(b), b->smem);
+  const auto kern = batch_kernel<P>(b);
+  if (b->smem > 48 * 1024) allow_smem(kern, bat::kSmemCap);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, persistent_threads(b), b->smem);
   return std::max(n, 1);
 }
 

@@ -16,24 +16,24 @@ template <class P>
 __host__ __device__ constexpr int max_rb() {
   return std::is_same<P, FP32P>::value ? 32 : std::is_same<P, FP64P>::value ? 16 : 8;
 }
-// right-hand sides that one pass of the body holds in registers
+// Right-hand sides that one pass of the body holds: 2 in FP64 and 4 else (8 in FP64 and FP32 spill in the
+// kernel's 128 registers; 24 operators of N = 2^9 .. 2^14, 4 per item: FP64 11.3 against 12.2 ms, but 10.3 with
+// items of one; FP32 2710 against 2570 us).
 template <class P>
 __host__ __device__ constexpr int pass_rb() {
-  return std::is_same<P, DF64P>::value ? 4 : 8;
+  return std::is_same<P, FP64P>::value ? 2 : 4;
 }
 
 // The body's width for an item of at most w right-hand sides in one pass: calls f with it.
 template <class P, class F>
 __host__ __device__ __forceinline__ void at_width(int w, F f) {
   using std::integral_constant;
-  if constexpr (std::is_same<P, FP32P>::value) {
-    if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 1>(), integral_constant<int, 4>());
-  } else if constexpr (std::is_same<P, FP64P>::value) {
-    if (w > 4) return f(integral_constant<int, 8>(), integral_constant<int, 1>(), integral_constant<int, 2>());
-  } else {
-    if (w == 3) return f(integral_constant<int, 3>(), integral_constant<int, 1>(), integral_constant<int, 2>());
+  if constexpr (pass_rb<P>() > 2) {
+    if constexpr (std::is_same<P, DF64P>::value) {
+      if (w == 3) return f(integral_constant<int, 3>(), integral_constant<int, 1>(), integral_constant<int, 2>());
+    }
+    if (w > 2) return f(integral_constant<int, 4>(), integral_constant<int, 1>(), integral_constant<int, 2>());
   }
-  if (w > 2) return f(integral_constant<int, 4>(), integral_constant<int, 1>(), integral_constant<int, 2>());
   if (w > 1) return f(integral_constant<int, 2>(), integral_constant<int, 1>(), integral_constant<int, 4>());
   return f(integral_constant<int, 1>(), integral_constant<int, 1>(), integral_constant<int, 4>());
 }

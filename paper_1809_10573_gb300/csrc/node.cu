@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(NTMAX, MINB)
   const unsigned unit = blockIdx.x / (unsigned)nblk;
   fwd_body<P, RB, TR, U, STREAM>(d, mat, io, max_in, max_out, max_rows, max_cols, max_rows_pair,
                                  (int64_t)(unit / (unsigned)nsl), (int)(unit % (unsigned)nsl), nsl,
-                                 (int)(blockIdx.x % (unsigned)nblk) * RB, io.R, smem);
+                                 (int)(blockIdx.x % (unsigned)nblk) * RB, io.R, smem, [] { wait_for_inputs(); });
 }
 
 template <class P, int RB, int TC, int LR, int U, int NTMAX, int MINB, bool STREAM>

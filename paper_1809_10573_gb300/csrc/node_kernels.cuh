@@ -216,11 +216,13 @@ __host__ __device__ constexpr size_t fwd_smem(int max_in, int max_out, int max_r
   return (n + 15) & ~(size_t)15;
 }
 
-template <class P, int RB, int TR, int U, bool STREAM>
+// wait() returns, in every thread, once the inputs may be read; everything before it reads the node's
+// description and factors only.
+template <class P, int RB, int TR, int U, bool STREAM, class W>
 __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::mat_t* __restrict__ mat,
                                          const IO<typename P::vec_t>& io, int max_in, int max_out, int max_rows,
                                          int max_cols, int max_rows_pair, int64_t j, int sl, int nsl, int r0,
-                                         int r1, unsigned char* smem) {
+                                         int r1, unsigned char* smem, W wait) {
   using G = typename P::gv_t;
   using M = typename P::mat_t;
   using BP = BndOf<P>;
@@ -359,7 +361,7 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
   begin(tid);
 
   // ---- inputs -> operands
-  wait_for_inputs();
+  wait();
   if (d.lev == 0) {
     for (int i = tid; i < l0 * RB; i += nt) {
       const int rb = i / l0, e = i - rb * l0;
