@@ -239,9 +239,7 @@ void at_level_width(int w, bool few, F f) {
     if (w > 1) IDBF_W(2, 1, 8, 256, 3);
     IDBF_W(1, 1, 6, 256, 4);
   } else if constexpr (std::is_same<P, FP64P>::value) {
-    if (w > 7) IDBF_W(8, 1, 2, 256, 2);
-    if (w > 6) IDBF_W(7, 1, 2, 256, 2);
-    if (w > 5) IDBF_W(6, 1, 2, 256, 2);
+    if (w > 5) IDBF_W(7, 1, 2, 256, 2);
     if (w > 4) IDBF_W(5, 1, 4, 256, 2);
     if (w > 3) IDBF_W(4, 1, 4, 256, 2);
     if (w > 2) IDBF_W(3, 1, 4, 256, 2);

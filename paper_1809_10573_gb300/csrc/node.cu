@@ -99,11 +99,9 @@ static idbf_status fwd_level(Plan* p, int l, const void* mat, const IO<typename 
     if (s == IDBF_EUNSUPPORTED && w > 1) s = fwd_launch<P, 2, 1, 8, 384, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED) s = fwd_launch<P, 1, 1, 6, 384, 3>(p, l, mat, io, after, st);
   } else if constexpr (std::is_same<P, FP64P>::value || std::is_same<P, FP64S32P>::value) {
-    // bound by the FP64 pipe: every width, so that no lane multiplies for right-hand sides past R
+    // bound by the FP64 pipe: widths that leave few lanes multiplying for right-hand sides past R
     const int w = fitting_block(io.R);
-    if (w > 7) s = fwd_launch<P, 8, 1, 2, 256, 2>(p, l, mat, io, after, st);
-    if (s == IDBF_EUNSUPPORTED && w > 6) s = fwd_launch<P, 7, 1, 2, 256, 2>(p, l, mat, io, after, st);
-    if (s == IDBF_EUNSUPPORTED && w > 5) s = fwd_launch<P, 6, 1, 2, 256, 2>(p, l, mat, io, after, st);
+    if (w > 5) s = fwd_launch<P, 7, 1, 2, 256, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 4) s = fwd_launch<P, 5, 1, 4, 256, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 3) s = fwd_launch<P, 4, 1, 4, 256, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 2) s = fwd_launch<P, 3, 1, 4, 256, 2>(p, l, mat, io, after, st);
@@ -137,9 +135,7 @@ static idbf_status adj_level(Plan* p, int l, const void* mat, const IO<typename 
     if (s == IDBF_EUNSUPPORTED) s = adj_launch<P, 1, 4, 16, 2, 256, 4>(p, l, mat, io, after, st);
   } else if constexpr (std::is_same<P, FP64P>::value) {
     const int w = fitting_block(io.R);
-    if (w > 7) s = adj_launch<P, 8, 1, 8, 2, 256, 2>(p, l, mat, io, after, st);
-    if (s == IDBF_EUNSUPPORTED && w > 6) s = adj_launch<P, 7, 1, 8, 2, 256, 2>(p, l, mat, io, after, st);
-    if (s == IDBF_EUNSUPPORTED && w > 5) s = adj_launch<P, 6, 1, 8, 2, 256, 2>(p, l, mat, io, after, st);
+    if (w > 5) s = adj_launch<P, 7, 1, 8, 2, 256, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 4) s = adj_launch<P, 5, 1, 8, 2, 256, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 3) s = adj_launch<P, 4, 2, 8, 2, 256, 2>(p, l, mat, io, after, st);
     if (s == IDBF_EUNSUPPORTED && w > 2) s = adj_launch<P, 3, 2, 8, 2, 256, 2>(p, l, mat, io, after, st);

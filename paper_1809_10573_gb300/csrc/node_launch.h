@@ -43,14 +43,15 @@ inline int even_block(int64_t R, int cap) {
   return (int)((R + nblk - 1) / nblk);
 }
 
-// FP64's block width, 3 to 8 (or R): the FP64 pipe is the bound, so the fewest right-hand sides past R
-// are computed, and of those widths the narrowest, whose more numerous CTAs balance better over the
-// SMs (NUFFT N = 30011, 18 vectors: 2.88 ms with 6; the factors' re-reads come from L2).
+// FP64's block width, 3, 4, 5 or 7 (or R): the FP64 pipe is the bound, so the fewest right-hand sides
+// past R are computed, and of those widths the narrowest, whose more numerous CTAs balance better over
+// the SMs (NUFFT N = 30011, 18 vectors: 2.61 ms with 3, 2.88 with 6; the factors' re-reads come from L2).
+// Blocks of 6 and 8 fit nothing that blocks of 3 and 4 do not.
 inline int fitting_block(int64_t R) {
   if (R <= 3) return (int)R;
   int best = 3;
-  for (int w = 4; w <= 8 && w <= R; ++w)
-    if ((R + w - 1) / w * w < (R + best - 1) / best * best) best = w;
+  for (const int w : {4, 5, 7})
+    if (w <= R && (R + w - 1) / w * w < (R + best - 1) / best * best) best = w;
   return best;
 }
 

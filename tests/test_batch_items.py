@@ -1,5 +1,6 @@
-"""Shared memory of the persistent batch launch, on the host: every item an operator is cut into runs
-a body whose buffers fit in what the launch is sized by, for any number of right-hand sides."""
+"""Cutting right-hand sides into blocks, on the host. The persistent batch launch: every item an operator
+is cut into runs a body whose buffers fit in what the launch is sized by, for any number of right-hand
+sides. FP64 blocks: every width chosen has a kernel instance, and no other computes less."""
 import os
 import subprocess
 
@@ -44,7 +45,18 @@ int check(const char* name) {
     }
   return bad;
 }
-int main() { return check<FP32P>("fp32") + check<DF64P>("df64") + check<FP64P>("fp64") ? 1 : 0; }
+int widths() {  // FP64 blocks: of the widths that have an instance, and none of 3 to 8 computes less
+  int bad = 0;
+  for (int64_t R = 1; R <= 5000; ++R) {
+    const int w = node::fitting_block(R);
+    int64_t least = (R + w - 1) / w * w;
+    for (int v = 3; v <= 8; ++v) least = std::min(least, (R + v - 1) / v * v);
+    const bool instance = w == 1 || w == 2 || w == 3 || w == 4 || w == 5 || w == 7;
+    if ((!instance || (R + w - 1) / w * w != least) && !bad++) printf("R %d: width %d\n", (int)R, w);
+  }
+  return bad;
+}
+int main() { return check<FP32P>("fp32") + check<DF64P>("df64") + check<FP64P>("fp64") + widths() ? 1 : 0; }
 """
 
 
