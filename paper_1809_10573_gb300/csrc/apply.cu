@@ -772,7 +772,7 @@ idbf_status ensure_workspace(Plan* p, int64_t nrhs) {
 // pair variant on level l runs levels l and l + 1 in one launch. Each launch reads the buffer the
 // previous one wrote and writes the other one.
 template <class P>
-static idbf_status run_fwd1(Plan* p, const void* x, void* y, int64_t ld, cudaStream_t st, int fmt) {
+static idbf_status run_fwd1(Plan* p, const void* x, void* y, cudaStream_t st, int fmt) {
   using V = typename P::vec_t;
   V* wb[2] = {(V*)p->d_ws, (V*)((char*)p->d_ws + (size_t)p->max_seg_total * 16)};
   int cur = 1;  // buffer holding the last boundary written (boundary b in b % 2 without pairs)
@@ -782,7 +782,6 @@ static idbf_status run_fwd1(Plan* p, const void* x, void* y, int64_t ld, cudaStr
     const int last = pair ? l + 1 : l;  // level whose outputs this launch writes
     const V* win = l > 0 ? wb[cur] : nullptr;
     V* wout = last < p->L ? wb[cur ^ 1] : nullptr;
-    (void)ld;
     idbf_status s = IDBF_EUNSUPPORTED;
     if (is_pair_variant(v) && !pair) v = default_variant(p, l, fmt);  // a pair variant on level L: one level
     s = launch_fwd_variant<P>(p, l, v, x, y, win, wout, st, fmt, l > 0);
@@ -809,7 +808,7 @@ static idbf_status run_fwd1(Plan* p, const void* x, void* y, int64_t ld, cudaStr
 template <class P>
 static idbf_status run_levels(Plan* p, const void* x, void* y, int64_t R, int64_t ld, bool adjoint, cudaStream_t st,
                               int fmt) {
-  if (!adjoint && R == 1) return run_fwd1<P>(p, x, y, ld, st, fmt);
+  if (!adjoint && R == 1) return run_fwd1<P>(p, x, y, st, fmt);
   void* wb[2] = {p->d_ws, (char*)p->d_ws + (size_t)p->max_seg_total * R * 16};
   for (int step = 0; step <= p->L; ++step) {
     const int l = adjoint ? p->L - step : step;

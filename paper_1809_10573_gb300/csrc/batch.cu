@@ -548,7 +548,6 @@ idbf_status layout(idbf_batch_s* b) {
     }
   b->nitems = (int)items.size();
   if (b->debug_extra > 0 && b->nlevels_total > 0) target[0] += b->debug_extra;
-  if (!tile_valid(b->mode, b->tile)) return IDBF_EUNSUPPORTED;
   if (b->nitems == 0) {  // every operator runs through idbf_apply: no persistent launch
     b->smem = 0;
     b->ctas = 0;

@@ -54,7 +54,6 @@ struct LevelInfo {
   int max_out = 0;       // max summed output length of a node
   int max_rows_pair = 0; // max rows_0 + rows_1 of a node
   int max_cols_pair = 0; // max cols_0 + cols_1 of a node
-  int64_t sum_rows = 0, sum_cols = 0;  // over all blocks of the level
   int kmin = 0, kmax = 0;  // output segment lengths
 };
 

@@ -69,13 +69,6 @@ struct FP64P {
   }
   __device__ static __forceinline__ void flush(acc_t&) {}
   __device__ static __forceinline__ vec_t fin(const acc_t& a) { return make_double2(a.re, a.im); }
-  __device__ static __forceinline__ void warp_sum(acc_t& a) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
-      a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
-    }
-  }
   __device__ static __forceinline__ vec_t add(vec_t a, vec_t b) { return make_double2(a.x + b.x, a.y + b.y); }
   __device__ static __forceinline__ vec_t zero() { return make_double2(0.0, 0.0); }
   using part_t = double2;  // a flushed accumulator, for combining partial sums
@@ -117,13 +110,6 @@ struct FP32P {
     a.re = a.im = 0.f;
   }
   __device__ static __forceinline__ vec_t fin(const acc_t& a) { return make_float2(a.tr, a.ti); }
-  __device__ static __forceinline__ void warp_sum(acc_t& a) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
-      a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
-    }
-  }
   __device__ static __forceinline__ vec_t add(vec_t a, vec_t b) { return make_float2(a.x + b.x, a.y + b.y); }
   __device__ static __forceinline__ vec_t zero() { return make_float2(0.f, 0.f); }
   using part_t = float2;
@@ -232,16 +218,6 @@ struct DF64P {
   __device__ static __forceinline__ vec_t fin(const acc_t& a) {
     return make_double2((double)a.hr + (double)a.lr, (double)a.hi + (double)a.li);
   }
-  __device__ static __forceinline__ void warp_sum(acc_t& a) {
-    flush(a);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float hr = __shfl_xor_sync(0xffffffffu, a.hr, o), lr = __shfl_xor_sync(0xffffffffu, a.lr, o);
-      const float hi = __shfl_xor_sync(0xffffffffu, a.hi, o), li = __shfl_xor_sync(0xffffffffu, a.li, o);
-      dw_accumulate(a.hr, a.lr, hr, lr);
-      dw_accumulate(a.hi, a.li, hi, li);
-    }
-  }
   __device__ static __forceinline__ vec_t add(vec_t a, vec_t b) { return make_double2(a.x + b.x, a.y + b.y); }
   __device__ static __forceinline__ vec_t zero() { return make_double2(0.0, 0.0); }
   using part_t = float4;  // (re_hi, re_lo, im_hi, im_lo) of a flushed accumulator
@@ -342,14 +318,7 @@ template <> constexpr int fmt_of<FP64S32P>() { return IDBF_STORE_C128; }
 template <> constexpr int fmt_of<DF64S32P>() { return IDBF_STORE_DF64; }
 
 // ---------------------------------------------------------------------------------------------
-// addressing of a node's input and output segments
-struct Seg {
-  int64_t base;  // element offset of element 0, rhs 0
-  int64_t es;    // element stride
-  int64_t rs;    // rhs stride
-  int len;
-};
-
+// the vectors of a level
 template <class V>
 struct IO {
   const V* x;  // user input (forward: level 0; adjoint: level L)

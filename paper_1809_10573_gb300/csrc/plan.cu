@@ -117,8 +117,6 @@ idbf_status finalize_structure(Plan* p) {
       li.max_out = std::max(li.max_out, out);
       for (int c = 0; c < 2; ++c) {
         li.entries += (int64_t)p->h_rows[o + c] * p->h_cols[o + c];
-        li.sum_rows += p->h_rows[o + c];
-        li.sum_cols += p->h_cols[o + c];
         li.max_rows = std::max(li.max_rows, p->h_rows[o + c]);
         li.max_cols = std::max(li.max_cols, p->h_cols[o + c]);
         if (li.kind == KIND_V) li.idx_entries += p->h_rows[o + c] + p->h_cols[o + c];
