@@ -373,8 +373,9 @@ idbf_status idbf_batch_sync_status(idbf_batch b, void* stream);
  * kernel's dependency waits (default 2 s) and, with extra_target > 0, raise the completion count
  * that the first operator's level-1 items wait for above the number of level-0 items, so that
  * those waits run out (a failure made on the host: no device fault). Each such item is then
- * skipped and counted as done, and idbf_batch_sync_status reports IDBF_ETIMEOUT. (limit, 0)
- * restores normal operation. Re-captures the graph. Not for production use. */
+ * computed from whatever its inputs hold and counted as done, and idbf_batch_sync_status reports
+ * IDBF_ETIMEOUT. (limit, 0) restores normal operation. Re-captures the graph; IDBF_EUNSUPPORTED, with
+ * nothing changed, if the persistent launch that it needs does not fit. Not for production use. */
 idbf_status idbf_batch_debug_set_wait(idbf_batch b, uint64_t limit_ns, int32_t extra_target);
 
 /* idbf_batch_destroy - release the batch (synchronises the device first; NULL is a no-op). */

@@ -398,8 +398,10 @@ idbf_status launch_levels(idbf_batch_s* b, cudaStream_t st) {
           cudaStream_t s = nullptr;
           cudaEvent_t ev = nullptr;
           IDBF_CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+          const cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+          if (e != cudaSuccess) cudaStreamDestroy(s);
+          IDBF_CUDA_TRY(e);
           b->side.push_back(s);
-          IDBF_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
           b->ev_join.push_back(ev);
         }
         cs = b->side[chain - 1];
@@ -666,6 +668,8 @@ idbf_status idbf_batch_apply(idbf_batch b, const void* const* x, void* const* y,
     memcpy(&tab[2 * b->nops + o], &ld[o], sizeof(int64_t));
   }
   cudaStream_t st = (cudaStream_t)stream;
+  // after a layout that failed there is no graph; without one, every operator must be above the split
+  if (!b->exec && std::find(b->sep.begin(), b->sep.end(), (char)0) != b->sep.end()) return IDBF_ECUDA;
   if (b->exec) {
     // pageable source: the copy is staged before the call returns, so tab may go out of scope
     IDBF_CUDA_TRY(cudaMemcpyAsync(b->d_ptrs, tab.data(), sizeof(void*) * tab.size(), cudaMemcpyHostToDevice, st));
@@ -808,9 +812,18 @@ idbf_status idbf_batch_set_tiling(idbf_batch b, int32_t tile, int32_t nodes_per_
 
 idbf_status idbf_batch_debug_set_wait(idbf_batch b, uint64_t limit_ns, int32_t extra_target) {
   if (!b || limit_ns == 0 || extra_target < 0) return IDBF_EINVAL;
+  const uint64_t old_limit = b->limit_ns;
+  const int old_extra = b->debug_extra;
   b->limit_ns = limit_ns;
   b->debug_extra = extra_target;
-  return layout(b);  // the limit and the targets are captured in the graph
+  const idbf_status s = layout(b);  // the limit and the targets are captured in the graph
+  if (s == IDBF_EUNSUPPORTED) {     // the persistent launch does not fit where level launches do
+    b->limit_ns = old_limit;
+    b->debug_extra = old_extra;
+    const idbf_status r = layout(b);
+    return r == IDBF_OK ? s : r;
+  }
+  return s;
 }
 
 idbf_status idbf_batch_info(idbf_batch b, int32_t* rhs_per_item, int32_t* nodes_per_item, int32_t* items, int32_t* ctas) {

@@ -424,7 +424,11 @@ idbf_status idbf_import_factors(const idbf_host_factors* f, int32_t storage, voi
     p.idx_len += itot;
     std::vector<double> colmajor;
     std::vector<int32_t> idx, ord;
-    try { colmajor.resize(2 * (size_t)tot); idx.resize(itot); } catch (...) { s = IDBF_ENOMEM; break; }
+    try {
+      colmajor.resize(2 * (size_t)tot);
+      idx.resize(itot);
+      ord.reserve(std::max(p.lv[l].max_rows, p.lv[l].max_cols));
+    } catch (...) { s = IDBF_ENOMEM; break; }
     for (int64_t o = l * nbl; o < (l + 1) * nbl; ++o) {
       const int64_t r = p.h_rows[o], c = p.h_cols[o];
       const double* src = f->mat + 2 * f->blk_moff[o];

@@ -45,3 +45,45 @@ def test_last_items_of_another_width_at_every_tiling(mode, fmt, dt, tol, R):
             y = y.cpu().numpy()
             assert np.linalg.norm(y - ref) / np.linalg.norm(ref) < tol, (tile, b.info())
     b.close()
+
+
+def _wide_middle(N0, k, k2, seed):
+    """Host factors of a made-up operator (L = 2): leaves of N0 points, k skeletons per V block, k2 per U
+    block, so that the middle nodes read 2 k elements and write few."""
+    rng = np.random.default_rng(seed)
+    m, L = 4, 2
+    rows = np.array([[[k, k]] * m, [[k2, k2]] * m, [[N0 - k2] * 2] * m], dtype=np.int32)
+    cols = np.array([[[N0 - k, N0 - k]] * m, [[2 * k] * 2] * m, [[k2, k2]] * m], dtype=np.int32)
+    mat, idx, mo, io = [], [], np.zeros(rows.shape, np.int64), np.zeros(rows.shape, np.int64)
+    nm = ni = 0
+    for l in range(L + 1):
+        for j in range(m):
+            for c in range(2):
+                r, q = int(rows[l, j, c]), int(cols[l, j, c])
+                mat.append((rng.standard_normal(r * q) + 1j * rng.standard_normal(r * q)) / np.sqrt(q))
+                mo[l, j, c], nm = nm, nm + r * q
+                io[l, j, c] = ni
+                if l != 1:
+                    p = rng.permutation(N0)
+                    nq = k if l == 0 else k2
+                    idx.append(np.concatenate([np.sort(p[:nq]), np.sort(p[nq:])]))
+                    ni += N0
+    return dict(N=m * N0, n0=N0, L=L, seg_len=np.array([[k] * 2 * m, [k2] * 2 * m], np.int32), blk_rows=rows, blk_cols=cols,
+                blk_moff=mo, blk_ioff=io, mat=np.concatenate(mat), idx=np.concatenate(idx).astype(np.int32))
+
+
+def test_a_refused_fault_injection_leaves_the_batch_working():
+    """Nine double-float vectors through middle nodes of 2400 inputs fit the level launches (three vectors
+    per CTA), not the persistent launch that the fault injection needs (items of 5 and 4)."""
+    plan = P.Plan.import_factors(_wide_middle(1204, 1200, 8, 1), storage=P.STORE_DF64)
+    x = torch.from_numpy(inputs.complex_gaussian(plan.N, 9, seed=2)).cuda()
+    b = P.Batch([plan], [9], mode=P.MODE_DF64)
+    for _ in range(2):
+        with pytest.raises(P.IDBFError) as e:
+            b.debug_set_wait(20_000_000, 1)
+        assert e.value.status == _lib.EUNSUPPORTED
+        y = b.apply([x])[0].cpu().numpy()
+        b.sync_status()
+        ref = plan.apply(x, mode=P.MODE_DF64).cpu().numpy()
+        assert np.linalg.norm(y - ref) / np.linalg.norm(ref) < 1e-13
+    b.close()
