@@ -34,8 +34,9 @@ __host__ __device__ constexpr int op_pitch() {
 //   FOLD  terms after which the running sums are folded into totals beside them: double-float, and
 //         complex64, where a fold is a small part of the arithmetic;
 //   K     independent sums that take the columns (rows) in turn and meet at the end: FP64, whose pipe
-//         is the bound and which folds would load further, and the complex64 adjoint of one or two
-//         vectors, whose lanes hold few rows.
+//         is the bound and which folds would load further (one sum for one vector forward, whose rows
+//         are cut over the most lanes), and the complex64 adjoint of one or two vectors, whose lanes
+//         hold few rows.
 // Errors against the FP64 apply, FIO N = 2^16, with single chains and now: complex64 4 vectors 7.8e-7
 // and 3.8e-7, 32 vectors 7.7e-7 and 3.9e-7, their adjoint 4.3e-7 and 3.5e-7, 5.5e-7 and 3.6e-7; double-float 4
 // vectors 4.1e-14 (folds of 16 terms) and 2.9e-14, adjoint 1.85e-14 and 1.72e-14.
@@ -43,8 +44,8 @@ template <class P, int RB, bool ADJ>
 struct Chains {
   static constexpr bool DF = std::is_same<typename P::part_t, float4>::value;
   static constexpr bool F64 = std::is_same<typename P::part_t, double2>::value;
-  static constexpr int K = F64 ? (ADJ && RB == 1 ? 4 : 2) : !DF && ADJ && RB <= 2 ? 2 : 1;
-  static constexpr int FOLD = DF ? (ADJ ? 2 : RB <= 2 ? 4 : 8) : K > 1 ? 0 : !ADJ && RB == 4 ? 8 : 4;
+  static constexpr int K = F64 ? (RB > 1 ? 2 : ADJ ? 4 : 1) : !DF && ADJ && RB <= 2 ? 2 : 1;
+  static constexpr int FOLD = DF ? (ADJ ? 2 : RB <= 2 ? 4 : 8) : K > 1 || F64 ? 0 : !ADJ && RB == 4 ? 8 : 4;
 };
 
 // The RB operands of one element and the sums they enter. In general operand rb is element rb of the
@@ -316,10 +317,11 @@ __device__ __forceinline__ void fwd_body(const DevLevel& d, const typename P::ma
   }
   const int nt0 = (rn[0] + TR - 1) / TR, T = nt0 + (rn[1] + TR - 1) / TR;
   const int maxc = max(colsv[0], colsv[1]);
-  // (four columns per lane at least; eight: double-float, FIO N = 2^12, one vector 68 us against 63, 2^14 221
-  // against 218)
+  // Four columns per lane at least (eight: double-float, FIO N = 2^12, one vector 68 us against 63, 2^14 221
+  // against 218), in FP64 with one vector eight, whose lanes' sums load its pipe (NUFFT N = 11331: 136 us,
+  // 177 with four).
   int S = 1;
-  while (S < 8 && 2 * S * T <= nt && maxc >= 8 * S) S *= 2;
+  while (S < 8 && 2 * S * T <= nt && maxc >= (CH::F64 && RB == 1 ? 16 : 8) * S) S *= 2;
   int64_t obv[2] = {0, 0};
   if (!ulev) {
     obv[0] = d.out_off[out_seg_id(d, j, 0)];
