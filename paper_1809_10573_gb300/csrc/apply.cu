@@ -2,10 +2,10 @@
 //
 // One launch per butterfly level. A node reads two vector segments, applies its two dense
 // blocks and writes two segments (Secs. 2.3-2.4: the fractal 2 x 2 structure of every factor).
-// The arithmetic policies (FP64, double-float, FP32) are in level_kernels.cuh.
-// Forward levels: thread per output row, blocks column-major so that a warp's loads of one
-// column are consecutive; adjoint levels: warp per output column (a contiguous run of the
-// block) with a warp-shuffle reduction.
+// The arithmetic policies (FP64, double-float, FP32) are in level_kernels.cuh. Here: the streaming
+// kernel and the warp-per-node kernel of the one-vector forward apply (a thread per output row,
+// blocks column-major so that a warp's loads of one column are consecutive), the level loops and the
+// autotuner. Levels of several vectors and of the adjoint run the node kernels (node.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -960,7 +960,7 @@ static idbf_status autotune_fmt(Plan* p, int fmt, cudaStream_t st, int reps, flo
     return IDBF_OK;
   };
   const int nl = p->L + 1;
-  std::vector<float> one(nl, 1e30f), two(nl, 1e30f);
+  std::vector<float> one(nl, 1e30f), two(nl, 1e30f), all((size_t)nl * kFirstPairVariant, 1e30f);
   std::vector<int> one_v(nl, 0), two_v(nl, -1);
   for (int l = 0; l < nl && s == IDBF_OK; ++l) {
     for (int v = 0; v < kNumFwdVariants && s == IDBF_OK; ++v) {
@@ -971,8 +971,9 @@ static idbf_status autotune_fmt(Plan* p, int fmt, cudaStream_t st, int reps, flo
       if (r != IDBF_OK) { s = r; break; }
       if (is_pair_variant(v)) {
         if (ms < two[l]) { two[l] = ms; two_v[l] = v; }
-      } else if (ms < one[l]) {
-        one[l] = ms; one_v[l] = v;
+      } else {
+        all[(size_t)l * kFirstPairVariant + v] = ms;
+        if (ms < one[l]) { one[l] = ms; one_v[l] = v; }
       }
     }
   }
@@ -995,6 +996,38 @@ static idbf_status autotune_fmt(Plan* p, int fmt, cudaStream_t st, int reps, flo
     } else {
       p->tuned[fmt][l] = one_v[l];
       l += 1;
+    }
+  }
+  // A level that L2 holds was timed from L2, not from HBM as in an apply. Where it is at least 2 % of the
+  // whole, the variants within 15 % of its best are tried in whole applies, and one that is faster
+  // there by more than 1 % is taken (double-float, FIO N = 2^15: 353 us against 372 without).
+  auto time_apply = [&](float* ms_out) -> idbf_status {
+    idbf_status r = IDBF_OK;
+    for (int k = -1; k < reps && r == IDBF_OK; ++k) {
+      if (k == 0) cudaEventRecord(e0, st);
+      r = run_levels<P>(p, x, y, 1, p->N, false, st, fmt);
+    }
+    cudaEventRecord(e1, st);
+    if (cudaEventSynchronize(e1) != cudaSuccess) return IDBF_ECUDA;
+    cudaEventElapsedTime(ms_out, e0, e1);
+    return r;
+  };
+  constexpr int64_t kL2Bytes = 192 << 20;  // 129 MB, and some more that is in part hit
+  float whole = 0.f;
+  if (s == IDBF_OK) s = time_apply(&whole);
+  for (int l = 0; l < nl && s == IDBF_OK; ++l) {
+    const int v0 = p->tuned[fmt][l];
+    if (is_pair_variant(v0) || one[l] < 0.02f * whole ||
+        p->lv[l].entries * (int64_t)sizeof(typename P::mat_t) > kL2Bytes)
+      continue;
+    for (int v = 0; v < kFirstPairVariant && s == IDBF_OK; ++v) {
+      if (v == v0 || all[(size_t)l * kFirstPairVariant + v] > 1.15f * one[l]) continue;
+      const int keep = p->tuned[fmt][l];
+      float ms = 0.f;
+      p->tuned[fmt][l] = v;
+      s = time_apply(&ms);
+      if (s == IDBF_OK && ms < 0.99f * whole) whole = ms;
+      else p->tuned[fmt][l] = keep;
     }
   }
   cudaEventDestroy(e0);
