@@ -599,7 +599,7 @@ def sub_autograd(plan, P, torch, inputs, steps, warmup, world, lpk, R=32):
 def sub_mrhs(P, torch, inputs, log2n, steps, warmup, world, lpk, R=256):
     """Many right-hand sides: N = 2^18, eps = 1e-6, 256 RHS, complex FP32 factors. Timed: 3xTF32
     tensor cores on every level; the same with the middle factor S^h in double-float on the CUDA
-    cores; the register-tiled FP32 CUDA-core apply (the same accuracy class without tensor cores);
+    cores; the FP32 CUDA-core apply (node kernels: the same accuracy class without tensor cores);
     and the FP64 apply of the same 256 vectors. Errors against that FP64 apply."""
     N = 1 << log2n
     x, xi = inputs.uniform_grid(N)

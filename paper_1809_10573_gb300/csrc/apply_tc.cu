@@ -1,4 +1,5 @@
-// Multi-right-hand-side apply on the tensor cores (tcgen05, kind::tf32, split precision).
+// Multi-right-hand-side apply on the tensor cores, split precision: the tcgen05 kernel (kind::tf32) of
+// split modes 1 and 2, described here, and the warp-level kernel of the default split mode further down.
 //
 // With R right-hand sides every butterfly block product M_c G (M_c: rows x cols complex, G:
 // cols x R) becomes a dense GEMM (Eq. 1 applied to a block of vectors). The complex product is
@@ -464,12 +465,13 @@ __global__ void __launch_bounds__(NT + 32, 1)
 // by the CTA, splits both in registers and feeds them straight to the MMAs: the slower tensor path (302
 // TFLOP/s measured, against ~1000 for tcgen05 TF32) is kept busier than the fast one was.
 //
-// One CTA (NT threads) takes node j and RB = 8 NTL right-hand sides; a warp's task is 16 rows of a block times
-// the RB right-hand sides. Complex products are four real ones: Re += Mr Gr + (-Mi) Gi, Im += Mr Gi +
+// One CTA (NT threads) takes node j and RB = 8 NTL right-hand sides; a warp's task is 16 rows of a block
+// times the RB right-hand sides. Complex products are four real ones: Re += Mr Gr + (-Mi) Gi, Im += Mr Gi +
 // Mi Gr. The tensor core rounds every accumulation downwards a little, so the main products hi hi
 // of every k-step (two accumulations) are added to a total in round-to-nearest FP32 (chains of two
-// k-steps: errors 15-20 % larger, the same time from 32 right-hand sides on); the two correction products,
-// 2^-11 of the main ones, keep an accumulator of their own. Columns past the block's end multiply zero entries with a row of zeros.
+// k-steps: errors 15-20 % larger, the same time from 32 right-hand sides on); the two correction
+// products, 2^-11 of the main ones, keep an accumulator of their own. Columns past the block's end
+// multiply zero entries with a row of zeros.
 // U levels: block 0 writes its term of every output position, block 1 adds its own after a barrier
 // (two terms: the order of the addition cannot change the sum).
 namespace wmma3 {
@@ -725,7 +727,7 @@ static cudaError_t launch(Plan* p, int l, const IO<float2>& io, bool after, cuda
 // 32 right-hand sides and three warps per CTA where blocks are short (at most 64 rows: four 16-row
 // tiles), 16 and four warps where they are tall, whose operands would leave one CTA per SM else; 8
 // where the level has too few nodes to fill the GPU or the operands do not fit. 256 vectors: DFT N =
-// 40960 2.76 ms with the first, 3.20 with the second; FIO N = 2^16 11.5 and 9.07 ms. False if not even
+// 40960 2.76 ms with the first, 3.20 with the second; FIO N = 2^16 11.5 and 9.2 ms. False if not even
 // eight right-hand sides fit.
 static bool level(Plan* p, int l, const IO<float2>& io, bool after, cudaStream_t st, cudaError_t* e) {
   const LevelInfo& li = p->lv[l];

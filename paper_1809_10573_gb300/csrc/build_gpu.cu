@@ -502,9 +502,10 @@ __device__ __forceinline__ double block_sum_d(double v, double* rv) {
 //
 // Bound by latency (each step waits for its loads) and, before the columns were taken NC at a time,
 // by the FP64 pipe (47 % busy with one column's scalars on all 32 lanes). Two shapes, by the batch's
-// blocks: 512 threads, one CTA per SM, for blocks of more than 128 columns (FIO N = 2^15: build 265
-// ms against 280 with 256 threads), else 256 threads, three CTAs per SM (NUFFT N = 50000: 89 against
-// 117 ms). One column at a time: 453 and 150 ms.
+// blocks: 512 threads, one CTA per SM, for blocks of more than 128 columns (FIO N = 2^15: with 256
+// threads the build took 6 % longer), else 256 threads, three CTAs per SM (NUFFT N = 50000: with 512
+// threads 31 % longer). The builds take 243 and 84 ms; one column at a time, IDs in their given order:
+// 453 and 150 ms.
 template <int NT, int NC, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_qr_df(const IDDesc* __restrict__ D, double2* __restrict__ Araw,
                                               int32_t* __restrict__ pscr, int32_t* __restrict__ kout,

@@ -1,5 +1,6 @@
-// Arithmetic policies and the per-node forward body shared by the per-level kernels (apply.cu)
-// and the persistent batch kernel (batch.cu). Three policies:
+// What the level kernels share: the arithmetic policies, the format of the vectors between levels, the
+// launch overlap, and the warp-per-node forward body of one vector (the node kernels' bodies are in
+// node_kernels.cuh). Three policies:
 //   FP64P - complex128 factors and vectors, FP64 FMA;
 //   DF64P - factors stored as double-float pairs (hi, lo) of binary32, complex128 vectors;
 //           products formed exactly with FMA (Dekker's product), sums accumulated with Knuth's
@@ -7,7 +8,7 @@
 //           and dot product", SIAM J. Sci. Comput. 26, 2005) and folded into a normalised
 //           double-float total (Joldes, Muller and Popescu, "Tight and rigorous error bounds for
 //           basic building blocks of double-word arithmetic", ACM TOMS 44, 2017);
-//   FP32P - complex64 factors and vectors, FP32 FMA.
+//   FP32P - complex64 factors and vectors, FP32 FMA, running sums folded into totals.
 #pragma once
 
 #include <cuda_runtime.h>
