@@ -654,8 +654,8 @@ def sub_mrhs(P, torch, inputs, log2n, steps, warmup, world, lpk, R=256):
 def sub_batch(P, torch, inputs, cap_log2n, steps, warmup, world, lpk):
     """Uneven batch: 64 operators, N = 2^e with e uniform in [12, 18], the first half the FIO and
     the second half the jittered DFT kernel, 1-32 RHS each, eps = 1e-6. Timed in FP32 (the value)
-    and double-float, each three ways: all 64 in one persistent launch in a CUDA graph (tiles
-    autotuned); with the split autotuned too (operators from some N up run through their own
+    and double-float, each three ways: all 64 in one CUDA graph of level launches or a persistent one
+    (tiles autotuned); with the split autotuned too (operators from some N up run through their own
     per-level kernels after the launch; the value); and the same 64 applies made one plan at a
     time. Errors against the FP64 apply. FIO operators of equal N are the
     same matrix: the first is built, the others are device copies of it (idbf_clone), so that every
@@ -693,7 +693,7 @@ def sub_batch(P, torch, inputs, cap_log2n, steps, warmup, world, lpk):
         xm = [x.to(vdt) for x in xs]
         ym = [torch.empty_like(x) for x in xm]
         b = P.Batch(plans, [o["nrhs"] for o in ops], mode=mode)
-        # every operator in the one persistent launch (tiles autotuned)
+        # every operator in the one graph (tiles autotuned)
         # a double-float batch takes 1-2 s and repeats to 0.1 %: fewer trials and steps there
         reps = 1 if name == "df64" else 2
         st_, wu_ = (min(steps, 3), min(warmup, 3)) if name == "df64" else (steps, warmup)
@@ -725,8 +725,8 @@ def sub_batch(P, torch, inputs, cap_log2n, steps, warmup, world, lpk):
     peak, kind = peaks()
     fma_pk = lpk["fp32_tflops"] / 2
     r32 = res["fp32"]
-    return {"metric": "IDBF uneven-batch applies/s (64 operators, N 2^12..2^18, 1-32 RHS; one persistent launch in a "
-                      "CUDA graph for the operators below an autotuned size split, their own per-level launches above)",
+    return {"metric": "IDBF uneven-batch applies/s (64 operators, N 2^12..2^18, 1-32 RHS; one CUDA "
+                      "graph for the operators below an autotuned size split, their own per-level launches above)",
             "value": value, "unit": "batches/s (64 operator applies each)", "ms_per_step": tmax * 1e3, "steps": steps,
             "dtype": "f32",
             "workload": "64 ops, seed 4: FIO (ops 0-31) / jittered DFT (32-63), eps=1e-6, leaf 64, complex64 factors"

@@ -259,7 +259,8 @@ idbf_status idbf_apply_noalloc(idbf_plan plan, const void* x, void* y, int64_t n
  * level l + 1 that read their four output segments, which stay in shared memory, the radix-2
  * case of level fusion) `reps` times with CUDA events on `stream`, and keep the cheapest cover
  * of the levels by single levels and fused pairs in the plan (idbf_stats reports the variant of
- * every level; both levels of a fused pair report the pair's variant). Later idbf_apply calls
+ * every level; both levels of a fused pair report the pair's variant). Levels that fit in L2 and are
+ * at least 2 % of the whole decide between close variants in whole applies. Later idbf_apply calls
  * use the choices; results are identical up to the summation order of the double-float / FP32
  * partial sums. Synchronous; allocates two N-vector temporaries. *apply_ms (if not NULL)
  * receives the summed best times. FP64 runs variants 0 and 7 only.
@@ -324,7 +325,8 @@ idbf_status idbf_batch_create(const idbf_plan* plans, int32_t nops, const int64_
 /* idbf_batch_apply - y[o] = K_o x[o] for every operator o (device pointers, column-major N_o x
  * nrhs[o] blocks with leading dimension ld[o] >= N_o, element type of `mode`): one graph launch
  * on `stream` after a small copy of the pointer table, then idbf_apply for each operator above
- * the split (idbf_batch_set_split). */
+ * the split (idbf_batch_set_split). ECUDA, with nothing computed, if the last change of the tiling
+ * or split failed for want of memory or with a CUDA error. */
 idbf_status idbf_batch_apply(idbf_batch b, const void* const* x, void* const* y, const int64_t* ld,
                              void* stream);
 
